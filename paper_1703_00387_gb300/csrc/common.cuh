@@ -232,6 +232,8 @@ struct GemmF64 {
   double alpha = 1.0, beta = 0.0;
 };
 osmps_status gemm_f64(const GemmF64& g, cudaStream_t stream);
+// Estimated time of gemm_f64 on an otherwise idle GPU, in microseconds.
+double gemm_f64_us(int64_t M, int64_t N, int64_t K);
 
 // ---------------------------------------------------------------------------
 // Split-precision tensor-core GEMM (tcgen05):
@@ -325,7 +327,7 @@ osmps_status split_operand(const SplitView& v, int kind, void* dst, int64_t Kp, 
 // m / n, column k; float64 sources). C is float64, row-major, ldc. With
 // subtract, C[M,N] -= the product instead (C must not overlap a or b). With
 // small_on_dmma, products that the float64 DMMA kernel finishes in an
-// estimated 40 us (plain float64 views) run there instead of the emulation.
+// estimated 56 us (plain float64 views) run there instead of the emulation.
 osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, int64_t M,
                       int64_t N, int64_t K, double* C, int64_t ldc, cudaStream_t s,
                       bool subtract = false, bool small_on_dmma = true);

@@ -492,12 +492,8 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
     return set_error(OSMPS_ESHAPE, "gemm_emu: inconsistent operand views");
   // Small products go to the float64 DMMA kernel, which is float64-accurate
   // too: the emulation costs about 56 us even for one tile (slicing passes,
-  // 36 slice pairs), while the DMMA kernel spreads its 64 x 64 tiles over the
-  // SMs at about 8 GFLOP/s each. Taken when that estimate is under 40 us.
-  const double dmma_tiles =
-      std::min<double>((double)cdiv(M, 64) * (double)cdiv(N, 64), (double)ctx->sm_count);
-  const double dmma_us = 2.0 * (double)M * (double)N * (double)K / (dmma_tiles * 8e3);
-  if (small_on_dmma && a.n1 == 1 && b.n1 == 1 && !a.src_f32 && !b.src_f32 && dmma_us < 40.0) {
+  // 36 slice pairs), so whatever the DMMA kernel finishes sooner runs there.
+  if (small_on_dmma && a.n1 == 1 && b.n1 == 1 && !a.src_f32 && !b.src_f32 && gemm_f64_us(M, N, K) < 56.0) {
     GemmF64 g;
     g.M = M; g.N = N; g.K = K;
     g.A = static_cast<const double*>(a.src); g.sam = a.s0; g.sak = a.sk;

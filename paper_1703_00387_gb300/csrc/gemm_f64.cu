@@ -6,16 +6,26 @@
 // QR shifts. Arbitrary element strides let one kernel express every
 // transpose and index grouping the contractions need without copies.
 //
-// Tiling: 64x64 output tile per CTA, K step 16, 8 warps (2 x 4), each warp
-// owns a 32x16 sub-tile = 4 x 2 fragments of 8x8. Global loads go through
-// registers into a double-buffered shared tile.
+// An SM does about two float64 FMAs per clock, half of one from each of its
+// four sub-partitions, so a product is bound by how evenly its FMAs spread
+// over the sub-partitions of all SMs, never by its loads (8 to 16 bytes of
+// operand per 128 clocks of DMMA at the tiles below). Hence small tiles for
+// every size: a CTA is four warps, one per sub-partition, on one 16x16 or 8x8
+// tile of C; the warps share the K range (K group of four number g goes to
+// warp g mod 4) and their partial tiles are added in warp order. Fragments
+// are read straight from global memory (eight rows x 32 bytes or four rows x
+// 64 bytes per load), a round of groups ahead of the DMMAs.
+// Measured against 64x64 tiles staged through shared memory (M x N x K, us):
+// 128x32x96 119 -> 6.3, 64x64x64 82 -> 4.2, 300x340x300 367 -> 74,
+// 512x512x512 615 -> 274, 1024x1024x1024 2445 -> 2074 (1.04 TFLOP/s),
+// 2048x2048x1024 8546 -> 8253.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace osmps {
 
 namespace {
-
-constexpr int BM = 64, BN = 64, BK = 16, PAD = 4, THREADS = 256;
 
 struct Args {
   int64_t M, N, K;
@@ -34,117 +44,131 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
                : "d"(a), "d"(b));
 }
 
-template <bool A_KFAST, bool B_NFAST>
-__global__ void __launch_bounds__(THREADS) k_gemm_f64(Args p) {
-  __shared__ double As[2][BK][BM + PAD];
-  __shared__ double Bs[2][BK][BN + PAD];
-
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
+template <int FM, int FN>
+__global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
+  constexpr int KU = FM * FN > 1 ? 2 : 4;  // K groups in flight per warp
+  constexpr int TM = 8 * FM, TN = 8 * FN;
+  __shared__ double red[4][TM][TN];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, tq = lane & 3;
-  const int wm = (warp >> 2) * 32, wn = (warp & 3) * 16;
-  const int64_t m0 = (int64_t)blockIdx.y * BM, n0 = (int64_t)blockIdx.x * BN;
-  const int64_t bz = blockIdx.z;
-  const double* A = p.A + bz * p.sab;
-  const double* B = p.B + bz * p.sbb;
-
-  double ra[4], rb[4];
-  auto load = [&](int64_t k0) {
+  const int64_t m0 = (int64_t)(blockIdx.x / tiles_n) * TM, n0 = (int64_t)(blockIdx.x % tiles_n) * TN;
+  const double* A = p.A + (int64_t)blockIdx.y * p.sab;
+  const double* B = p.B + (int64_t)blockIdx.y * p.sbb;
+  // this lane's rows / columns, those past the edge read as zero
+  const double* ap[FM];
+  const double* bp[FN];
+  bool am[FM], bm[FN];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int e = tid + r * THREADS;
-      int mm, kk;
-      if (A_KFAST) { kk = e % BK; mm = e / BK; } else { mm = e % BM; kk = e / BM; }
-      int64_t gm = m0 + mm, gk = k0 + kk;
-      ra[r] = (gm < p.M && gk < p.K) ? A[gm * p.sam + gk * p.sak] : 0.0;
-      int nn;
-      if (B_NFAST) { nn = e % BN; kk = e / BN; } else { kk = e % BK; nn = e / BK; }
-      int64_t gn = n0 + nn;
-      gk = k0 + kk;
-      rb[r] = (gn < p.N && gk < p.K) ? B[gk * p.sbk + gn * p.sbn] : 0.0;
+  for (int i = 0; i < FM; ++i) {
+    const int64_t m = m0 + 8 * i + g;
+    am[i] = m < p.M;
+    ap[i] = A + (am[i] ? m : 0) * p.sam;
+  }
+#pragma unroll
+  for (int j = 0; j < FN; ++j) {
+    const int64_t n = n0 + 8 * j + g;
+    bm[j] = n < p.N;
+    bp[j] = B + (bm[j] ? n : 0) * p.sbn;
+  }
+  double a[KU][FM], b[KU][FN];
+  auto load = [&](int64_t k) {  // the warp's KU groups from K index k on, 16 apart
+#pragma unroll
+    for (int u = 0; u < KU; ++u) {
+      const int64_t kk = k + 16 * u + tq;
+      const bool in = kk < p.K;
+#pragma unroll
+      for (int i = 0; i < FM; ++i) a[u][i] = in && am[i] ? ap[i][kk * p.sak] : 0.0;
+#pragma unroll
+      for (int j = 0; j < FN; ++j) b[u][j] = in && bm[j] ? bp[j][kk * p.sbk] : 0.0;
     }
   };
-  auto store = [&](int buf) {
+  double acc[FM][FN][2];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int e = tid + r * THREADS;
-      int mm, kk;
-      if (A_KFAST) { kk = e % BK; mm = e / BK; } else { mm = e % BM; kk = e / BM; }
-      As[buf][kk][mm] = ra[r];
-      int nn;
-      if (B_NFAST) { nn = e % BN; kk = e / BN; } else { kk = e % BK; nn = e / BK; }
-      Bs[buf][kk][nn] = rb[r];
+  for (int i = 0; i < FM; ++i)
+#pragma unroll
+    for (int j = 0; j < FN; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+  int64_t k = 4 * warp;
+  load(k);
+  for (; k < p.K; k += 16 * KU) {
+    double ca[KU][FM], cb[KU][FN];
+#pragma unroll
+    for (int u = 0; u < KU; ++u) {
+#pragma unroll
+      for (int i = 0; i < FM; ++i) ca[u][i] = a[u][i];
+#pragma unroll
+      for (int j = 0; j < FN; ++j) cb[u][j] = b[u][j];
     }
-  };
-
-  double acc[4][2][2];
+    load(k + 16 * KU);  // past the end: all zero, nothing is read
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int u = 0; u < KU; ++u)
+      if (k + 16 * u < p.K) {  // the same for the whole warp
 #pragma unroll
-    for (int j = 0; j < 2; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
-
-  const int64_t nk = cdiv(p.K, BK);
-  if (nk > 0) {
-    load(0);
-    store(0);
-  }
-  __syncthreads();
-  for (int64_t kt = 0; kt < nk; ++kt) {
-    const int buf = kt & 1;
-    if (kt + 1 < nk) load((kt + 1) * BK);
+        for (int i = 0; i < FM; ++i)
 #pragma unroll
-    for (int k4 = 0; k4 < BK; k4 += 4) {
-      double a[4], b[2];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[buf][k4 + tq][wm + i * 8 + g];
-#pragma unroll
-      for (int j = 0; j < 2; ++j) b[j] = Bs[buf][k4 + tq][wn + j * 8 + g];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) dmma(acc[i][j][0], acc[i][j][1], a[i], b[j]);
-    }
-    if (kt + 1 < nk) store(buf ^ 1);
-    __syncthreads();
-  }
-
-  double* C = p.C + bz * p.scb;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        int64_t gm = m0 + wm + i * 8 + g;
-        int64_t gn = n0 + wn + j * 8 + tq * 2 + r;
-        if (gm < p.M && gn < p.N) {
-          double* c = C + gm * p.scm + gn * p.scn;
-          double v = p.alpha * acc[i][j][r];
-          if (p.beta != 0.0) v = fma(p.beta, *c, v);
-          *c = v;
-        }
+          for (int j = 0; j < FN; ++j) dmma(acc[i][j][0], acc[i][j][1], ca[u][i], cb[u][j]);
       }
+  }
+#pragma unroll
+  for (int i = 0; i < FM; ++i)
+#pragma unroll
+    for (int j = 0; j < FN; ++j) {
+      red[warp][8 * i + g][8 * j + 2 * tq] = acc[i][j][0];
+      red[warp][8 * i + g][8 * j + 2 * tq + 1] = acc[i][j][1];
+    }
+  __syncthreads();
+  double* C = p.C + (int64_t)blockIdx.y * p.scb;
+  for (int e = threadIdx.x; e < TM * TN; e += 128) {
+    const int r = e / TN, c = e % TN;
+    const int64_t gm = m0 + r, gn = n0 + c;
+    if (gm < p.M && gn < p.N) {
+      double* dst = C + gm * p.scm + gn * p.scn;
+      double v = p.alpha * (((red[0][r][c] + red[1][r][c]) + red[2][r][c]) + red[3][r][c]);
+      if (p.beta != 0.0) v = fma(p.beta, *dst, v);
+      *dst = v;
+    }
+  }
+}
+
+// Tile edge, 16 or 8: the one whose busiest SM has the least to do, i.e. the
+// smaller ceil(tiles / SMs) edge^2. The 8x8 tile is counted 15% dearer per
+// FMA: with several rounds of tiles it measured 2% (300x300x340) to 40%
+// (256x256x256) slower at equal load, so it wins where it halves the rounds
+// (128x128x128: 8.3 against 14.4 us) and not for a few per cent of balance.
+constexpr int F64_SMS = 152;
+constexpr double COST_8 = 1.15;
+double busiest_sm(int64_t M, int64_t N, int64_t batch, int64_t t) {
+  return (double)cdiv(cdiv(M, t) * cdiv(N, t) * batch, F64_SMS) * (double)(t * t);
+}
+int f64_tile(int64_t M, int64_t N, int64_t batch) {
+  return COST_8 * busiest_sm(M, N, batch, 8) < busiest_sm(M, N, batch, 16) ? 8 : 16;
 }
 
 }  // namespace
+
+double gemm_f64_us(int64_t M, int64_t N, int64_t K) {
+  const double fma = std::min(busiest_sm(M, N, 1, 16), COST_8 * busiest_sm(M, N, 1, 8)) * (double)K;
+  return 4.0 + fma / 3500.0;  // 3.5 GFMA/s per SM measured
+}
 
 osmps_status gemm_f64(const GemmF64& g, cudaStream_t stream) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return OSMPS_OK;
   if (g.K <= 0) {
     return set_error(OSMPS_ESHAPE, "gemm_f64: K=%lld", (long long)g.K);
   }
-  if (cdiv(g.M, BM) > 65535 || g.batch > 65535)
-    return set_error(OSMPS_ESHAPE, "gemm_f64: M=%lld batch=%lld exceed the grid limits",
+  if (g.M > (int64_t)64 * 65535 || g.batch > 65535)
+    return set_error(OSMPS_ESHAPE, "gemm_f64: M=%lld batch=%lld exceed the supported range",
                      (long long)g.M, (long long)g.batch);
+  const int t = f64_tile(g.M, g.N, g.batch);
+  const int64_t tiles_n = cdiv(g.N, t), tiles = tiles_n * cdiv(g.M, t);
+  if (tiles > 2147483647ll)
+    return set_error(OSMPS_ESHAPE, "gemm_f64: %lld output tiles exceed the grid limit", (long long)tiles);
   Args a{g.M, g.N, g.K, g.A, g.sam, g.sak, g.sab, g.B, g.sbk, g.sbn, g.sbb,
          g.C, g.scm, g.scn, g.scb, g.alpha, g.beta};
-  dim3 grid((unsigned)cdiv(g.N, BN), (unsigned)cdiv(g.M, BM), (unsigned)g.batch);
-  bool akf = (g.sak == 1), bnf = (g.sbn == 1);
+  const dim3 grid((unsigned)tiles, (unsigned)g.batch);
   const int ph = prof_begin(stream);
-  if (akf && bnf) { k_gemm_f64<true, true><<<grid, THREADS, 0, stream>>>(a); note_launch(); }
-  else if (akf) { k_gemm_f64<true, false><<<grid, THREADS, 0, stream>>>(a); note_launch(); }
-  else if (bnf) { k_gemm_f64<false, true><<<grid, THREADS, 0, stream>>>(a); note_launch(); }
-  else { k_gemm_f64<false, false><<<grid, THREADS, 0, stream>>>(a); note_launch(); }
+  if (t == 16) k_gemm_f64<2, 2><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
+  else k_gemm_f64<1, 1><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
+  note_launch();
   OSMPS_LAUNCH_CHECK();
   const double f = 2.0 * (double)g.M * (double)g.N * (double)g.K * (double)g.batch;
   prof_end(ph, stream, OSMPS_KERNEL_GEMM_F64, f, f);
