@@ -213,9 +213,10 @@ osmps_status osmps_heff_apply(osmps_ctx* ctx, const double* L, const double* W1,
  * context) it is stale, so do not call this entry point again in a process
  * that has reset the device.
  * Every call shares the one array and it keeps the previous call's
- * contents (nothing in it is read before the call writes it), so calls
- * that can overlap on the GPU (other streams or threads) race: serialise
- * them.                                                                      */
+ * contents (nothing in it is read before the call writes it), so calls on
+ * different streams or threads run one after another on the GPU, in the
+ * order of the calls. A call captured into a CUDA graph is outside that
+ * order: serialise the graph's replays with other calls.                     */
 osmps_status osmps_heff_apply_noalloc(const double* L, const double* W1, const double* W2,
                                       const double* R, const double* theta, double* y,
                                       int64_t chi_l, int64_t d1, int64_t d2, int64_t chi_r,

@@ -45,6 +45,46 @@ osmps_status scratch_address(void** out) {
   return OSMPS_OK;
 }
 
+// Calls share the scratch, so each waits on the GPU for the one before it: an
+// event recorded after every call and waited on by the next. Launches are made under the lock, so threads cannot
+// interleave theirs. A call that is being captured into a graph neither waits
+// nor records (a capture cannot depend on work outside it): its replays are
+// the caller's to order.
+struct ScratchTurn {
+  cudaEvent_t done = nullptr;
+  bool used = false;
+};
+ScratchTurn g_turn[MAX_DEVICES];
+std::mutex g_turn_mu;
+
+class ScratchUse {
+ public:
+  osmps_status begin(cudaStream_t s) {
+    int dev = 0;
+    OSMPS_CUDA(cudaGetDevice(&dev));
+    turn_ = &g_turn[dev];  // scratch_address has checked the range
+    s_ = s;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    OSMPS_CUDA(cudaStreamIsCapturing(s, &cap));
+    capturing_ = cap != cudaStreamCaptureStatusNone;
+    if (capturing_) return OSMPS_OK;
+    if (!turn_->done) OSMPS_CUDA(cudaEventCreateWithFlags(&turn_->done, cudaEventDisableTiming));
+    if (turn_->used) OSMPS_CUDA(cudaStreamWaitEvent(s, turn_->done, 0));
+    return OSMPS_OK;
+  }
+  ~ScratchUse() {  // also after a launch that failed: earlier ones may still run
+    if (!turn_ || capturing_ || !turn_->done) return;
+    if (cudaEventRecord(turn_->done, s_) != cudaSuccess) return;
+    turn_->used = true;
+  }
+
+ private:
+  std::lock_guard<std::mutex> lock_{g_turn_mu};
+  ScratchTurn* turn_ = nullptr;
+  cudaStream_t s_ = nullptr;
+  bool capturing_ = false;
+};
+
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Bytes of a float64 array with the given extents, 256-byte aligned, or
@@ -107,6 +147,8 @@ extern "C" osmps_status osmps_heff_apply_noalloc(const double* L, const double* 
   double* T2 = reinterpret_cast<double*>(p + b_mat1 + b_mat2 + b_t1);
   double* T3 = reinterpret_cast<double*>(p + b_mat1 + b_mat2 + b_t1 + b_t2);
   cudaStream_t s = (cudaStream_t)stream;
+  ScratchUse use;
+  OSMPS_TRY(use.begin(s));
 
   // Every scratch region below is fully written before it is read, so the
   // previous call's contents never leak into this one.
