@@ -353,9 +353,14 @@ osmps_status fiber_contract_f32(const Fiber& f, const double* Mat, const float* 
 osmps_status fiber_contract_f32_split(const Fiber& f, const double* Mat, const float* in,
                                       void* dst, int kind, int64_t Kcols, int64_t Kp,
                                       cudaStream_t stream);
-// Both W-steps of H_eff.theta fused (T1 -> split T3) for the d = 2 MPO
-// shapes it is specialised for; *done = false means the caller must fall back
-// to the two fiber contractions.
+// Both W-steps of H_eff.theta fused, T1 -> T3 in float64; *done = false means
+// the caller must run the two fiber contractions.
+osmps_status wsteps_f64(const double* T1, const double* Mat1, const double* Mat2, double* T3,
+                        int64_t chi_l, int64_t d1, int64_t d2, int64_t chi_r, int64_t wl,
+                        int64_t wm, int64_t wr, cudaStream_t s, bool* done);
+// The same from float32 into the split operand, with kernels specialised for
+// the d = 2 MPO shapes of the spin chains; *done = false means the caller must
+// run the two fiber contractions.
 // Identity environment channels: with skip_l >= 0, T1 holds the wl - 1 other
 // channels and channel skip_l is theta (L[:, skip_l, :] = 1); with
 // skip_r >= 0, the split operand holds the wr - 1 other output channels and

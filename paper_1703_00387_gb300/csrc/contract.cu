@@ -118,11 +118,21 @@ static osmps_status heff_apply_prepared(osmps_ctx* ctx, const double* theta, dou
   f3.is1 = wm * d2 * chi_r; f3.is2 = 0; f3.istride = chi_r;
   f3.os1 = d2 * wr * chi_r; f3.os2 = 0; f3.ostride = chi_r;
 
+  // float64 stages 2 and 3: one pass, or two through T2 where that has no form
+  const auto wsteps = [&](const double* T1, double* T3) -> osmps_status {
+    bool done = false;
+    OSMPS_TRY(wsteps_f64(T1, mat1, mat2, T3, chi_l, d1, d2, chi_r, wl, wm, wr, stream, &done));
+    if (done) return OSMPS_OK;
+    osmps_status ws = OSMPS_OK;
+    double* T2 = (double*)ws_get(ctx, SLOT_HEFF_T2, (size_t)(chi_l * d1 * wm) * d2 * chi_r * 8, stream, &ws);
+    if (!T2) return ws;
+    OSMPS_TRY(fiber_contract_f64(f2, mat1, T1, T2, stream));
+    return fiber_contract_f64(f3, mat2, T2, T3, stream);
+  };
+
   if (precision == OSMPS_PREC_FP64_EMU) {
     double* T1 = (double*)ws_get(ctx, SLOT_HEFF_T1, (size_t)(chi_l * wl) * N1 * 8, stream, &st);
     if (!T1) return st;
-    double* T2 = (double*)ws_get(ctx, SLOT_HEFF_T2, (size_t)(chi_l * d1 * wm) * d2 * chi_r * 8, stream, &st);
-    if (!T2) return st;
     double* T3 = (double*)ws_get(ctx, SLOT_HEFF_T3, (size_t)(chi_l * d1 * d2) * wr * chi_r * 8, stream, &st);
     if (!T3) return st;
     SplitView la;  // L as (a2 w) x a
@@ -130,8 +140,7 @@ static osmps_status heff_apply_prepared(osmps_ctx* ctx, const double* theta, dou
     SplitView tt;  // theta^T: row n = (s1 s2 c), column a
     tt.src = theta; tt.rows = N1; tt.K = chi_l; tt.s0 = 1; tt.sk = N1;
     OSMPS_TRY(gemm_emu(ctx, la, tt, chi_l * wl, N1, chi_l, T1, N1, stream));
-    OSMPS_TRY(fiber_contract_f64(f2, mat1, T1, T2, stream));
-    OSMPS_TRY(fiber_contract_f64(f3, mat2, T2, T3, stream));
+    OSMPS_TRY(wsteps(T1, T3));
     const int64_t M4 = chi_l * d1 * d2, K4 = wr * chi_r;
     SplitView t3; t3.src = T3; t3.rows = M4; t3.K = K4; t3.s0 = K4; t3.sk = 1;
     SplitView rr; rr.src = ctx->slots[SLOT_HEFF_ROP].ptr; rr.rows = chi_r; rr.K = K4; rr.s0 = K4; rr.sk = 1;
@@ -141,8 +150,6 @@ static osmps_status heff_apply_prepared(osmps_ctx* ctx, const double* theta, dou
   if (precision == OSMPS_PREC_FP64) {
     double* T1 = (double*)ws_get(ctx, SLOT_HEFF_T1, (size_t)(chi_l * wl) * N1 * 8, stream, &st);
     if (!T1) return st;
-    double* T2 = (double*)ws_get(ctx, SLOT_HEFF_T2, (size_t)(chi_l * d1 * wm) * d2 * chi_r * 8, stream, &st);
-    if (!T2) return st;
     double* T3 = (double*)ws_get(ctx, SLOT_HEFF_T3, (size_t)(chi_l * d1 * d2) * wr * chi_r * 8, stream, &st);
     if (!T3) return st;
     GemmF64 g1;
@@ -152,8 +159,7 @@ static osmps_status heff_apply_prepared(osmps_ctx* ctx, const double* theta, dou
     g1.B = theta; g1.sbk = N1; g1.sbn = 1;
     g1.C = T1; g1.scm = N1; g1.scn = 1;
     OSMPS_TRY(gemm_f64(g1, stream));
-    OSMPS_TRY(fiber_contract_f64(f2, mat1, T1, T2, stream));
-    OSMPS_TRY(fiber_contract_f64(f3, mat2, T2, T3, stream));
+    OSMPS_TRY(wsteps(T1, T3));
     GemmF64 g4;
     g4.M = chi_l * d1 * d2; g4.N = chi_r; g4.K = wr * chi_r;
     g4.A = T3; g4.sam = wr * chi_r; g4.sak = 1;

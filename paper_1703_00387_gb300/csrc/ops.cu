@@ -7,7 +7,9 @@
 // * fiber contractions: the W-steps of Sec. 3.4, where the MPO tensors
 //   M^[k] (few entries, Eq. MPOdef) act on the small (w, s) index pair of an
 //   intermediate, for every (outer, inner) fiber. These are bandwidth-bound:
-//   one coalesced pass over the input and the output.
+//   one coalesced pass over the input and the output, summing only over the
+//   nonzero MPO entries (an Inf or NaN input reaches the outputs it is
+//   connected to).
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -126,78 +128,412 @@ int grid_for(int64_t n, int threads) {
   return (int)b;
 }
 
-template <typename T, int QMAX, int MODE>  // MODE 0: plain output, 1/2: split bf16/tf32
-__global__ void k_fiber(Fiber f, const double* __restrict__ Mat, const T* __restrict__ in,
-                        T* __restrict__ out, void* __restrict__ sdst, int64_t Kcols, int64_t Kp) {
-  extern __shared__ uint8_t fsm[];
-  T* Ms = reinterpret_cast<T*>(fsm);
-  const int P = (int)f.P, Q = (int)f.Q;
-  for (int i = threadIdx.x; i < P * Q; i += blockDim.x) Ms[i] = (T)Mat[i];
-  __syncthreads();
-  const int64_t total = f.n_o1 * f.n_o2 * f.nc;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = e % f.nc;
-    const int64_t o12 = e / f.nc;
-    const int64_t o2 = o12 % f.n_o2, o1 = o12 / f.n_o2;
-    const T* src = in + o1 * f.is1 + o2 * f.is2 + c;
-    T acc[QMAX];
-#pragma unroll
-    for (int o = 0; o < QMAX; ++o) acc[o] = (T)0;
-    for (int i = 0; i < P; ++i) {
-      const T x = src[(int64_t)i * f.istride];
-      const T* mrow = Ms + i * Q;
-#pragma unroll
-      for (int o = 0; o < QMAX; ++o)
-        if (o < Q) acc[o] = fma(mrow[o], x, acc[o]);
+// n / d for 0 <= n < 2^31 by a multiplication and a shift (Granlund and
+// Montgomery, PLDI 1994): a 64-bit division costs more than a whole fiber.
+struct FastDiv {
+  uint32_t d = 1, m = 0, s = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t div) : d(div) {
+    while (s < 32 && (1ull << s) < div) ++s;
+    m = (uint32_t)((((1ull << s) - div) << 32) / div + 1);
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t n) const {
+    return (uint32_t)(((uint64_t)__umulhi(m, n) + n) >> s);
+  }
+};
+
+// One nonzero entry of a W-step matrix: value, input index, and whether the
+// value is 1 (a comparison of float64 values runs on the float64 pipe).
+template <typename T>
+struct WTerm {
+  T v;
+  short i, one;
+};
+
+// The nonzero entries of a P x Q W-step matrix by output: output o's terms
+// are terms[ptr[o] .. ptr[o + 1]), inputs ascending. MPO tensors are an
+// identity in two corners and a few local operators (12 of 100 entries for
+// XXZ, 4% for AKLT), so the table holds WT_CAP entries; a matrix with more of
+// them is read entry by entry instead (dense).
+constexpr int WT_CAP = 640;
+constexpr int WT_QMAX = 64;
+template <typename T>
+struct WTable {
+  WTerm<T> terms[WT_CAP];
+  int ptr[WT_QMAX + 1];
+  const double* Mat;
+  int P, Q;
+  bool dense;
+};
+
+// Every thread of the block calls it (whole warps): a warp per output, lanes
+// over the inputs, the nonzero ones compacted by ballots.
+template <typename T>
+__device__ __forceinline__ void gather_terms(const double* __restrict__ Mat, int P, int Q,
+                                             WTable<T>& w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  for (int o = warp; o < Q; o += warps) {
+    int n = 0;
+    for (int i0 = 0; i0 < P; i0 += 32) {
+      const double m = i0 + lane < P ? Mat[(i0 + lane) * Q + o] : 0.0;
+      n += __popc(__ballot_sync(0xffffffffu, m != 0.0));
     }
-    const int64_t ob = o1 * f.os1 + o2 * f.os2 + c;
-#pragma unroll
-    for (int o = 0; o < QMAX; ++o) {
-      if (o < Q) {
-        const int64_t off = ob + (int64_t)o * f.ostride;
-        if (MODE == 0) {
-          out[off] = acc[o];
-        } else {
-          const int64_t row = off / Kcols, col = off - row * Kcols;
-          split_store_f32<MODE == 1 ? TC_BF16 : TC_TF32>(sdst, row * 2 * Kp + col, Kp, (float)acc[o]);
-        }
+    if (lane == 0) w.ptr[o + 1] = n;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    w.ptr[0] = 0;
+    for (int q = 0; q < Q; ++q) w.ptr[q + 1] += w.ptr[q];
+    w.Mat = Mat;
+    w.P = P;
+    w.Q = Q;
+    w.dense = w.ptr[Q] > WT_CAP || P > 32767;
+  }
+  __syncthreads();
+  if (!w.dense)
+    for (int o = warp; o < Q; o += warps) {
+      int n = w.ptr[o];
+      for (int i0 = 0; i0 < P; i0 += 32) {
+        const double m = i0 + lane < P ? Mat[(i0 + lane) * Q + o] : 0.0;
+        const unsigned nz = __ballot_sync(0xffffffffu, m != 0.0);
+        if (m != 0.0) w.terms[n + __popc(nz & ((1u << lane) - 1u))] = WTerm<T>{(T)m, (short)(i0 + lane), (short)(m == 1.0)};
+        n += __popc(nz);
       }
     }
+  __syncthreads();
+}
+
+// V fibers of one thread.
+template <typename T, int V>
+struct alignas(sizeof(T) * V) Pack {
+  T a[V];
+};
+
+// Output o of a W-step: sum over its nonzero entries of v x_i, inputs in
+// ascending order; x_i is at xs[i stride]. A first entry of 1 is taken over
+// as it is in float64, whose pipe is the narrow one.
+template <typename T, int V>
+__device__ __forceinline__ Pack<T, V> sum_terms(const WTable<T>& w, int o,
+                                                const Pack<T, V>* __restrict__ xs, int64_t stride) {
+  Pack<T, V> acc;
+#pragma unroll
+  for (int v = 0; v < V; ++v) acc.a[v] = (T)0;
+  const auto add = [&](T m, const Pack<T, V>& x) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc.a[v] = fma(m, x.a[v], acc.a[v]);
+  };
+  if (w.dense) {
+    for (int i = 0; i < w.P; ++i) {
+      const T m = (T)w.Mat[i * w.Q + o];
+      if (m != (T)0) add(m, xs[i * stride]);
+    }
+    return acc;
   }
+  int t = w.ptr[o];
+  const int t1 = w.ptr[o + 1];
+  if (sizeof(T) == 8 && t < t1 && w.terms[t].one) acc = xs[w.terms[t++].i * stride];
+#pragma unroll 2
+  for (; t < t1; ++t) {
+    const WTerm<T> e = w.terms[t];
+    add(e.v, xs[e.i * stride]);
+  }
+  return acc;
+}
+
+// V consecutive values of a split-operand row (off_hi a multiple of V).
+template <int KIND, int V>
+__device__ __forceinline__ void split_store_pack(void* dst, int64_t off_hi, int64_t Kp,
+                                                 const float (&x)[V]) {
+  if (KIND == TC_BF16) {
+    Pack<__nv_bfloat16, V> h, l;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      h.a[v] = __float2bfloat16_rn(x[v]);
+      l.a[v] = __float2bfloat16_rn(x[v] - __bfloat162float(h.a[v]));
+    }
+    __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(dst) + off_hi;
+    *reinterpret_cast<Pack<__nv_bfloat16, V>*>(d) = h;
+    *reinterpret_cast<Pack<__nv_bfloat16, V>*>(d + Kp) = l;
+  } else {
+    Pack<uint32_t, V> h, l;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      h.a[v] = to_tf32(x[v]);
+      l.a[v] = to_tf32(x[v] - __uint_as_float(h.a[v]));
+    }
+    uint32_t* d = reinterpret_cast<uint32_t*>(dst) + off_hi;
+    *reinterpret_cast<Pack<uint32_t, V>*>(d) = h;
+    *reinterpret_cast<Pack<uint32_t, V>*>(d + Kp) = l;
+  }
+}
+
+// The V fibers of a thread in memory. PACKED: neighbours, one 16-byte access
+// (every stride and address allows it). Otherwise fibers 32 apart, so that a
+// warp's V scalar accesses are each coalesced. at[]: element offsets of the
+// fibers, ok[]: false past the last fiber (such lanes read a valid fiber and
+// store nothing).
+template <typename T, int V, bool PACKED>
+struct Fibers {
+  static constexpr int N = PACKED ? 1 : V;
+  int64_t at[N];
+  bool ok[N];
+  __device__ __forceinline__ Pack<T, V> load(const T* in, int64_t off) const {
+    if (PACKED) return *reinterpret_cast<const Pack<T, V>*>(in + at[0] + off);
+    Pack<T, V> p;
+#pragma unroll
+    for (int v = 0; v < V; ++v) p.a[v] = in[at[PACKED ? 0 : v] + off];
+    return p;
+  }
+  // MODE 0: to out[base + off]; 1 / 2: to the bf16 / tf32 split operand
+  template <int MODE>
+  __device__ __forceinline__ void store(T* out, void* sdst, const int64_t (&base)[N], int64_t off,
+                                        int64_t Kp, const Pack<T, V>& x) const {
+    constexpr int KIND = MODE == 1 ? TC_BF16 : TC_TF32;
+    if (PACKED) {
+      if (!ok[0]) return;
+      if (MODE == 0) {
+        *reinterpret_cast<Pack<T, V>*>(out + base[0] + off) = x;
+      } else {
+        float f[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) f[v] = (float)x.a[v];
+        split_store_pack<KIND, V>(sdst, base[0] + off, Kp, f);
+      }
+    } else {
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (ok[PACKED ? 0 : v]) {
+          if (MODE == 0) out[base[PACKED ? 0 : v] + off] = x.a[v];
+          else split_store_f32<KIND>(sdst, base[PACKED ? 0 : v] + off, Kp, (float)x.a[v]);
+        }
+    }
+  }
+};
+
+// n / d with d's reciprocal in f while n < 2^31 (wide: beyond that).
+__device__ __forceinline__ int64_t div_by(const FastDiv& f, int64_t n, int64_t d, int wide) {
+  return wide ? n / d : (int64_t)f((uint32_t)n);
+}
+
+// One W-step. A block takes 32 V fibers (o1, o2, c), V to a lane, and its
+// eight warps share the work of each: first the P input rows to load into
+// shared memory, then the Q outputs to sum from there. Loops over all P x Q
+// entries with a thread per fiber had made this pass bound by its
+// multiply-adds (P = Q = 10, 381x500 fibers, float64: 60 us, now 16).
+// MODE 0: plain output, 1 / 2: split bf16 / tf32.
+constexpr int FIB_WARPS = 8;
+template <typename T, int MODE, int V, bool PACKED>
+__global__ void __launch_bounds__(32 * FIB_WARPS)
+    k_fiber(Fiber f, const double* __restrict__ Mat, const T* __restrict__ in, T* __restrict__ out,
+            void* __restrict__ sdst, int64_t Kcols, int64_t Kp, int staged, FastDiv by_nc,
+            FastDiv by_o2, int wide) {
+  extern __shared__ __align__(16) uint8_t fsm[];
+  __shared__ WTable<T> tab;
+  using F = Fibers<T, V, PACKED>;
+  const int P = (int)f.P, Q = (int)f.Q;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Pack<T, V>* xs = reinterpret_cast<Pack<T, V>*>(fsm) + lane;
+  gather_terms<T>(Mat, P, Q, tab);
+  const int64_t nc = PACKED ? f.nc / V : f.nc, total = f.n_o1 * f.n_o2 * nc;
+  for (int64_t e0 = (int64_t)blockIdx.x * (32 * F::N); e0 < total; e0 += (int64_t)gridDim.x * (32 * F::N)) {
+    F fib;
+    int64_t ob[F::N];
+#pragma unroll
+    for (int v = 0; v < F::N; ++v) {
+      const int64_t ev = e0 + 32 * v + lane, e = ev < total ? ev : e0;
+      const int64_t o12 = div_by(by_nc, e, nc, wide), o1 = div_by(by_o2, o12, f.n_o2, wide);
+      const int64_t c = (e - o12 * nc) * (PACKED ? V : 1), o2 = o12 - o1 * f.n_o2;
+      fib.ok[v] = ev < total;
+      fib.at[v] = o1 * f.is1 + o2 * f.is2 + c;
+      ob[v] = o1 * f.os1 + o2 * f.os2 + c;
+    }
+    if (staged) {
+#pragma unroll 4
+      for (int i = warp; i < P; i += FIB_WARPS) xs[i * 32] = fib.load(in, (int64_t)i * f.istride);
+      __syncthreads();
+    }
+    for (int o = warp; o < Q; o += FIB_WARPS) {
+      Pack<T, V> acc;
+      if (staged) {
+        acc = sum_terms<T, V>(tab, o, xs, 32);
+      } else {  // read where they are used
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc.a[v] = (T)0;
+        for (int i = 0; i < P; ++i) {
+          const T m = (T)Mat[i * Q + o];
+          if (m == (T)0) continue;
+          const Pack<T, V> x = fib.load(in, (int64_t)i * f.istride);
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc.a[v] = fma(m, x.a[v], acc.a[v]);
+        }
+      }
+      const int64_t off = (int64_t)o * f.ostride;
+      if (MODE == 0) {
+        fib.template store<MODE>(out, sdst, ob, off, Kp, acc);
+      } else {
+        int64_t sb[F::N];
+#pragma unroll
+        for (int v = 0; v < F::N; ++v) {
+          const int64_t row = (ob[v] + off) / Kcols;
+          sb[v] = row * 2 * Kp + (ob[v] + off - row * Kcols);
+        }
+        fib.template store<MODE>(out, sdst, sb, 0, Kp, acc);
+      }
+    }
+    if (staged) __syncthreads();  // the next fibers' inputs overwrite these
+  }
+}
+
+// 16-byte packs of neighbouring fibers: every stride and address allows them.
+template <typename T>
+bool packs(std::initializer_list<int64_t> strides, std::initializer_list<const void*> ptrs) {
+  constexpr int V = 16 / sizeof(T);
+  for (int64_t x : strides)
+    if (x % V != 0) return false;
+  for (const void* p : ptrs)
+    if ((reinterpret_cast<uintptr_t>(p) & 15) != 0) return false;
+  return true;
+}
+
+// Blocks of a W-step kernel: as many as share the SMs (sm bytes of shared
+// memory each), so that each builds its term table once.
+int wstep_blocks(int64_t groups, size_t sm) {
+  const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(2048 / (32 * FIB_WARPS), 225 * 1024 / (int64_t)sm));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(groups, 152 * per_sm));
 }
 
 template <typename T, int MODE>
 osmps_status fiber_dispatch(const Fiber& f, const double* Mat, const T* in, T* out, void* sdst,
                             int64_t Kcols, int64_t Kp, cudaStream_t s) {
   if (f.P <= 0 || f.Q <= 0 || f.nc <= 0 || f.n_o1 <= 0 || f.n_o2 <= 0) return OSMPS_OK;
-  const size_t sm = (size_t)f.P * f.Q * sizeof(T);
-  if (sm > 96 * 1024)
+  if ((size_t)f.P * f.Q * sizeof(T) > 96 * 1024)
     return set_error(OSMPS_EUNSUPPORTED, "W-step: MPO block %lld x %lld too large",
                      (long long)f.P, (long long)f.Q);
-  const int64_t total = f.n_o1 * f.n_o2 * f.nc;
-  const int threads = 256;
-  const int blocks = grid_for(total, threads);
-  if (f.Q <= 8) {
-    auto k = k_fiber<T, 8, MODE>;
-    if (sm > 48 * 1024) OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    { k<<<blocks, threads, sm, s>>>(f, Mat, in, out, sdst, Kcols, Kp); note_launch(); }
-  } else if (f.Q <= 16) {
-    auto k = k_fiber<T, 16, MODE>;
-    if (sm > 48 * 1024) OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    { k<<<blocks, threads, sm, s>>>(f, Mat, in, out, sdst, Kcols, Kp); note_launch(); }
-  } else if (f.Q <= 32) {
-    auto k = k_fiber<T, 32, MODE>;
-    if (sm > 48 * 1024) OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    { k<<<blocks, threads, sm, s>>>(f, Mat, in, out, sdst, Kcols, Kp); note_launch(); }
-  } else if (f.Q <= 64) {
-    auto k = k_fiber<T, 64, MODE>;
-    if (sm > 48 * 1024) OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    { k<<<blocks, threads, sm, s>>>(f, Mat, in, out, sdst, Kcols, Kp); note_launch(); }
-  } else {
+  if (f.Q > WT_QMAX)
     return set_error(OSMPS_EUNSUPPORTED, "W-step: output block %lld > 64", (long long)f.Q);
+  const auto launch = [&](auto k, int V, bool packed) -> osmps_status {
+    const int64_t nc = packed ? f.nc / V : f.nc, total = f.n_o1 * f.n_o2 * nc;
+    // the inputs of a block's fibers are staged while they leave room for two
+    // blocks per SM; past that they are read where they are used
+    const size_t stage = (size_t)f.P * 32 * V * sizeof(T);
+    const bool staged = stage <= 96 * 1024;
+    const size_t sm = staged ? stage : 0;
+    if (sm > 32 * 1024)
+      OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    const bool wide = total > 2147483647ll;
+    const FastDiv by_nc(wide ? 1 : (uint32_t)nc), by_o2(wide ? 1 : (uint32_t)f.n_o2);
+    const int blocks = wstep_blocks(cdiv(total, 32 * (packed ? 1 : V)), sm + sizeof(WTable<T>) + 1024);
+    k<<<blocks, 32 * FIB_WARPS, sm, s>>>(f, Mat, in, out, sdst, Kcols, Kp, staged ? 1 : 0, by_nc, by_o2,
+                                         wide ? 1 : 0);
+    note_launch();
+    OSMPS_LAUNCH_CHECK();
+    return OSMPS_OK;
+  };
+  constexpr int V = 16 / sizeof(T);
+  if (packs<T>({f.nc, f.is1, f.is2, f.istride, f.os1, f.os2, f.ostride, Kcols * (MODE != 0)}, {in, out, sdst}))
+    return launch(k_fiber<T, MODE, V, true>, V, true);
+  return launch(k_fiber<T, MODE, 2, false>, 2, false);
+}
+
+// Both W-steps of H_eff.theta in one pass for any MPO bond dimensions
+// (d1 = d2 = D), the work of 32 V fibers (a2, c) shared by a block's warps as
+// in k_fiber: they load the wl D D values T1[a2, w, s1, s2, c] into shared
+// memory, form T2[t1, w1, s2] beside them, then the outputs T3[t1, t2, w2], so
+// the intermediate never crosses memory. The sums are those of the two
+// separate passes, term by term. Traffic: one read of T1, one write of T3; in
+// float64 the ~36 FMAs per fiber come next (XXZ chi = 512: 55 us, float64 pipe
+// 44% active, against 158 + 158 us for two dense passes); AKLT 301x257 in
+// float32 61 us against 152 + 147.
+template <typename T, int MODE, int D, int V, bool PACKED>
+__global__ void __launch_bounds__(32 * FIB_WARPS)
+    k_wsteps(const T* __restrict__ T1, const double* __restrict__ Mat1,
+             const double* __restrict__ Mat2, int wl, int wm, int wr, T* __restrict__ out,
+             void* __restrict__ sdst, int64_t Kp, int64_t chi_l, int64_t chi_r, FastDiv by_c,
+             int wide) {
+  extern __shared__ __align__(16) uint8_t fsm[];
+  __shared__ WTable<T> tab1, tab2;
+  __shared__ int64_t ooff[WT_QMAX];  // output (t2, w2): offset from (t1, 0, 0)
+  using F = Fibers<T, V, PACKED>;
+  const int P1 = wl * D, Q1 = D * wm, P2 = wm * D, Q2 = D * wr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Pack<T, V>* xs = reinterpret_cast<Pack<T, V>*>(fsm) + lane;
+  Pack<T, V>* ms = xs + P1 * D * 32;
+  const int64_t ldo = MODE == 0 ? wr * chi_r : 2 * Kp;
+  if (threadIdx.x < Q2) {
+    const int t2 = threadIdx.x / wr;
+    ooff[threadIdx.x] = t2 * ldo + (int64_t)(threadIdx.x - t2 * wr) * chi_r;
   }
-  OSMPS_LAUNCH_CHECK();
+  gather_terms<T>(Mat1, P1, Q1, tab1);
+  gather_terms<T>(Mat2, P2, Q2, tab2);
+  const int64_t nc = PACKED ? chi_r / V : chi_r, total = chi_l * nc;
+  for (int64_t e0 = (int64_t)blockIdx.x * (32 * F::N); e0 < total; e0 += (int64_t)gridDim.x * (32 * F::N)) {
+    F fib;
+    int64_t ob[F::N];
+#pragma unroll
+    for (int v = 0; v < F::N; ++v) {
+      const int64_t ev = e0 + 32 * v + lane, e = ev < total ? ev : e0;
+      const int64_t a2 = div_by(by_c, e, nc, wide), c = (e - a2 * nc) * (PACKED ? V : 1);
+      fib.ok[v] = ev < total;
+      fib.at[v] = a2 * (P1 * D) * chi_r + c;
+      ob[v] = a2 * (D * D) * ldo + c;
+    }
+#pragma unroll 4
+    for (int k = warp; k < P1 * D; k += FIB_WARPS) xs[k * 32] = fib.load(T1, k * chi_r);
+    __syncthreads();
+    for (int o = warp; o < Q1; o += FIB_WARPS)
+#pragma unroll
+      for (int s2 = 0; s2 < D; ++s2) ms[(o * D + s2) * 32] = sum_terms<T, V>(tab1, o, xs + s2 * 32, D * 32);
+    __syncthreads();  // T2 complete; T1's copy may be overwritten by the next fibers
+    for (int o = warp; o < Q2; o += FIB_WARPS)
+#pragma unroll
+      for (int t1 = 0; t1 < D; ++t1)
+        fib.template store<MODE>(out, sdst, ob, t1 * D * ldo + ooff[o], Kp,
+                                 sum_terms<T, V>(tab2, o, ms + t1 * (P2 * 32), 32));
+    // (the next fibers' T2 is written only after the barrier that follows their loads)
+  }
+}
+
+// *done = false where the fused pass does not apply (physical dimensions
+// other than 2 to 5, MPO blocks beyond the separate passes' own limits, or
+// columns of which not 64 fit shared memory).
+template <typename T, int MODE>
+osmps_status wsteps_dispatch(const T* T1, const double* Mat1, const double* Mat2, int64_t chi_l,
+                             int64_t d1, int64_t d2, int64_t chi_r, int64_t wl, int64_t wm,
+                             int64_t wr, T* out, void* sdst, int64_t Kp, cudaStream_t s,
+                             bool* done) {
+  *done = false;
+  if (d1 != d2 || d1 < 2 || d1 > 5 || d1 * std::max(wm, wr) > WT_QMAX || d1 * wl > 2048) return OSMPS_OK;
+  const int64_t P1 = wl * d1, Q1 = d1 * wm, P2 = wm * d1, Q2 = d1 * wr;
+  if ((size_t)std::max(P1 * Q1, P2 * Q2) * sizeof(T) > 96 * 1024) return OSMPS_OK;
+  // 16-byte packs of neighbouring fibers while two blocks still share an SM,
+  // else two fibers 32 apart
+  const size_t column = (size_t)(P1 + Q1) * d1 * sizeof(T);  // one fiber's T1 and T2
+  constexpr size_t MOST = 180 * 1024;
+  constexpr int VMAX = 16 / sizeof(T);
+  if (column * 64 > MOST) return OSMPS_OK;
+  const bool packed = column * 32 * VMAX <= 90 * 1024 && packs<T>({chi_r}, {T1, out, sdst});
+  const auto launch = [&](auto k, int V) -> osmps_status {
+    const size_t sm = column * 32 * V;
+    const int64_t nc = packed ? chi_r / V : chi_r, total = chi_l * nc;
+    const bool wide = total > 2147483647ll;
+    const FastDiv by_c(wide ? 1 : (uint32_t)nc);
+    const int blocks = wstep_blocks(cdiv(total, 32 * (packed ? 1 : V)), sm + 2 * sizeof(WTable<T>) + 1600);
+    if (sm > 24 * 1024)
+      OSMPS_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MOST));
+    k<<<blocks, 32 * FIB_WARPS, sm, s>>>(T1, Mat1, Mat2, (int)wl, (int)wm, (int)wr, out, sdst, Kp, chi_l,
+                                         chi_r, by_c, wide ? 1 : 0);
+    note_launch();
+    OSMPS_LAUNCH_CHECK();
+    return OSMPS_OK;
+  };
+#define OSMPS_WSTEPS(D_) \
+  OSMPS_TRY(packed ? launch(k_wsteps<T, MODE, D_, VMAX, true>, VMAX) : launch(k_wsteps<T, MODE, D_, 2, false>, 2))
+  if (d1 == 2) OSMPS_WSTEPS(2);
+  else if (d1 == 3) OSMPS_WSTEPS(3);
+  else if (d1 == 4) OSMPS_WSTEPS(4);
+  else OSMPS_WSTEPS(5);
+#undef OSMPS_WSTEPS
+  *done = true;
   return OSMPS_OK;
 }
 
@@ -471,6 +807,13 @@ osmps_status fiber_contract_f32_split(const Fiber& f, const double* Mat, const f
   return fiber_dispatch<float, 2>(f, Mat, in, nullptr, dst, Kcols, Kp, s);
 }
 
+osmps_status wsteps_f64(const double* T1, const double* Mat1, const double* Mat2, double* T3,
+                        int64_t chi_l, int64_t d1, int64_t d2, int64_t chi_r, int64_t wl,
+                        int64_t wm, int64_t wr, cudaStream_t s, bool* done) {
+  return wsteps_dispatch<double, 0>(T1, Mat1, Mat2, chi_l, d1, d2, chi_r, wl, wm, wr, T3, nullptr,
+                                    0, s, done);
+}
+
 // max over (a, b) of |E[a, w, b] - delta_ab| for w = 0 (blockIdx.y = 0) and
 // w = w_count - 1 (blockIdx.y = 1), as the bit patterns of non-negative
 // doubles (ordered like the values) combined by atomicMax
@@ -527,8 +870,14 @@ osmps_status fused_wsteps_f32_split(const float* T1, const double* Mat1, const d
   *done = false;
   if ((id.skip_l >= 0 && !id.theta) || (id.skip_r >= 0 && !id.yid))
     return set_error(OSMPS_EINVAL, "fused W-steps: identity channel without its buffer");
-  if (!fused_dispatch(d1, d2, wl, wm, wr, kind, T1, Mat1, Mat2, dst, chi_l, chi_r, Kp, id, s, true))
-    return OSMPS_OK;
+  if (!fused_dispatch(d1, d2, wl, wm, wr, kind, T1, Mat1, Mat2, dst, chi_l, chi_r, Kp, id, s, true)) {
+    if (id.skip_l >= 0 || id.skip_r >= 0) return OSMPS_OK;
+    if (kind == TC_BF16)
+      return wsteps_dispatch<float, 1>(T1, Mat1, Mat2, chi_l, d1, d2, chi_r, wl, wm, wr, nullptr,
+                                       dst, Kp, s, done);
+    return wsteps_dispatch<float, 2>(T1, Mat1, Mat2, chi_l, d1, d2, chi_r, wl, wm, wr, nullptr, dst,
+                                     Kp, s, done);
+  }
   OSMPS_LAUNCH_CHECK();
   *done = true;
   return OSMPS_OK;
