@@ -217,6 +217,20 @@ osmps_status pinned_reserve(osmps_ctx* ctx, size_t count);
 __host__ __device__ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return cdiv(a, b) * b; }
 
+// n / d for 0 <= n < 2^31 by a multiplication and a shift (Granlund and
+// Montgomery, PLDI 1994): a 64-bit division costs more than a whole fiber.
+struct FastDiv {
+  uint32_t d = 1, m = 0, s = 0;
+  FastDiv() = default;
+  explicit FastDiv(uint32_t div) : d(div) {
+    while (s < 32 && (1ull << s) < div) ++s;
+    m = (uint32_t)((((1ull << s) - div) << 32) / div + 1);
+  }
+  __device__ __forceinline__ uint32_t operator()(uint32_t n) const {
+    return (uint32_t)(((uint64_t)__umulhi(m, n) + n) >> s);
+  }
+};
+
 // ---------------------------------------------------------------------------
 // Float64 strided batched GEMM: C[b] = alpha * A[b] B[b] + beta * C[b] with
 // element (m,k) of A at A[b*sab + m*sam + k*sak] (likewise B (k,n), C (m,n)).
@@ -394,6 +408,9 @@ enum WOrder {
 };
 osmps_status w_reorder(const double* W, int64_t dw, int64_t d, int64_t dw2, int order, double* Mat,
                        cudaStream_t stream);
+// Both site tensors of H_eff in the left-side order, one launch.
+osmps_status w_reorder_pair(const double* W1, const double* W2, int64_t wl, int64_t d1, int64_t wm,
+                            int64_t d2, int64_t wr, double* M1, double* M2, cudaStream_t stream);
 
 // ---------------------------------------------------------------------------
 // Vector primitives (float64) used by Lanczos and normalisations.

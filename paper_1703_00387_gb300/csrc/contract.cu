@@ -39,8 +39,7 @@ osmps_status heff_prepare(osmps_ctx* ctx, const double* L, const double* W1, con
   const int64_t P1 = wl * d1, Q1 = d1 * wm, P2 = wm * d2, Q2 = d2 * wr;
   double* small = (double*)ws_get(ctx, SLOT_HEFF_SMALL, (P1 * Q1 + P2 * Q2) * sizeof(double), stream, &st);
   if (!small) return st;
-  OSMPS_TRY(w_reorder(W1, wl, d1, wm, WORD_IN_W_S__OUT_T_W2, small, stream));
-  OSMPS_TRY(w_reorder(W2, wm, d2, wr, WORD_IN_W_S__OUT_T_W2, small + P1 * Q1, stream));
+  OSMPS_TRY(w_reorder_pair(W1, W2, wl, d1, wm, d2, wr, small, small + P1 * Q1, stream));
   if (precision == OSMPS_PREC_FP64 || precision == OSMPS_PREC_FP64_EMU) {
     OSMPS_TRY(prepare_f64_copies(ctx, L, R, chi_l, chi_r, wl, wr, stream));
   } else {

@@ -320,13 +320,6 @@ __global__ void __launch_bounds__(E_THREADS, 1)
 // ---------------------------------------------------------------------------
 // Slicing
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double load_view(const SplitView& v, int64_t r, int64_t k) {
-  const int64_t r0 = r / v.n1, r1 = r - r0 * v.n1;
-  const int64_t off = r0 * v.s0 + r1 * v.s1 + k * v.sk;
-  return v.src_f32 ? (double)reinterpret_cast<const float*>(v.src)[off]
-                   : reinterpret_cast<const double*>(v.src)[off];
-}
-
 // Biased exponent field of |x| (0 for zero and subnormals): comparing the
 // magnitude bits as integers orders doubles by size.
 __device__ __forceinline__ unsigned long long mag_bits(double x) {
@@ -336,48 +329,6 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
 __device__ __forceinline__ int exponent_of_max(unsigned long long mbits) {
   const int E = (int)(mbits >> 52);
   return E == 0 ? 0 : E - 1022;  // |x| < 2^(E - 1022) for every x of the row
-}
-
-// e[r] for rows whose K index is contiguous: one block per row.
-__global__ void k_rowexp_contig(SplitView v, int* __restrict__ e) {
-  __shared__ unsigned long long sh[8];
-  const int64_t r = blockIdx.x;
-  unsigned long long m = 0;
-  for (int64_t k = threadIdx.x; k < v.K; k += blockDim.x) m = max(m, mag_bits(load_view(v, r, k)));
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) m = max(m, sh[i]);
-    e[r] = exponent_of_max(max(m, sh[0]));
-  }
-}
-
-// Row maxima (of the magnitude bits) for rows that are adjacent in memory (K
-// strided): 32 rows x a chunk of K per block, threads along the rows read
-// neighbouring addresses; partial maxima combined with atomicMax into m[r].
-constexpr int ROWMAX_KCHUNK = 256;
-__global__ void k_rowmax_strided(SplitView v, unsigned long long* __restrict__ m) {
-  __shared__ unsigned long long sh[8][33];
-  const int64_t r = (int64_t)blockIdx.x * 32 + threadIdx.x;
-  const int64_t k0 = (int64_t)blockIdx.y * ROWMAX_KCHUNK;
-  const int64_t k1 = min(k0 + (int64_t)ROWMAX_KCHUNK, v.K);
-  unsigned long long a = 0;
-  if (r < v.rows)
-    for (int64_t k = k0 + threadIdx.y; k < k1; k += 8) a = max(a, mag_bits(load_view(v, r, k)));
-  sh[threadIdx.y][threadIdx.x] = a;
-  __syncthreads();
-  if (threadIdx.y == 0 && r < v.rows) {
-    for (int i = 1; i < 8; ++i) a = max(a, sh[i][threadIdx.x]);
-    atomicMax(&m[r], a);
-  }
-}
-
-__global__ void k_exp_from_max(const unsigned long long* __restrict__ m, int64_t rows,
-                               int* __restrict__ e) {
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
-       r += (int64_t)gridDim.x * blockDim.x)
-    e[r] = exponent_of_max(m[r]);
 }
 
 // x * 2^(56 - e) rounded to the nearest integer, from the IEEE bits (integer
@@ -397,74 +348,170 @@ __device__ __forceinline__ long long fixed56(double x, int e) {
 
 // Balanced base-128 digits of X: X = sum_p d_p 128^(7 - p); d_1..d_7 in
 // [-64, 63], d_0 in [-128, 128]; slice p of the operand is the integer d_p
-// (exact in bf16) and stands for d_p 2^(-7 (p + 1)) 2^e.
-__device__ __forceinline__ void store_slices(__nv_bfloat16* dst, int64_t base, int64_t Kp, double x,
-                                             int e) {
-  long long X = fixed56(x, e);
-  int d[SLICES];
+// (exact in bf16) and stands for d_p 2^(-7 (p + 1)) 2^e. Eight consecutive
+// columns of a row are cut together and stored 16 bytes per slice. An integer
+// |d| < 2^22 added to the bits of 1.5 2^23 is that float plus d, so the
+// difference is (float)d without a conversion; its upper half is the bf16.
+__device__ __forceinline__ void store_slices8(__nv_bfloat16* dst, int64_t base, int64_t Kp,
+                                              const long long (&Xs)[8]) {
+  uint32_t w[SLICES][4];
 #pragma unroll
-  for (int p = SLICES - 1; p > 0; --p) {
-    const int dig = (int)(((X + 64) & 127) - 64);
-    d[p] = dig;
-    X = (X - dig) >> SLICE_BITS;
+  for (int i = 0; i < 4; ++i) {
+    long long X0 = Xs[2 * i], X1 = Xs[2 * i + 1];
+#pragma unroll
+    for (int p = SLICES - 1; p >= 0; --p) {
+      int d0 = (int)X0, d1 = (int)X1;
+      if (p > 0) {
+        d0 = (int)(((uint32_t)d0 + 64u) & 127u) - 64;
+        d1 = (int)(((uint32_t)d1 + 64u) & 127u) - 64;
+        X0 = (X0 - d0) >> SLICE_BITS;
+        X1 = (X1 - d1) >> SLICE_BITS;
+      }
+      const float f0 = __int_as_float(0x4B400000 + d0) - 12582912.0f;
+      const float f1 = __int_as_float(0x4B400000 + d1) - 12582912.0f;
+      w[p][i] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+    }
   }
-  d[0] = (int)X;
 #pragma unroll
-  for (int p = 0; p < SLICES; ++p) dst[base + (int64_t)p * Kp] = __float2bfloat16_rn((float)d[p]);
+  for (int p = 0; p < SLICES; ++p)
+    *reinterpret_cast<uint4*>(dst + base + (int64_t)p * Kp) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
 }
 
-__global__ void k_slice_direct(SplitView v, const int* __restrict__ e, __nv_bfloat16* __restrict__ dst,
-                               int64_t Kp) {
-  const int64_t total = v.rows * Kp;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / Kp, k = t - r * Kp;
-    const double x = (k < v.K) ? load_view(v, r, k) : 0.0;
-    store_slices(dst, r * SLICES * Kp + k, Kp, x, e[r]);
+// Rows whose K index is contiguous: one block per row finds the row's largest
+// exponent, writes it to e[r] and cuts the row (read a second time from L1
+// where it is longer than eight columns per thread).
+template <typename S>
+__global__ void __launch_bounds__(256) k_slice_rows(SplitView v, int* __restrict__ e,
+                                                    __nv_bfloat16* __restrict__ dst, int64_t Kp,
+                                                    int vec) {
+  __shared__ unsigned long long sh[8];
+  const int64_t r = blockIdx.x, r0 = r / v.n1, r1 = r - r0 * v.n1;
+  const S* src = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1;
+  const auto load = [&](int64_t k, double (&x)[8]) {
+    if (vec && k + 8 <= v.K) {
+      constexpr int PER = 16 / sizeof(S);
+      S q[8];
+#pragma unroll
+      for (int i = 0; i < 8; i += PER)
+        *reinterpret_cast<uint4*>(q + i) = *reinterpret_cast<const uint4*>(src + k + i);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = (double)q[i];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = k + i < v.K ? (double)src[k + i] : 0.0;
+    }
+  };
+  const int64_t step = 8 * (int64_t)blockDim.x, first = 8 * (int64_t)threadIdx.x;
+  double x[8];
+  unsigned long long m = 0;
+  if (first < Kp) load(first, x);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) m = first < Kp ? max(m, mag_bits(x[i])) : m;
+  for (int64_t k = first + step; k < Kp; k += step) {
+    double y[8];
+    load(k, y);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = max(m, mag_bits(y[i]));
+  }
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  __syncthreads();
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = max(m, sh[i]);
+  const int ex = exponent_of_max(m);
+  if (threadIdx.x == 0) e[r] = ex;
+  for (int64_t k = first; k < Kp; k += step) {
+    if (k != first) load(k, x);
+    long long X[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) X[i] = fixed56(x[i], ex);
+    store_slices8(dst, r * SLICES * Kp + k, Kp, X);
   }
 }
 
-__global__ void k_slice_transpose(SplitView v, const int* __restrict__ e,
-                                  __nv_bfloat16* __restrict__ dst, int64_t Kp) {
-  __shared__ double tile[32][33];
-  const int64_t r_base = (int64_t)blockIdx.x * 32, k_base = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t k = k_base + j, r = r_base + tx;
-    tile[j][tx] = (k < v.K && r < v.rows) ? load_view(v, r, k) : 0.0;
+// Rows that are adjacent in memory (K strided), first pass: row maxima of the
+// magnitude bits, 64 rows x a chunk of K per block, neighbouring threads on
+// neighbouring rows, partial maxima combined with atomicMax into m[r].
+constexpr int ROWMAX_KCHUNK = 256;
+template <typename S>
+__global__ void __launch_bounds__(256) k_rowmax_strided(SplitView v, unsigned long long* __restrict__ m) {
+  __shared__ unsigned long long sh[4][64];
+  const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+  const int64_t r = (int64_t)blockIdx.x * 64 + tx, rr = r < v.rows ? r : 0;
+  const int64_t r0 = rr / v.n1, r1 = rr - r0 * v.n1;
+  const S* src = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1;
+  const int64_t k0 = (int64_t)blockIdx.y * ROWMAX_KCHUNK, k1 = min(k0 + (int64_t)ROWMAX_KCHUNK, v.K);
+  unsigned long long a = 0;
+#pragma unroll 8
+  for (int64_t k = k0 + ty; k < k1; k += 4) a = max(a, mag_bits((double)src[k * v.sk]));
+  sh[ty][tx] = a;
+  __syncthreads();
+  if (ty == 0 && r < v.rows) {
+    for (int i = 1; i < 4; ++i) a = max(a, sh[i][tx]);
+    atomicMax(&m[r], a);
+  }
+}
+
+// Second pass: tiles of 64 rows x 64 columns read along the rows, brought to
+// fixed point, and cut along the columns through shared memory. The blocks of
+// the first column tile also write the exponents.
+template <typename S>
+__global__ void __launch_bounds__(256) k_slice_transpose(SplitView v,
+                                                         const unsigned long long* __restrict__ m,
+                                                         int* __restrict__ e,
+                                                         __nv_bfloat16* __restrict__ dst, int64_t Kp) {
+  __shared__ long long tile[64][65];
+  const int64_t r_base = (int64_t)blockIdx.x * 64, k_base = (int64_t)blockIdx.y * 64;
+  {
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int64_t r = r_base + tx, rr = r < v.rows ? r : 0;
+    const int64_t r0 = rr / v.n1, r1 = rr - r0 * v.n1;
+    const S* p = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1 + (k_base + ty) * v.sk;
+    S x[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      x[j] = (r < v.rows && k_base + ty + 4 * j < v.K) ? p[4 * j * v.sk] : (S)0;
+    const int ex = exponent_of_max(m[rr]);
+    if (blockIdx.y == 0 && ty == 0 && r < v.rows) e[r] = ex;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tile[ty + 4 * j][tx] = fixed56((double)x[j], ex);
   }
   __syncthreads();
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t r = r_base + j, k = k_base + tx;
-    if (r < v.rows && k < Kp) store_slices(dst, r * SLICES * Kp + k, Kp, tile[tx][j], e[r]);
+  for (int u = threadIdx.x; u < 512; u += 256) {
+    const int row = u >> 3, g = 8 * (u & 7);
+    if (r_base + row >= v.rows) continue;
+    long long X[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) X[i] = tile[g + i][row];
+    store_slices8(dst, (r_base + row) * SLICES * Kp + k_base + g, Kp, X);
   }
 }
 
-int blocks_1d(int64_t n, int t) {
-  int64_t b = cdiv(n, t);
-  return (int)std::max<int64_t>(1, std::min<int64_t>(b, 65536));
-}
-
+// Traffic: 8 bytes read (twice for strided rows) and 16 written per value.
+template <typename S>
 osmps_status slice_operand(osmps_ctx* ctx, const SplitView& v, int64_t Kp, int* e,
                            __nv_bfloat16* dst, cudaStream_t s) {
   if (v.rows <= 0) return OSMPS_OK;
-  const bool contig = (v.sk == 1);
-  if (contig) {
+  if (v.sk == 1) {
     if (v.rows > 2147483647ll) return set_error(OSMPS_ESHAPE, "emulated GEMM: too many rows");
-    { k_rowexp_contig<<<(unsigned)v.rows, 256, 0, s>>>(v, e); note_launch(); }
-    { k_slice_direct<<<blocks_1d(v.rows * Kp, 256), 256, 0, s>>>(v, e, dst, Kp); note_launch(); }
+    constexpr int64_t PER = 16 / sizeof(S);
+    const bool vec = (reinterpret_cast<uintptr_t>(v.src) & 15) == 0 && v.s0 % PER == 0 &&
+                     (v.n1 == 1 || v.s1 % PER == 0);
+    const int threads = (int)std::min<int64_t>(256, round_up(cdiv(Kp, 8), 32));
+    k_slice_rows<S><<<(unsigned)v.rows, threads, 0, s>>>(v, e, dst, Kp, vec ? 1 : 0);
+    note_launch();
   } else {
-    if (cdiv(Kp, 32) > 65535 || cdiv(v.K, ROWMAX_KCHUNK) > 65535)
+    if (cdiv(Kp, 64) > 65535 || cdiv(v.K, ROWMAX_KCHUNK) > 65535)
       return set_error(OSMPS_ESHAPE, "emulated GEMM: K too large");
     osmps_status st = OSMPS_OK;
     auto* mx = (unsigned long long*)ws_get(ctx, SLOT_EMU_MAX, (size_t)v.rows * 8, s, &st);
     if (!mx) return st;
     OSMPS_CUDA(cudaMemsetAsync(mx, 0, (size_t)v.rows * 8, s));
-    dim3 g1((unsigned)cdiv(v.rows, 32), (unsigned)std::max<int64_t>(1, cdiv(v.K, ROWMAX_KCHUNK)));
-    { k_rowmax_strided<<<g1, dim3(32, 8), 0, s>>>(v, mx); note_launch(); }
-    { k_exp_from_max<<<blocks_1d(v.rows, 256), 256, 0, s>>>(mx, v.rows, e); note_launch(); }
-    dim3 grid((unsigned)cdiv(v.rows, 32), (unsigned)cdiv(Kp, 32));
-    { k_slice_transpose<<<grid, dim3(32, 8), 0, s>>>(v, e, dst, Kp); note_launch(); }
+    const dim3 g1((unsigned)cdiv(v.rows, 64), (unsigned)std::max<int64_t>(1, cdiv(v.K, ROWMAX_KCHUNK)));
+    k_rowmax_strided<S><<<g1, 256, 0, s>>>(v, mx);
+    note_launch();
+    const dim3 grid((unsigned)cdiv(v.rows, 64), (unsigned)cdiv(Kp, 64));
+    k_slice_transpose<S><<<grid, 256, 0, s>>>(v, mx, e, dst, Kp);
+    note_launch();
   }
   OSMPS_LAUNCH_CHECK();
   return OSMPS_OK;
@@ -517,8 +564,8 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   if (!ex) return st;
   int* eA = ex;
   int* eB = ex + ((M + 63) / 64) * 64;
-  OSMPS_TRY(slice_operand(ctx, a, Kp, eA, sa, s));
-  OSMPS_TRY(slice_operand(ctx, b, Kp, eB, sb, s));
+  OSMPS_TRY(a.src_f32 ? slice_operand<float>(ctx, a, Kp, eA, sa, s) : slice_operand<double>(ctx, a, Kp, eA, sa, s));
+  OSMPS_TRY(b.src_f32 ? slice_operand<float>(ctx, b, Kp, eB, sb, s) : slice_operand<double>(ctx, b, Kp, eB, sb, s));
   CUtensorMap ma, mb;
   OSMPS_TRY(tc_make_map(&ma, sa, TC_BF16, M, SLICES * Kp, EBM));
   OSMPS_TRY(tc_make_map(&mb, sb, TC_BF16, N, SLICES * Kp, EBN));

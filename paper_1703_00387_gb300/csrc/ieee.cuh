@@ -45,33 +45,70 @@ __device__ __forceinline__ float f64_to_f32_rn(double x) {
   return __uint_as_float((uint32_t)(b >> 63) << 31 | mag);
 }
 
-// (float)x rounded to odd: the fraction truncated to 23 bits, its last bit
-// set when any dropped bit was set. Rounding that to nearest-even at 7
-// fraction bits (bf16) equals rounding x to bf16 directly, since float keeps
-// more than 7 + 2 bits (the round-to-odd argument of Boldo and Melquiond,
-// "Emulation of FMA and correctly rounded sums: proved algorithms using
-// rounding to odd", IEEE Trans. Computers 57 (2008)). Normal floats only:
-// returns false (and leaves *out) when x is zero, subnormal, infinite, NaN
-// or outside the float exponent range.
-__device__ __forceinline__ bool f64_to_f32_odd(double x, float* out) {
-  const uint64_t b = (uint64_t)__double_as_longlong(x);
-  const int ef = (int)((b >> 52) & 0x7FFu) - 896;
-  if (ef < 1 || ef > 254) return false;
-  const uint64_t frac = b & 0xFFFFFFFFFFFFFull;
-  const uint32_t keep = (uint32_t)(frac >> 29) | ((frac & 0x1FFFFFFFu) != 0 ? 1u : 0u);
-  *out = __uint_as_float((uint32_t)(b >> 63) << 31 | ((uint32_t)ef << 23) | keep);
-  return true;
+// The rounded magnitude a (a > 0, leading bit p) at 2^n kept bits, n = 8 or
+// 24: a 2^(n - 1 - p) to nearest-even, in [2^(n-1), 2^n].
+template <int N>
+__device__ __forceinline__ uint32_t round_bits(uint64_t a, int p) {
+  if (p < N) return (uint32_t)(a << (N - 1 - p));
+  const int s = p - (N - 1);
+  return (uint32_t)((a + ((1ull << (s - 1)) - 1) + ((a >> s) & 1)) >> s);
 }
 
-// x rounded to nearest-even bf16: through float32 rounded to odd (integer
-// fields, exact under the double rounding), then the float-to-bf16
-// conversion; signed zeros directly, the hardware conversion where x is not
-// a normal float.
-__device__ __forceinline__ __nv_bfloat16 f64_to_bf16_rn(double x) {
+// x as a bf16 pair, hi = x and lo = x - hi rounded to nearest-even, with
+// integer operations: the rounded mantissa of hi, the exact difference of the
+// 53-bit mantissas and its rounding. The raw bits come back as hi | lo << 16.
+// Through the float64 pipe (two conversions and a subtraction per value) this
+// split was what bound the operand passes: 5.2M values 41 us. Values whose hi
+// or lo is not a normal bf16 number go through the hardware conversions.
+__device__ __forceinline__ uint32_t f64_to_bf16_pair(double x) {
   const uint64_t b = (uint64_t)__double_as_longlong(x);
-  if ((b << 1) == 0) return __ushort_as_bfloat16((unsigned short)((b >> 48) & 0x8000u));
-  float xo;
-  return f64_to_f32_odd(x, &xo) ? __float2bfloat16_rn(xo) : __double2bfloat16(x);
+  if ((b << 1) == 0) return (uint32_t)(b >> 48) & 0x8000u;  // +-0, lo = +0
+  const int E = (int)((b >> 52) & 0x7FFu);
+  const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const uint32_t sign = (uint32_t)(b >> 48) & 0x8000u;
+  const int ef = E - 896;  // bf16 biased exponent of hi
+  const uint32_t hm = round_bits<8>(m, 52);
+  const int64_t R = (int64_t)(m - ((uint64_t)hm << 45));
+  const uint64_t a = (uint64_t)(R < 0 ? -R : R);
+  const int p = a ? 63 - __clzll((long long)a) : 0;
+  const int el = p + E - 948;  // bf16 biased exponent of lo
+  if (ef < 1 || ef > 253 || (a != 0 && el < 1)) {
+    const __nv_bfloat16 h = __double2bfloat16(x);
+    const __nv_bfloat16 l = __double2bfloat16(x - (double)__bfloat162float(h));
+    return (uint32_t)__bfloat16_as_ushort(h) | (uint32_t)__bfloat16_as_ushort(l) << 16;
+  }
+  const uint32_t hi = sign | (((uint32_t)ef << 7) + hm - 128u);
+  if (a == 0) return hi;  // lo = +0
+  const uint32_t lo = (R < 0 ? sign ^ 0x8000u : sign) | (((uint32_t)el << 7) + round_bits<8>(a, p) - 128u);
+  return hi | lo << 16;
+}
+
+__device__ __forceinline__ uint32_t cvt_rna_tf32(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return r;
+}
+
+// x as a tf32 pair: hi = x and lo = x - hi, each rounded to float32 (nearest
+// even) and then to tf32 (ties away), the difference exact as above.
+__device__ __forceinline__ uint2 f64_to_tf32_pair(double x) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  const int E = (int)((b >> 52) & 0x7FFu);
+  const uint32_t h = cvt_rna_tf32(f64_to_f32_rn(x));
+  const int eh = (int)((h >> 23) & 0xFFu);  // E - 896, or one more after a carry
+  const uint64_t m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const uint64_t hm = (uint64_t)((h & 0x7FFFFFu) | 0x800000u);
+  const int up = eh - (E - 896);
+  const int64_t R = (int64_t)(m - (hm << (29 + (up & 1))));
+  const uint64_t a = (uint64_t)(R < 0 ? -R : R);
+  const int p = a ? 63 - __clzll((long long)a) : 0;
+  const int el = p + E - 948;  // float biased exponent of x - hi
+  if ((b << 1) == 0 || E < 897 || E > 1149 || (unsigned)up > 1u || (a != 0 && el < 1))
+    return make_uint2(h, cvt_rna_tf32((float)(x - (double)__uint_as_float(h))));
+  if (a == 0) return make_uint2(h, 0u);
+  const uint32_t sign = (uint32_t)(b >> 63) << 31;
+  const uint32_t lf = (R < 0 ? sign ^ 0x80000000u : sign) | (((uint32_t)el << 23) + round_bits<24>(a, p) - 0x800000u);
+  return make_uint2(h, cvt_rna_tf32(__uint_as_float(lf)));
 }
 
 }  // namespace osmps

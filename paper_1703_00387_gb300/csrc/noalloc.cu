@@ -152,8 +152,7 @@ extern "C" osmps_status osmps_heff_apply_noalloc(const double* L, const double* 
 
   // Every scratch region below is fully written before it is read, so the
   // previous call's contents never leak into this one.
-  OSMPS_TRY(w_reorder(W1, wl, d1, wm, WORD_IN_W_S__OUT_T_W2, mat1, s));
-  OSMPS_TRY(w_reorder(W2, wm, d2, wr, WORD_IN_W_S__OUT_T_W2, mat2, s));
+  OSMPS_TRY(w_reorder_pair(W1, W2, wl, d1, wm, d2, wr, mat1, mat2, s));
   GemmF64 g1;  // T1[(a2,w),(s1,s2,c)] = L[(a2,w),a] theta[a,(s1,s2,c)]
   g1.M = chi_l * wl; g1.N = N1; g1.K = chi_l;
   g1.A = L; g1.sam = chi_l; g1.sak = 1;

@@ -3,7 +3,7 @@
 // * split_operand: float64/float32 -> [hi | lo] rows in bf16 or tf32 for the
 //   tensor-core GEMM (x = hi + lo + O(2^-17 |x|) for bf16, O(2^-22 |x|) for tf32).
 //   Rows are written K-major; a source whose K index is not contiguous is read
-//   through a 32 x 32 shared-memory transpose so both sides stay coalesced.
+//   through a shared-memory transpose so both sides stay coalesced.
 // * fiber contractions: the W-steps of Sec. 3.4, where the MPO tensors
 //   M^[k] (few entries, Eq. MPOdef) act on the small (w, s) index pair of an
 //   intermediate, for every (outer, inner) fiber. These are bandwidth-bound:
@@ -13,35 +13,15 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "operand.cuh"
 
 namespace osmps {
 
 namespace {
 
-__device__ __forceinline__ uint32_t to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
-template <int KIND>
-__device__ __forceinline__ void split_store(void* dst, int64_t off_hi, int64_t Kp, double x) {
-  if (KIND == TC_BF16) {
-    __nv_bfloat16 h = __double2bfloat16(x);
-    __nv_bfloat16 l = __double2bfloat16(x - (double)__bfloat162float(h));
-    reinterpret_cast<__nv_bfloat16*>(dst)[off_hi] = h;
-    reinterpret_cast<__nv_bfloat16*>(dst)[off_hi + Kp] = l;
-  } else {
-    uint32_t h = to_tf32((float)x);
-    uint32_t l = to_tf32((float)(x - (double)__uint_as_float(h)));
-    reinterpret_cast<uint32_t*>(dst)[off_hi] = h;
-    reinterpret_cast<uint32_t*>(dst)[off_hi + Kp] = l;
-  }
-}
-
-// The same split for a float32 value with float32 arithmetic only (the
-// float64 pipe is narrow on this GPU). x - hi is exact in float32 (hi keeps
-// the leading bits of x), so the result equals split_store's bit for bit.
+// The hi / lo split of a float32 value (x - hi is exact in float32: hi keeps
+// the leading bits of x), equal bit for bit to that of the same value as
+// float64.
 template <int KIND>
 __device__ __forceinline__ void split_store_f32(void* dst, int64_t off_hi, int64_t Kp, float x) {
   if (KIND == TC_BF16) {
@@ -77,47 +57,64 @@ __device__ __forceinline__ void split_store2_f32(void* dst, int64_t off_hi, int6
   }
 }
 
-__device__ __forceinline__ double load_src(const void* src, bool f32, int64_t off) {
-  return f32 ? (double)reinterpret_cast<const float*>(src)[off]
-             : reinterpret_cast<const double*>(src)[off];
-}
-
-// K contiguous in the source: thread per (row, k), k fastest.
-template <int KIND>
-__global__ void k_split_direct(SplitView v, void* __restrict__ dst, int64_t Kp) {
-  const int64_t total = v.rows * Kp;
+// K contiguous in the source: a thread per eight columns of a row, read in
+// 16-byte loads where every row starts on such a boundary (vec).
+template <int KIND, typename S>
+__global__ void __launch_bounds__(256) k_split_direct(SplitView v, void* __restrict__ dst, int64_t Kp,
+                                                      FastDiv by_k8, FastDiv by_n1, int vec, int wide) {
+  const int64_t k8 = Kp / 8, total = v.rows * k8;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / Kp, k = e - r * Kp;
-    double x = 0.0;
-    if (k < v.K) {
-      const int64_t r0 = r / v.n1, r1 = r - r0 * v.n1;
-      x = load_src(v.src, v.src_f32, r0 * v.s0 + r1 * v.s1 + k * v.sk);
+    const int64_t r = wide ? e / k8 : (int64_t)by_k8((uint32_t)e), k = (e - r * k8) * 8;
+    const int64_t r0 = wide ? r / v.n1 : (int64_t)by_n1((uint32_t)r), r1 = r - r0 * v.n1;
+    const S* p = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1 + k * v.sk;
+    S x[8];
+    if (vec && k + 8 <= v.K) {
+      constexpr int PER = 16 / sizeof(S);
+#pragma unroll
+      for (int i = 0; i < 8; i += PER) {
+        const uint4 q = *reinterpret_cast<const uint4*>(p + i);
+        *reinterpret_cast<uint4*>(x + i) = q;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = k + i < v.K ? p[i * v.sk] : (S)0;
     }
-    split_store<KIND>(dst, r * 2 * Kp + k, Kp, x);
+    typename SplitWord<KIND>::T w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = split_word<KIND, S>(x[i]);
+    store_words(dst, r * 2 * Kp + k, Kp, w);
   }
 }
 
-// K strided in the source: 32x32 tiles transposed through shared memory.
-template <int KIND>
-__global__ void k_split_transpose(SplitView v, void* __restrict__ dst, int64_t Kp) {
-  __shared__ double tile[32][33];
-  const int64_t r_base = (int64_t)blockIdx.x * 32;
-  const int64_t k_base = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t k = k_base + j, r = r_base + tx;  // rows fastest while reading
-    double x = 0.0;
-    if (k < v.K && r < v.rows) {
-      const int64_t r0 = r / v.n1, r1 = r - r0 * v.n1;
-      x = load_src(v.src, v.src_f32, r0 * v.s0 + r1 * v.s1 + k * v.sk);
-    }
-    tile[j][tx] = x;
+// K strided in the source, rows close together: tiles of 64 rows x 64 columns,
+// read along the rows (512 bytes a time, sixteen loads in flight per thread),
+// split, and written along the columns through shared memory.
+template <int KIND, typename S>
+__global__ void __launch_bounds__(256) k_split_transpose(SplitView v, void* __restrict__ dst, int64_t Kp) {
+  using W = typename SplitWord<KIND>::T;
+  __shared__ W tile[64][65];
+  const int64_t r_base = (int64_t)blockIdx.x * 64, k_base = (int64_t)blockIdx.y * 64;
+  {
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int64_t r = r_base + tx, rr = r < v.rows ? r : 0;
+    const int64_t r0 = rr / v.n1, r1 = rr - r0 * v.n1;
+    const S* p = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1 + (k_base + ty) * v.sk;
+    S x[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      x[j] = (r < v.rows && k_base + ty + 4 * j < v.K) ? p[4 * j * v.sk] : (S)0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tile[ty + 4 * j][tx] = split_word<KIND, S>(x[j]);
   }
   __syncthreads();
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t r = r_base + j, k = k_base + tx;  // k fastest while writing
-    if (r < v.rows && k < Kp) split_store<KIND>(dst, r * 2 * Kp + k, Kp, tile[tx][j]);
+  for (int u = threadIdx.x; u < 512; u += 256) {
+    const int row = u >> 3, g = 8 * (u & 7);
+    if (r_base + row >= v.rows) continue;
+    W w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = tile[g + i][row];
+    store_words(dst, (r_base + row) * 2 * Kp + k_base + g, Kp, w);
   }
 }
 
@@ -127,20 +124,6 @@ int grid_for(int64_t n, int threads) {
   if (b > 65536) b = 65536;
   return (int)b;
 }
-
-// n / d for 0 <= n < 2^31 by a multiplication and a shift (Granlund and
-// Montgomery, PLDI 1994): a 64-bit division costs more than a whole fiber.
-struct FastDiv {
-  uint32_t d = 1, m = 0, s = 0;
-  FastDiv() = default;
-  explicit FastDiv(uint32_t div) : d(div) {
-    while (s < 32 && (1ull << s) < div) ++s;
-    m = (uint32_t)((((1ull << s) - div) << 32) / div + 1);
-  }
-  __device__ __forceinline__ uint32_t operator()(uint32_t n) const {
-    return (uint32_t)(((uint64_t)__umulhi(m, n) + n) >> s);
-  }
-};
 
 // One nonzero entry of a W-step matrix: value, input index, and whether the
 // value is 1 (a comparison of float64 values runs on the float64 pipe).
@@ -772,22 +755,38 @@ bool try_fused(int64_t d, int64_t wl, int64_t wm, int64_t wr, int kind, const fl
 
 }  // namespace
 
+template <int KIND, typename S>
+static osmps_status split_operand_as(const SplitView& v, void* dst, int64_t Kp, cudaStream_t s) {
+  if (v.sk == 1 || v.K == 1) {
+    const int64_t units = v.rows * (Kp / 8);
+    const bool wide = units > 2147483647ll || v.n1 > 2147483647ll;
+    constexpr int64_t PER = 16 / sizeof(S);
+    const bool vec = v.sk == 1 && (reinterpret_cast<uintptr_t>(v.src) & 15) == 0 && v.s0 % PER == 0 &&
+                     (v.n1 == 1 || v.s1 % PER == 0);
+    const FastDiv by_k8(wide ? 1 : (uint32_t)(Kp / 8)), by_n1(wide ? 1 : (uint32_t)v.n1);
+    k_split_direct<KIND, S><<<grid_for(units, 256), 256, 0, s>>>(v, dst, Kp, by_k8, by_n1, vec ? 1 : 0,
+                                                                wide ? 1 : 0);
+  } else {
+    if (cdiv(Kp, 64) > 65535) return set_error(OSMPS_ESHAPE, "split_operand: K too large");
+    const dim3 grid((unsigned)cdiv(v.rows, 64), (unsigned)cdiv(Kp, 64));
+    k_split_transpose<KIND, S><<<grid, 256, 0, s>>>(v, dst, Kp);
+  }
+  note_launch();
+  OSMPS_LAUNCH_CHECK();
+  return OSMPS_OK;
+}
+
+// Traffic: 8 (4) bytes read and 4 (8) written per value. chi = 1024, bf16: L
+// (5120 rows of 1024) 41 us and theta transposed (4096 x 1024) 35 us before
+// the integer split and the wide accesses.
 osmps_status split_operand(const SplitView& v, int kind, void* dst, int64_t Kp, cudaStream_t s) {
   if (v.rows <= 0) return OSMPS_OK;
   if (Kp < v.K || Kp % 64 != 0) return set_error(OSMPS_ESHAPE, "split_operand: bad Kp");
-  if (v.sk == 1 || v.K == 1) {
-    const int blocks = grid_for(v.rows * Kp, 256);
-    if (kind == TC_BF16) { k_split_direct<TC_BF16><<<blocks, 256, 0, s>>>(v, dst, Kp); note_launch(); }
-    else { k_split_direct<TC_TF32><<<blocks, 256, 0, s>>>(v, dst, Kp); note_launch(); }
-  } else {
-    if (cdiv(Kp, 32) > 65535) return set_error(OSMPS_ESHAPE, "split_operand: K too large");
-    dim3 grid((unsigned)cdiv(v.rows, 32), (unsigned)cdiv(Kp, 32));
-    dim3 block(32, 8);
-    if (kind == TC_BF16) { k_split_transpose<TC_BF16><<<grid, block, 0, s>>>(v, dst, Kp); note_launch(); }
-    else { k_split_transpose<TC_TF32><<<grid, block, 0, s>>>(v, dst, Kp); note_launch(); }
-  }
-  OSMPS_LAUNCH_CHECK();
-  return OSMPS_OK;
+  if (kind == TC_BF16)
+    return v.src_f32 ? split_operand_as<TC_BF16, float>(v, dst, Kp, s)
+                     : split_operand_as<TC_BF16, double>(v, dst, Kp, s);
+  return v.src_f32 ? split_operand_as<TC_TF32, float>(v, dst, Kp, s)
+                   : split_operand_as<TC_TF32, double>(v, dst, Kp, s);
 }
 
 osmps_status fiber_contract_f64(const Fiber& f, const double* Mat, const double* in, double* out,
@@ -889,6 +888,31 @@ osmps_status zero_pad_columns(void* dst, int kind, int64_t rows, int64_t Kcols, 
   const int blocks = grid_for(rows * (Kp - Kcols), 256);
   if (kind == TC_BF16) { k_zero_pad<TC_BF16><<<blocks, 256, 0, s>>>(dst, rows, Kcols, Kp); note_launch(); }
   else { k_zero_pad<TC_TF32><<<blocks, 256, 0, s>>>(dst, rows, Kcols, Kp); note_launch(); }
+  OSMPS_LAUNCH_CHECK();
+  return OSMPS_OK;
+}
+
+// H_eff's two site tensors in one launch, one block row each.
+__global__ void k_w_reorder_pair(const double* __restrict__ W1, const double* __restrict__ W2,
+                                 int64_t wl, int64_t d1, int64_t wm, int64_t d2, int64_t wr,
+                                 double* __restrict__ M1, double* __restrict__ M2) {
+  const bool second = blockIdx.y == 1;
+  const double* W = second ? W2 : W1;
+  double* Mat = second ? M2 : M1;
+  const int64_t dw = second ? wm : wl, d = second ? d2 : d1, dw2 = second ? wr : wm;
+  const int64_t total = dw * d * d * dw2;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t w2 = e % dw2, r = e / dw2, s = r % d, q = r / d, t = q % d, w = q / d;
+    Mat[(w * d + s) * (d * dw2) + t * dw2 + w2] = W[e];
+  }
+}
+
+osmps_status w_reorder_pair(const double* W1, const double* W2, int64_t wl, int64_t d1, int64_t wm,
+                            int64_t d2, int64_t wr, double* M1, double* M2, cudaStream_t s) {
+  const int64_t most = std::max(wl * d1 * d1 * wm, wm * d2 * d2 * wr);
+  k_w_reorder_pair<<<dim3(std::min(grid_for(most, 256), 1024), 2), 256, 0, s>>>(W1, W2, wl, d1, wm, d2, wr, M1, M2);
+  note_launch();
   OSMPS_LAUNCH_CHECK();
   return OSMPS_OK;
 }

@@ -68,7 +68,7 @@ __global__ void k_selftest_bf16(const double* __restrict__ x, uint16_t* __restri
                                 uint16_t* __restrict__ y_hw, int64_t n) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    y_int[i] = __bfloat16_as_ushort(f64_to_bf16_rn(x[i]));
+    y_int[i] = (unsigned short)(f64_to_bf16_pair(x[i]) & 0xFFFFu);
     y_hw[i] = __bfloat16_as_ushort(__double2bfloat16(x[i]));
   }
 }

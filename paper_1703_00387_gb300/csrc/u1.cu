@@ -27,7 +27,7 @@
 #include <atomic>
 
 #include "common.cuh"
-#include "ieee.cuh"
+#include "operand.cuh"
 
 struct osmps_u1_heff {
   osmps_ctx* ctx = nullptr;
@@ -90,62 +90,57 @@ __device__ __forceinline__ void store_split_f(void* dst, int64_t off_hi, int64_t
   }
 }
 
-// Split of a float64 value: hi = round(x), lo = round(x - hi) in the operand
-// type. The roundings and the widening of hi use the integer fields
-// (ieee.cuh); only the exact subtraction x - hi runs on GB300's narrow
-// float64 pipe. Bit for bit the split of the hardware conversions.
-template <int KIND>
-__device__ __forceinline__ void store_split_d(void* dst, int64_t off_hi, int64_t Kpl, double x) {
-  if (KIND == TC_BF16) {
-    const __nv_bfloat16 h = f64_to_bf16_rn(x);
-    const __nv_bfloat16 l = f64_to_bf16_rn(x - f32_to_f64(__bfloat162float(h)));
-    reinterpret_cast<__nv_bfloat16*>(dst)[off_hi] = h;
-    reinterpret_cast<__nv_bfloat16*>(dst)[off_hi + Kpl] = l;
-  } else {
-    uint32_t h, l;
-    const float xf = f64_to_f32_rn(x);
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(xf));
-    const float r = f64_to_f32_rn(x - f32_to_f64(__uint_as_float(h)));
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(l) : "f"(r));
-    reinterpret_cast<uint32_t*>(dst)[off_hi] = h;
-    reinterpret_cast<uint32_t*>(dst)[off_hi + Kpl] = l;
-  }
-}
-
-// Operand row r = src[row_src[r] + k] for k < row_len[r], zero up to Kpl.
+// Operand row r = src[row_src[r] + k] for k < row_len[r], zero up to Kpl; a
+// thread per eight columns.
 template <int KIND>
 __global__ void k_row_gather_split(const double* __restrict__ src, const int64_t* __restrict__ row_src,
                                    const int64_t* __restrict__ row_len, int64_t rows, int64_t Kpl,
                                    void* __restrict__ dst) {
-  const int64_t total = rows * Kpl;
+  const int64_t k8 = Kpl / 8, total = rows * k8;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / Kpl, k = e - r * Kpl;
-    const double x = k < row_len[r] ? src[row_src[r] + k] : 0.0;
-    store_split_d<KIND>(dst, r * 2 * Kpl + k, Kpl, x);
+    const int64_t r = e / k8, k = (e - r * k8) * 8, n = row_len[r];
+    const double* p = src + row_src[r] + k;
+    double x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = k + i < n ? p[i] : 0.0;
+    typename SplitWord<KIND>::T w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = split_word<KIND, double>(x[i]);
+    store_words(dst, r * 2 * Kpl + k, Kpl, w);
   }
 }
 
 // theta^T blocks: operand row r, column k = theta[base[r] + k * stride[r]] for
-// k < len[r], zero up to Kpl; 32 x 32 tiles through shared memory (reads
-// along r, which is contiguous in theta, writes along k).
+// k < len[r], zero up to Kpl; 64 x 64 tiles through shared memory (reads
+// along r, which is contiguous in theta, writes along k), as k_split_transpose.
 template <int KIND>
-__global__ void k_theta_split(const double* __restrict__ th, const int64_t* __restrict__ base,
-                              const int64_t* __restrict__ stride, const int64_t* __restrict__ len,
-                              int64_t rows, int64_t Kpl, void* __restrict__ dst) {
-  __shared__ double tile[32][33];
-  const int64_t r0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t r = r0 + tx, k = k0 + j;
-    double x = 0.0;
-    if (r < rows && k < len[r]) x = th[base[r] + k * stride[r]];
-    tile[j][tx] = x;
+__global__ void __launch_bounds__(256)
+    k_theta_split(const double* __restrict__ th, const int64_t* __restrict__ base,
+                  const int64_t* __restrict__ stride, const int64_t* __restrict__ len, int64_t rows,
+                  int64_t Kpl, void* __restrict__ dst) {
+  using W = typename SplitWord<KIND>::T;
+  __shared__ W tile[64][65];
+  const int64_t r_base = (int64_t)blockIdx.x * 64, k_base = (int64_t)blockIdx.y * 64;
+  {
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int64_t r = r_base + tx, k0 = k_base + ty;
+    const int64_t n = r < rows ? len[r] : 0, st = r < rows ? stride[r] : 0;
+    const double* p = th + (r < rows ? base[r] + k0 * st : 0);
+    double x[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) x[j] = k0 + 4 * j < n ? p[4 * j * st] : 0.0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) tile[ty + 4 * j][tx] = split_word<KIND, double>(x[j]);
   }
   __syncthreads();
-  for (int j = ty; j < 32; j += 8) {
-    const int64_t r = r0 + j, k = k0 + tx;
-    if (r < rows && k < Kpl) store_split_d<KIND>(dst, r * 2 * Kpl + k, Kpl, tile[tx][j]);
+  for (int u = threadIdx.x; u < 512; u += 256) {
+    const int row = u >> 3, g = 8 * (u & 7);
+    if (r_base + row >= rows) continue;
+    W w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = tile[g + i][row];
+    store_words(dst, (r_base + row) * 2 * Kpl + k_base + g, Kpl, w);
   }
 }
 
@@ -601,12 +596,12 @@ osmps_status u1_prepare_kind(osmps_u1_heff* h, const double* L, const double* W1
   }
   // L and R as split operands, combined W coefficients
   if (h->rowsA1 > 0) {
-    k_row_gather_split<KIND><<<ew_grid(h->rowsA1 * h->Kpl1), 256, 0, s>>>(
+    k_row_gather_split<KIND><<<ew_grid(h->rowsA1 * (h->Kpl1 / 8)), 256, 0, s>>>(
         L, T + h->t_a1src, T + h->t_a1len, h->rowsA1, h->Kpl1, B + h->o_A1);
     note_launch();
   }
   if (h->rowsB4 > 0) {
-    k_row_gather_split<KIND><<<ew_grid(h->rowsB4 * h->Kpl4), 256, 0, s>>>(
+    k_row_gather_split<KIND><<<ew_grid(h->rowsB4 * (h->Kpl4 / 8)), 256, 0, s>>>(
         R, T + h->t_b4src, T + h->t_b4len, h->rowsB4, h->Kpl4, B + h->o_B4);
     note_launch();
   }
@@ -670,8 +665,8 @@ osmps_status u1_apply_kind(osmps_ctx* ctx, osmps_u1_heff* h, const double* theta
   uint8_t* B = h->d_buf;
   // stage 1
   if (h->rowsB1 > 0) {
-    dim3 grid((unsigned)cdiv(h->rowsB1, 32), (unsigned)cdiv(h->Kpl1, 32));
-    k_theta_split<KIND><<<grid, dim3(32, 8), 0, s>>>(theta, T + h->t_b1base, T + h->t_b1stride,
+    dim3 grid((unsigned)cdiv(h->rowsB1, 64), (unsigned)(h->Kpl1 / 64));
+    k_theta_split<KIND><<<grid, 256, 0, s>>>(theta, T + h->t_b1base, T + h->t_b1stride,
                                                      T + h->t_b1len, h->rowsB1, h->Kpl1, B + h->o_B1);
     note_launch();
   }
