@@ -156,6 +156,9 @@ struct osmps_ctx {
   // stream used only to record CUDA graphs (created on first use), and a flag
   // that makes workspace growth an error while a capture is open
   cudaStream_t capture_stream = nullptr;
+  // stream and events for work beside the caller's stream (created on first use)
+  cudaStream_t side_stream = nullptr;
+  cudaEvent_t side_ev[2] = {nullptr, nullptr};
   bool capturing = false;
   // tcgen05 GEMM tile widths chosen by measurement (OSMPS_AUTOTUNE_ON) per
   // size class: key, chosen width, microseconds at widths 256 / 128 / 64

@@ -327,6 +327,9 @@ osmps_status osmps_ctx_destroy(osmps_ctx* ctx) {
     if (gr.g) cudaGraphDestroy(gr.g);
   }
   if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
+  if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
+  for (cudaEvent_t e : ctx->side_ev)
+    if (e) cudaEventDestroy(e);
   delete ctx;
   return OSMPS_OK;
 }

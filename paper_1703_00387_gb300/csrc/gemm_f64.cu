@@ -11,10 +11,12 @@
 // over the sub-partitions of all SMs, never by its loads (8 to 16 bytes of
 // operand per 128 clocks of DMMA at the tiles below). Hence small tiles for
 // every size: a CTA is four warps, one per sub-partition, on one 16x16 or 8x8
-// tile of C; the warps share the K range (K group of four number g goes to
-// warp g mod 4) and their partial tiles are added in warp order. Fragments
-// are read straight from global memory (eight rows x 32 bytes or four rows x
-// 64 bytes per load), a round of groups ahead of the DMMAs.
+// tile of C. With tiles enough for four CTAs per SM each warp has an 8x8 part
+// of the tile and all of K, in order; with fewer, the warps share the K range
+// (K group of four number g goes to warp g mod 4) and their partial tiles are
+// added in warp order. Fragments are read straight from global memory (eight
+// rows x 32 bytes or four rows x 64 bytes per load), a round of groups ahead
+// of the DMMAs.
 // Measured against 64x64 tiles staged through shared memory (M x N x K, us):
 // 128x32x96 119 -> 6.3, 64x64x64 82 -> 4.2, 300x340x300 367 -> 74,
 // 512x512x512 615 -> 274, 1024x1024x1024 2445 -> 2074 (1.04 TFLOP/s),
@@ -44,14 +46,18 @@ __device__ __forceinline__ void dmma(double& c0, double& c1, double a, double b)
                : "d"(a), "d"(b));
 }
 
-template <int FM, int FN>
+// FM x FN: 8x8 fragments per warp. SPLIT: all four warps on the CTA's one
+// 8 FM x 8 FN tile, sharing K; else 2 x 2 warps on a tile of twice that edge.
+template <int FM, int FN, bool SPLIT>
 __global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
   constexpr int KU = FM * FN > 1 ? 2 : 4;  // K groups in flight per warp
-  constexpr int TM = 8 * FM, TN = 8 * FN;
-  __shared__ double red[4][TM][TN];
+  constexpr int TM = 8 * FM, TN = 8 * FN, W = SPLIT ? 1 : 2;
+  constexpr int KSTEP = SPLIT ? 16 : 4;    // between a warp's K groups
+  __shared__ double red[SPLIT ? 4 : 1][SPLIT ? TM : 1][SPLIT ? TN : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, tq = lane & 3;
-  const int64_t m0 = (int64_t)(blockIdx.x / tiles_n) * TM, n0 = (int64_t)(blockIdx.x % tiles_n) * TN;
+  const int64_t m0 = (int64_t)(blockIdx.x / tiles_n) * (W * TM) + (SPLIT ? 0 : (warp >> 1) * TM);
+  const int64_t n0 = (int64_t)(blockIdx.x % tiles_n) * (W * TN) + (SPLIT ? 0 : (warp & 1) * TN);
   const double* A = p.A + (int64_t)blockIdx.y * p.sab;
   const double* B = p.B + (int64_t)blockIdx.y * p.sbb;
   // this lane's rows / columns, those past the edge read as zero
@@ -71,10 +77,10 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
     bp[j] = B + (bm[j] ? n : 0) * p.sbn;
   }
   double a[KU][FM], b[KU][FN];
-  auto load = [&](int64_t k) {  // the warp's KU groups from K index k on, 16 apart
+  auto load = [&](int64_t k) {  // the warp's KU groups from K index k on, KSTEP apart
 #pragma unroll
     for (int u = 0; u < KU; ++u) {
-      const int64_t kk = k + 16 * u + tq;
+      const int64_t kk = k + KSTEP * u + tq;
       const bool in = kk < p.K;
 #pragma unroll
       for (int i = 0; i < FM; ++i) a[u][i] = in && am[i] ? ap[i][kk * p.sak] : 0.0;
@@ -87,9 +93,9 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
   for (int i = 0; i < FM; ++i)
 #pragma unroll
     for (int j = 0; j < FN; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
-  int64_t k = 4 * warp;
+  int64_t k = SPLIT ? 4 * warp : 0;
   load(k);
-  for (; k < p.K; k += 16 * KU) {
+  for (; k < p.K; k += KSTEP * KU) {
     double ca[KU][FM], cb[KU][FN];
 #pragma unroll
     for (int u = 0; u < KU; ++u) {
@@ -98,34 +104,44 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
 #pragma unroll
       for (int j = 0; j < FN; ++j) cb[u][j] = b[u][j];
     }
-    load(k + 16 * KU);  // past the end: all zero, nothing is read
+    load(k + KSTEP * KU);  // past the end: all zero, nothing is read
 #pragma unroll
     for (int u = 0; u < KU; ++u)
-      if (k + 16 * u < p.K) {  // the same for the whole warp
+      if (k + KSTEP * u < p.K) {  // the same for the whole warp
 #pragma unroll
         for (int i = 0; i < FM; ++i)
 #pragma unroll
           for (int j = 0; j < FN; ++j) dmma(acc[i][j][0], acc[i][j][1], ca[u][i], cb[u][j]);
       }
   }
-#pragma unroll
-  for (int i = 0; i < FM; ++i)
-#pragma unroll
-    for (int j = 0; j < FN; ++j) {
-      red[warp][8 * i + g][8 * j + 2 * tq] = acc[i][j][0];
-      red[warp][8 * i + g][8 * j + 2 * tq + 1] = acc[i][j][1];
-    }
-  __syncthreads();
   double* C = p.C + (int64_t)blockIdx.y * p.scb;
-  for (int e = threadIdx.x; e < TM * TN; e += 128) {
-    const int r = e / TN, c = e % TN;
-    const int64_t gm = m0 + r, gn = n0 + c;
+  const auto put = [&](int64_t gm, int64_t gn, double sum) {
     if (gm < p.M && gn < p.N) {
       double* dst = C + gm * p.scm + gn * p.scn;
-      double v = p.alpha * (((red[0][r][c] + red[1][r][c]) + red[2][r][c]) + red[3][r][c]);
+      double v = p.alpha * sum;
       if (p.beta != 0.0) v = fma(p.beta, *dst, v);
       *dst = v;
     }
+  };
+  if constexpr (SPLIT) {
+#pragma unroll
+    for (int i = 0; i < FM; ++i)
+#pragma unroll
+      for (int j = 0; j < FN; ++j)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) red[warp][8 * i + g][8 * j + 2 * tq + r] = acc[i][j][r];
+    __syncthreads();
+    for (int e = threadIdx.x; e < TM * TN; e += 128) {
+      const int r = e / TN, c = e % TN;
+      put(m0 + r, n0 + c, ((red[0][r][c] + red[1][r][c]) + red[2][r][c]) + red[3][r][c]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < FM; ++i)
+#pragma unroll
+      for (int j = 0; j < FN; ++j)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) put(m0 + 8 * i + g, n0 + 8 * j + 2 * tq + r, acc[i][j][r]);
   }
 }
 
@@ -166,8 +182,9 @@ osmps_status gemm_f64(const GemmF64& g, cudaStream_t stream) {
          g.C, g.scm, g.scn, g.scb, g.alpha, g.beta};
   const dim3 grid((unsigned)tiles, (unsigned)g.batch);
   const int ph = prof_begin(stream);
-  if (t == 16) k_gemm_f64<2, 2><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
-  else k_gemm_f64<1, 1><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
+  if (t == 16 && tiles * g.batch >= 4 * F64_SMS) k_gemm_f64<1, 1, false><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
+  else if (t == 16) k_gemm_f64<2, 2, true><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
+  else k_gemm_f64<1, 1, true><<<grid, 128, 0, stream>>>(a, (int)tiles_n);
   note_launch();
   OSMPS_LAUNCH_CHECK();
   const double f = 2.0 * (double)g.M * (double)g.N * (double)g.K * (double)g.batch;

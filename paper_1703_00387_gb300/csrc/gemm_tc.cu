@@ -73,8 +73,10 @@ __device__ __forceinline__ void store_tile_rows(void* C, int64_t row0, int64_t c
                                                 int64_t N, int64_t ldc, const float (&acc)[EPI_COLS],
                                                 float* __restrict__ stg, int lane,
                                                 const float* __restrict__ addend) {
+  if (row0 >= M) return;  // nothing of this warp's rows or columns is inside
 #pragma unroll
   for (int pass = 0; pass < EPI_COLS / STG_COLS; ++pass) {
+    if (col0 + STG_COLS * pass >= N) return;
 #pragma unroll
     for (int v = 0; v < STG_COLS / 4; ++v) {
       const int g = v ^ (lane & 3);

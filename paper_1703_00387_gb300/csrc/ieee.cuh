@@ -20,13 +20,10 @@ namespace osmps {
 
 // (double)x, exactly.
 __device__ __forceinline__ double f32_to_f64(float x) {
-  const uint32_t u = __float_as_uint(x);
-  if ((u << 1) == 0) return __longlong_as_double((long long)((uint64_t)(u >> 31) << 63));  // +-0
-  const uint32_t e = (u >> 23) & 0xFFu;
-  if (e == 0u || e == 0xFFu) return (double)x;  // zero, subnormal, inf, nan
-  const uint64_t bits = ((uint64_t)(u >> 31) << 63) | ((uint64_t)(e + 896u) << 52) |
-                        ((uint64_t)(u & 0x7FFFFFu) << 29);
-  return __longlong_as_double((long long)bits);
+  const uint32_t u = __float_as_uint(x), mag = u & 0x7FFFFFFFu;
+  if (mag - 0x00800000u >= 0x7F000000u && mag != 0u) return (double)x;  // subnormal, inf, nan
+  const uint32_t hi = mag == 0u ? 0u : (mag >> 3) + 0x38000000u;  // exponent + 896
+  return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
 }
 
 // (float)x, rounded to nearest with ties to even.

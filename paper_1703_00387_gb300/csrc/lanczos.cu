@@ -3,9 +3,9 @@
 //
 // Krylov vectors, orthogonalisation and the tridiagonal eigensolve are all
 // float64 on the device. Each step applies H_eff (any precision), projects
-// the result against every stored Krylov vector twice (classical
-// Gram-Schmidt, two passes: full reorthogonalisation), normalises, and
-// solves the small tridiagonal problem for the lowest Ritz pair:
+// the result against every stored Krylov vector (full reorthogonalisation,
+// see `orthogonalise`), normalises, and solves the small tridiagonal problem
+// for the lowest Ritz pair:
 //   * the eigenvalue by Sturm-count multisection (128 points per round),
 //   * its eigenvector from the twisted factorisation of T - e I.
 // The stopping test (residual estimate beta_j |s_j| <= tol, the iteration
@@ -43,12 +43,17 @@ constexpr int MAX_PROJ = 64;
 constexpr int OFF_URE = 5 * MAXIT + 16 + 2 * MAX_PROJ;  // exp(-i tau T) e_1 (Krylov propagator)
 constexpr int OFF_UIM = OFF_URE + MAXIT;
 constexpr int SCAL_COUNT = OFF_UIM + MAXIT;
+// the partial-sum buffer: a row of DOT_MAX_BLOCKS per Krylov vector, then one
+// for the partial squared norms of the orthogonalised w
+constexpr int ROW_NORM = MAXIT;
+constexpr size_t PART_BYTES = (size_t)(MAXIT + 1) * DOT_MAX_BLOCKS * 8;
 constexpr int MISC_READ = 10;  // doubles of OFF_MISC the host reads (the state included)
 
 // Iteration state (ints at OFF_STATE): the index J of the Krylov vector the
-// next step applies H_eff to, the stop code, and the number of Krylov vectors
-// the Ritz vector combines.
-constexpr int ST_J = 0, ST_STOP = 1, ST_M = 2;
+// next step applies H_eff to, the stop code, the number of Krylov vectors the
+// Ritz vector combines, and the index of the next T to be solved (the
+// tridiagonal solve can run beside the following step, so it counts apart).
+constexpr int ST_J = 0, ST_STOP = 1, ST_M = 2, ST_T = 3;
 constexpr int STOP_NONE = 0, STOP_CONVERGED = 1, STOP_CAP = 2, STOP_NONFINITE = 3;
 
 __host__ __device__ inline int* lz_state(double* sc) { return reinterpret_cast<int*>(sc + OFF_STATE); }
@@ -63,6 +68,38 @@ inline const int* lz_state_in_misc(const double* misc) {
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// out[v] = sum over the warp of acc[v], v < G <= 8. From three values on by a
+// butterfly that halves the live values at each of the first three steps: nine
+// additions for eight sums instead of forty (the float64 pipe is the limit).
+template <int G>
+__device__ __forceinline__ void warp_sums(const double (&acc)[G], double* out) {
+  const int lane = threadIdx.x & 31;
+  if (G <= 2) {
+#pragma unroll
+    for (int v = 0; v < G; ++v) {
+      const double t = warp_sum(acc[v]);
+      if (lane == 0) out[v] = t;
+    }
+    return;
+  }
+  constexpr unsigned ALL = 0xffffffffu;
+  double a[8], h4[4], h2[2], h1;
+#pragma unroll
+  for (int v = 0; v < 8; ++v) a[v] = v < G ? acc[v < G ? v : 0] : 0.0;
+  const bool u16 = lane & 16, u8 = lane & 8, u4 = lane & 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    h4[i] = (u16 ? a[i + 4] : a[i]) + __shfl_xor_sync(ALL, u16 ? a[i] : a[i + 4], 16);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    h2[i] = (u8 ? h4[i + 2] : h4[i]) + __shfl_xor_sync(ALL, u8 ? h4[i] : h4[i + 2], 8);
+  h1 = (u4 ? h2[1] : h2[0]) + __shfl_xor_sync(ALL, u4 ? h2[0] : h2[1], 4);
+  h1 += __shfl_xor_sync(ALL, h1, 2);
+  h1 += __shfl_xor_sync(ALL, h1, 1);
+  const int v = (u16 ? 4 : 0) + (u8 ? 2 : 0) + (u4 ? 1 : 0);
+  if ((lane & 3) == 0 && v < G) out[v] = h1;
 }
 
 // Block-partial dot products of G consecutive Krylov vectors with w:
@@ -97,18 +134,13 @@ __device__ __forceinline__ void multidot_group(const double* __restrict__ V, int
 #pragma unroll
     for (int v = 0; v < G; ++v) acc[v] = fma(V[(int64_t)(g0 + v) * ld + n - 1], w[n - 1], acc[v]);
   }
-#pragma unroll
-  for (int v = 0; v < G; ++v) {
-    const double t = warp_sum(acc[v]);
-    if (lane == 0) sh[warp][v] = t;
-  }
+  warp_sums<G>(acc, sh[warp]);
   __syncthreads();
   if (threadIdx.x < G) {
     double t = 0.0;
     for (int k = 0; k < DOT_THREADS / 32; ++k) t += sh[k][threadIdx.x];
     part[(int64_t)(g0 + threadIdx.x) * nb + blockIdx.x] = t;
   }
-  __syncthreads();
 }
 
 // part[i * nb + b] = sum over block b's elements of V[i][e] * w[e], i < nv:
@@ -241,8 +273,7 @@ __global__ void k_combine_scalar(const double* __restrict__ V, int64_t ld,
   }
 }
 
-// Step j = state J: record alpha_j, beta_j, then the lowest eigenpair of
-// T_{j+1}; one block of four warps (one per SM sub-partition: the float64
+// The lowest eigenpair of T_{j+1}, j = state ST_T; one block of four warps (one per SM sub-partition: the float64
 // pipe of a sub-partition is the limit for a single warp).
 //   * Eigenvalue: multisection, 128 points per round (one per thread),
 //     from the Gershgorin interval: first on float32 Sturm counts of T/||T||
@@ -256,10 +287,7 @@ __global__ void k_combine_scalar(const double* __restrict__ V, int64_t ld,
 //     parallel.
 // Then the stopping decision: a non-finite Ritz value or residual; converged
 // (residual estimate <= tol, beta = 0, or the Krylov space is the whole
-// space); the step cap. Without a stop, J advances. With set_cond, the
-// decision is also the loop condition of the CUDA graph this kernel runs in
-// (1 = run another step), so a graph loop ends after at most max_iter steps:
-// J only advances below max_iter - 1.
+// space); the step cap. After a stop the kernel returns at once.
 constexpr int TRI_THREADS = 128;
 
 // The first thread index whose flag is set (TRI_THREADS if none), for every
@@ -276,31 +304,26 @@ __device__ __forceinline__ int first_set(bool flag, int* sh4) {
 }
 
 __global__ void __launch_bounds__(TRI_THREADS) k_tridiag(double* __restrict__ sc, int max_iter,
-                                                         double tol, long long n,
-                                                         cudaGraphConditionalHandle cond,
-                                                         int set_cond) {
-  __shared__ double a[MAXIT], b[MAXIT], b2[MAXIT], x[MAXIT], dd[MAXIT], du[MAXIT], ml[MAXIT],
-      rd[MAXIT];
+                                                         double tol, long long n) {
+  __shared__ double a[MAXIT], b[MAXIT], b2[MAXIT], x[MAXIT], uu[MAXIT], vv[MAXIT], rb[MAXIT];
+  __shared__ int ue[MAXIT], ve[MAXIT];
+  __shared__ double xs[TRI_THREADS], ps[TRI_THREADS];
+  __shared__ int pes[TRI_THREADS];
   __shared__ float af[MAXIT], b2f[MAXIT];
   __shared__ double red[2][TRI_THREADS / 32];
   __shared__ int sh4[TRI_THREADS / 32];
   int* st = lz_state(sc);
-  const int j = st[ST_J];
+  if (st[ST_STOP] != STOP_NONE) return;
+  const int j = st[ST_T];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (j < 0 || j >= max_iter || j >= MAXIT) {  // not reachable from the drivers below
     if (tid == 0) {
       st[ST_STOP] = STOP_NONFINITE;
       st[ST_M] = 1;
-      if (set_cond) cudaGraphSetConditional(cond, 0u);
     }
     return;
   }
   const int m = j + 1;
-  if (tid == 0) {
-    sc[OFF_ALPHA + j] = sc[OFF_C1 + j] + sc[OFF_C2 + j];
-    sc[OFF_BETA + j] = sqrt(sc[OFF_MISC + 3]);
-  }
-  __syncthreads();
   for (int i = tid; i < m; i += TRI_THREADS) {
     a[i] = sc[OFF_ALPHA + i];
     b[i] = sc[OFF_BETA + i];  // b[i] couples i and i+1 (b[j] is the residual norm)
@@ -356,78 +379,161 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag(double* __restrict__ sc
     lo = fmax(gl, lo - fpad);
     hi = fmin(gh, hi + fpad);
   }
-  bool check = true;  // this round includes the bracket's ends
+  // Rounds of 128 counts. The first spreads its points evenly over the bracket,
+  // ends included. Each round also keeps the minors p_m(x) = det(T - x I) at
+  // its points, and the next one puts its points around the zero e0 of the
+  // secant between the two that enclose the eigenvalue, at distances growing
+  // geometrically from the wanted width to the bracket's: the bracket then
+  // shrinks to about the secant's own error, quadratically small, whatever
+  // that is. (A round is 3 m float64 instructions per warp, 64 clocks each;
+  // narrowing by 129 a round took seven of them, this takes three or four.)
+  // Where a round narrows the bracket by less than 50, the next one spreads
+  // its points evenly again.
+  bool check = true, even = true;
+  double e0 = 0.0;
   for (int round = 0; round < 40; ++round) {
-    if (!check && !(hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)))) break;
-    double xt, step;
+    const double width = 4e-16 * fmax(fabs(lo), fabs(hi));
+    if (!check && !(hi - lo > width)) break;
+    double xt;
     if (check) {  // points lo, ..., hi (ends included)
-      step = (hi - lo) * (1.0 / (TRI_THREADS - 1));
-      xt = (tid == TRI_THREADS - 1) ? hi : lo + step * (double)tid;
+      xt = (tid == TRI_THREADS - 1) ? hi : lo + (hi - lo) * (1.0 / (TRI_THREADS - 1)) * (double)tid;
+    } else if (even) {
+      xt = lo + (hi - lo) * (1.0 / (TRI_THREADS + 1)) * (double)(tid + 1);
     } else {
-      step = (hi - lo) * (1.0 / (TRI_THREADS + 1));
-      xt = lo + step * (double)(tid + 1);
+      const bool up = tid >= TRI_THREADS / 2;
+      const int k = up ? tid - TRI_THREADS / 2 : TRI_THREADS / 2 - 1 - tid;  // 0 nearest e0
+      const double least = 0.25 * width;
+      const float span = log2f((float)((hi - lo) / least)) * (1.0f / (TRI_THREADS / 2 - 1));
+      const double off = least * (double)exp2f(span * (float)k);
+      xt = fmin(fmax(up ? e0 + off : e0 - off, lo), hi);
     }
-    const double xs[1] = {xt};
-    int c[1];
-    sturm_counts<1>(a, b2, m, xs, c);
-    const int t = first_set(c[0] >= 1, sh4);
-    if (check) {
+    double pv;
+    int pe;
+    const int c = sturm_count_minor(a, b2, m, xt, &pv, &pe);
+    xs[tid] = xt;
+    ps[tid] = pv;
+    pes[tid] = pe;
+    const int t = first_set(c >= 1, sh4);
+    if (check && (t == 0 || t == TRI_THREADS)) {  // the float32 bracket missed: the full interval
       check = false;
-      if (t == 0 || t == TRI_THREADS) {  // the float32 bracket missed: the full interval
-        lo = gl;
-        hi = gh;
-        continue;
-      }
-      const double nlo = lo + step * (double)(t - 1);
-      const double nhi = (t == TRI_THREADS - 1) ? hi : lo + step * (double)t;
-      lo = nlo;
-      hi = nhi;
-    } else {
-      const double nlo = lo + step * (double)t;
-      const double nhi = (t < TRI_THREADS) ? lo + step * (double)(t + 1) : hi;
-      lo = nlo;
-      hi = nhi;
+      lo = gl;
+      hi = gh;
+      continue;
     }
+    check = false;
+    const double was = hi - lo;
+    const double nlo = t > 0 ? xs[t - 1] : lo, nhi = t < TRI_THREADS ? xs[t] : hi;
+    even = true;
+    if (t > 0 && t < TRI_THREADS && (hi - lo) > 0.0) {
+      const double pl = fabs(ps[t - 1]), pr = fabs(ps[t]);
+      const double q = pr / pl;  // p_r / p_l = q 2^(pes[t] - pes[t - 1])
+      const int de = max(-1000, min(1000, pes[t] - pes[t - 1]));
+      const double frac = 1.0 / (1.0 + scalbn(q, de));
+      e0 = nlo + (nhi - nlo) * frac;
+      even = !(e0 > nlo && e0 < nhi) || (nhi - nlo) * 50.0 > was;
+    }
+    lo = nlo;
+    hi = nhi;
+    __syncthreads();  // xs, ps, pes are rewritten by the next round
   }
   const double e = 0.5 * (lo + hi);
-  // Eigenvector of T - e I by the twisted factorisation: the top-down pivots
-  // dp (T - e I = L D+ L^T, multipliers lq) and the bottom-up pivots dm
-  // (= U D- U^T, multipliers uq) on two warps at once; the twist index r
-  // minimises |gamma_k| = |dp_k + dm_k - (a_k - e)| (gamma_k^-1 is the k-th
-  // diagonal entry of (T - e I)^-1, largest where the eigenvector is); then
-  // z_r = 1, z_i = -lq_i z_(i+1) above r and z_(i+1) = -uq_i z_i below it, the
-  // two product chains again on two warps. A zero pivot becomes a tiny one of
-  // the same sign.
-  const double tiny = 1e-300 + 1e-18 * tn;
-  if (tid == 0) {
-    double d = a[0] - e;
-    for (int i = 0; i + 1 < m; ++i) {
-      if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
-      dd[i] = d;
-      const double l = b[i] / d;
-      ml[i] = l;
-      d = (a[i + 1] - e) - l * b[i];
+  // Eigenvector of T - e I, twisted: u_i from the top (u_0 = 1, row i of
+  // (T - e I) u = 0 gives u_(i+1)) and v_i from the bottom likewise, on two
+  // warps at once; the twist index r minimises |gamma_k|, gamma_k = (a_k - e) +
+  // b_(k-1) u_(k-1) / u_k + b_k v_(k+1) / v_k (its inverse is the k-th
+  // diagonal entry of (T - e I)^-1, largest where the eigenvector is), and z is
+  // u / u_r up to r and v / v_r from there. The chains multiply by
+  // reciprocals of the off-diagonals formed beforehand in parallel, two
+  // dependent operations a row (the pivot form of the same factorisation has
+  // a division, 628 clocks, on its chain); every four rows the running pair
+  // is scaled by a power of two, kept in ue / ve.
+  const double tiny = 1e-30 * tn;
+  bool splits = false;  // an off-diagonal so small that the chains could overflow
+  for (int i = tid; i + 1 < m; i += TRI_THREADS) {
+    rb[i] = 1.0 / b[i];
+    splits |= !(b[i] > tiny);
+  }
+  splits = __syncthreads_or(splits);
+  if (!splits) {
+    if (tid == 0) {
+      double um = 0.0, u = 1.0, bm = 0.0;
+      int ex = 0;
+      for (int i = 0; i < m; ++i) {
+        uu[i] = u;
+        ue[i] = ex;
+        if (i + 1 == m) break;
+        const double un = -(fma(a[i] - e, u, bm * um) * rb[i]);
+        um = u;
+        u = un;
+        bm = b[i];
+        if ((i & 3) == 3) {
+          const int ee = (int)((__double_as_longlong(fmax(fabs(u), fabs(um))) >> 52) & 0x7FF);
+          if (ee > 0 && ee < 2046) {
+            const double f = __longlong_as_double((long long)(2046 - ee) << 52);
+            u *= f;
+            um *= f;
+            // the stored predecessor keeps its own exponent
+            ex += ee - 1023;
+          }
+        }
+      }
+    } else if (tid == 32) {
+      double vp = 0.0, v = 1.0, bp = 0.0;
+      int ex = 0;
+      for (int i = m - 1; i >= 0; --i) {
+        vv[i] = v;
+        ve[i] = ex;
+        if (i == 0) break;
+        const double vn = -(fma(a[i] - e, v, bp * vp) * rb[i - 1]);
+        vp = v;
+        v = vn;
+        bp = b[i - 1];
+        if (((m - 1 - i) & 3) == 3) {
+          const int ee = (int)((__double_as_longlong(fmax(fabs(v), fabs(vp))) >> 52) & 0x7FF);
+          if (ee > 0 && ee < 2046) {
+            const double f = __longlong_as_double((long long)(2046 - ee) << 52);
+            v *= f;
+            vp *= f;
+            ex += ee - 1023;
+          }
+        }
+      }
     }
-    if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
-    dd[m - 1] = d;
-  } else if (tid == 32) {
-    double d = a[m - 1] - e;
-    for (int i = m - 2; i >= 0; --i) {
-      if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
-      du[i + 1] = d;
-      const double u = b[i] / d;
-      rd[i] = u;
-      d = (a[i] - e) - u * b[i];
+  } else {
+    // T all but splits: the pivots of T - e I = L D+ L^T and U D- U^T by
+    // division, a zero pivot made tiny, and u, v as the products of the
+    // multipliers' reciprocals would overflow, so as running ratios:
+    // ratio form u_k / u_(k+1) = -b_k / dp_k in uu, v_(k+1) / v_k = -b_k / dm_(k+1) in vv
+    const double zero = 1e-300 + 1e-18 * tn;
+    if (tid == 0) {
+      double d = a[0] - e;
+      for (int i = 0; i + 1 < m; ++i) {
+        if (fabs(d) < zero) d = d < 0.0 ? -zero : zero;
+        const double l = b[i] / d;
+        uu[i] = -l;
+        d = (a[i + 1] - e) - l * b[i];
+      }
+    } else if (tid == 32) {
+      double d = a[m - 1] - e;
+      for (int i = m - 2; i >= 0; --i) {
+        if (fabs(d) < zero) d = d < 0.0 ? -zero : zero;
+        const double u = b[i] / d;
+        vv[i] = -u;
+        d = (a[i] - e) - u * b[i];
+      }
     }
-    if (fabs(d) < tiny) d = d < 0.0 ? -tiny : tiny;
-    du[0] = d;
   }
   __syncthreads();
   // twist index: smallest |gamma|, ties to the smallest index
+  const auto ratio = [&](const double* y, const int* ye, int i, int k) {  // y_i / y_k
+    return scalbn(y[i] / y[k], max(-1000, min(1000, ye[i] - ye[k])));
+  };
   double gbest = 1e308;
   int rbest = 0;
   for (int k = tid; k < m; k += TRI_THREADS) {
-    const double g = fabs(dd[k] + du[k] - (a[k] - e));
+    const double up = k == 0 ? 0.0 : splits ? uu[k - 1] : ratio(uu, ue, k - 1, k);
+    const double dn = k + 1 == m ? 0.0 : splits ? vv[k] : ratio(vv, ve, k + 1, k);
+    const double g = fabs((a[k] - e) + (k > 0 ? b[k - 1] * up : 0.0) + (k + 1 < m ? b[k] * dn : 0.0));
     if (g < gbest) {
       gbest = g;
       rbest = k;
@@ -454,11 +560,13 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag(double* __restrict__ sc
       r = sh4[w];
     }
   __syncthreads();  // red / sh4 are reused below
-  if (tid == 0) {
+  if (!splits) {
+    for (int i = tid; i < m; i += TRI_THREADS) x[i] = i == r ? 1.0 : i < r ? ratio(uu, ue, i, r) : ratio(vv, ve, i, r);
+  } else if (tid == 0) {
     x[r] = 1.0;
-    for (int i = r - 1; i >= 0; --i) x[i] = -ml[i] * x[i + 1];
+    for (int i = r - 1; i >= 0; --i) x[i] = uu[i] * x[i + 1];
   } else if (tid == 32) {
-    for (int i = r; i + 1 < m; ++i) x[i + 1] = -rd[i] * (i == r ? 1.0 : x[i]);
+    for (int i = r; i + 1 < m; ++i) x[i + 1] = vv[i] * (i == r ? 1.0 : x[i]);
   }
   __syncthreads();
   // normalise (fixed-order block sum)
@@ -489,20 +597,24 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag(double* __restrict__ sc
     else if (m >= max_iter)
       stop = STOP_CAP;
     st[ST_M] = m;
+    st[ST_T] = j + 1;
     st[ST_STOP] = stop;
-    if (stop == STOP_NONE) st[ST_J] = j + 1;
-    if (set_cond) cudaGraphSetConditional(cond, stop == STOP_NONE ? 1u : 0u);
   }
 }
 
-// Next Krylov vector V[J] = w / beta_{J-1} after a step that did not stop
-// (the same arithmetic as vec_scale_by_inv), also into x when it is set: the
+// Next Krylov vector V[J] = w / beta_{J-1} (J already advanced) unless the
+// iteration has stopped or the basis is full, also into x when it is set: the
 // fixed input buffer of the matrix-vector product recorded in the step graph.
+// With set_cond, whether V[J] was formed is the loop condition of the graph
+// this kernel runs in, so the loop ends after at most max_iter steps.
 __global__ void k_next_vector(double* __restrict__ V, int64_t ld, const double* __restrict__ w,
-                              int64_t n, const double* __restrict__ sc, double* __restrict__ x) {
+                              int64_t n, const double* __restrict__ sc, double* __restrict__ x,
+                              int max_iter, cudaGraphConditionalHandle cond, int set_cond) {
   const int* st = lz_state(sc);
-  if (st[ST_STOP] != STOP_NONE) return;
   const int jn = st[ST_J];
+  const bool go = st[ST_STOP] == STOP_NONE && jn < max_iter;
+  if (set_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, go ? 1u : 0u);
+  if (!go) return;
   const double f = 1.0 / sc[OFF_BETA + jn - 1];
   double* y = V + (int64_t)jn * ld;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -515,15 +627,17 @@ __global__ void k_next_vector(double* __restrict__ V, int64_t ld, const double* 
 
 // First node of the step graph: enter the loop only if the step run before
 // the graph did not stop.
-__global__ void k_loop_init(const double* __restrict__ sc, cudaGraphConditionalHandle cond) {
-  cudaGraphSetConditional(cond, lz_state(sc)[ST_STOP] == STOP_NONE ? 1u : 0u);
+__global__ void k_loop_init(const double* __restrict__ sc, int max_iter, cudaGraphConditionalHandle cond) {
+  const int* st = lz_state(sc);
+  cudaGraphSetConditional(cond, st[ST_STOP] == STOP_NONE && st[ST_J] < max_iter ? 1u : 0u);
 }
 
-// Element chunks for k_multidot: about two element pairs per thread, and no
+// Element chunks for k_multidot: about two element pairs per thread (one for
+// short vectors, whose chunks would leave SMs idle), and no
 // more chunks than fit on the GPU in one wave (3 blocks per SM at its
 // register use); the vector groups multiply the blocks.
 int dot_blocks(int64_t n, int sm_count) {
-  int64_t b = cdiv(n, DOT_THREADS * 4);
+  int64_t b = cdiv(n, DOT_THREADS * (n <= ((int64_t)1 << 15) ? 2 : 4));
   const int64_t wave = 3 * (int64_t)(sm_count > 0 ? sm_count : 1);
   if (b > wave) b = wave;
   if (b > DOT_MAX_BLOCKS) b = DOT_MAX_BLOCKS;
@@ -554,6 +668,122 @@ __global__ void k_reorth_decide(const double* __restrict__ c, const double* __re
   if (threadIdx.x == 0) *flag = (isfinite(sq) && sq <= 0.5 * w2[0]) ? 1 : 0;
 }
 
+__device__ __forceinline__ double dot_block_sum(double v, double* sh) {
+  v = warp_sum(v);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  __syncthreads();
+  if (lane == 0) sh[warp] = v;
+  __syncthreads();
+  double t = 0.0;
+  for (int i = 0; i < warps; ++i) t += sh[i];
+  return t;
+}
+
+// One projection of a short w, w -= sum_i c_i V_i, with the partial squared
+// norms of the result. The coefficients are in c, or with nb > 0 still
+// block-partial in part (every block adds them up itself; block 0 stores them
+// in c). PAIR: two elements per
+// thread, the sums over i interleaved by four as in k_combine; the shortest
+// vectors take one element per thread, in 64-thread blocks, to reach more
+// SMs, and request their first vectors' values before the coefficients.
+template <bool PAIR>
+__global__ void __launch_bounds__(DOT_THREADS)
+    k_lz_update(const double* __restrict__ V, int64_t ld, double* __restrict__ w, int64_t n,
+                double* __restrict__ c, double* __restrict__ part, int nb,
+                const int* __restrict__ jcur) {
+  __shared__ double cs[MAXIT], sh[DOT_THREADS / 32];
+  const int nv = jcur[0] + 1, T = blockDim.x;
+  constexpr int AHEAD = 16;
+  const int64_t e1 = (int64_t)blockIdx.x * T + threadIdx.x;
+  double xq[PAIR ? 1 : AHEAD], w1 = 0.0;
+  if constexpr (!PAIR) {
+#pragma unroll
+    for (int q = 0; q < AHEAD; ++q) xq[q] = q < nv && e1 < n ? V[(int64_t)q * ld + e1] : 0.0;
+    if (e1 < n) w1 = w[e1];
+  }
+  if (nb == 0)
+    for (int i = threadIdx.x; i < nv; i += T) cs[i] = c[i];
+  // one lane per eight partial sums, all of a lane's loads in flight together
+  int lg = 0;
+  while (lg < 5 && (8 << lg) < nb) ++lg;
+  const int lanes = 1 << lg, sub = threadIdx.x & (lanes - 1);
+  for (int i0 = 0; nb > 0 && i0 < nv; i0 += T >> lg) {
+    const int i = i0 + (threadIdx.x >> lg);
+    double t = 0.0;
+    for (int b0 = sub; b0 < nb; b0 += 8 * lanes) {
+      double y[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) y[k] = i < nv && b0 + k * lanes < nb ? part[(int64_t)i * nb + b0 + k * lanes] : 0.0;
+      t += ((y[0] + y[1]) + (y[2] + y[3])) + ((y[4] + y[5]) + (y[6] + y[7]));
+    }
+    for (int o = lanes >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (i < nv && sub == 0) {
+      cs[i] = t;
+      if (blockIdx.x == 0) c[i] = t;
+    }
+  }
+  __syncthreads();
+  double nn = 0.0;
+  if constexpr (PAIR) {
+    for (int64_t e = e1; e < n >> 1; e += (int64_t)gridDim.x * T) {
+      double ax[4] = {0.0, 0.0, 0.0, 0.0}, ay[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int i = 0; i < nv; i += 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (i + q < nv) {
+            const double2 x = reinterpret_cast<const double2*>(V + (int64_t)(i + q) * ld)[e];
+            ax[q] = fma(cs[i + q], x.x, ax[q]);
+            ay[q] = fma(cs[i + q], x.y, ay[q]);
+          }
+      }
+      const double2 o = reinterpret_cast<const double2*>(w)[e];
+      const double2 r = make_double2(o.x - ((ax[0] + ax[1]) + (ax[2] + ax[3])),
+                                     o.y - ((ay[0] + ay[1]) + (ay[2] + ay[3])));
+      reinterpret_cast<double2*>(w)[e] = r;
+      nn = fma(r.x, r.x, fma(r.y, r.y, nn));
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+      double a = 0.0;
+      for (int i = 0; i < nv; ++i) a = fma(cs[i], V[(int64_t)i * ld + n - 1], a);
+      const double r = w[n - 1] - a;
+      w[n - 1] = r;
+      nn = fma(r, r, nn);
+    }
+  } else if (e1 < n) {  // (the grid covers n)
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int i = 0; i < nv; i += AHEAD) {
+      if (i > 0) {
+#pragma unroll
+        for (int q = 0; q < AHEAD; ++q) xq[q] = i + q < nv ? V[(int64_t)(i + q) * ld + e1] : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < AHEAD; ++q)
+        if (i + q < nv) a[q & 3] = fma(cs[i + q], xq[q], a[q & 3]);
+    }
+    const double r = w1 - ((a[0] + a[1]) + (a[2] + a[3]));
+    w[e1] = r;
+    nn = r * r;
+  }
+  nn = dot_block_sum(nn, sh);
+  if (threadIdx.x == 0) part[(int64_t)ROW_NORM * DOT_MAX_BLOCKS + blockIdx.x] = nn;
+}
+
+// alpha_J and beta_J = ||w||, from the nb block partials of ||w||^2 or, with
+// nb = 0, from its value at OFF_MISC + 3; J advances.
+__global__ void k_lz_norm(double* __restrict__ sc, const double* __restrict__ part, int nb) {
+  __shared__ double sh[DOT_THREADS / 32];
+  int* st = lz_state(sc);
+  const int j = st[ST_J];
+  double t = 0.0;
+  for (int b = threadIdx.x; b < nb; b += DOT_THREADS) t += part[(int64_t)ROW_NORM * DOT_MAX_BLOCKS + b];
+  t = dot_block_sum(t, sh);
+  if (threadIdx.x == 0) {
+    sc[OFF_ALPHA + j] = sc[OFF_C1 + j] + sc[OFF_C2 + j];
+    sc[OFF_BETA + j] = sqrt(nb > 0 ? t : sc[OFF_MISC + 3]);
+    st[ST_J] = j + 1;
+  }
+}
+
 int ew_blocks(int64_t n) {
   int64_t b = cdiv(n, 256 * 4);
   if (b < 1) b = 1;
@@ -577,6 +807,55 @@ osmps_status project(osmps_ctx* ctx, const double* V, int64_t ld, int64_t n, int
   } else {
     k_combine<1><<<ew_blocks(n), 256, 0, s>>>(V, ld, nv, coef, w, n, 0, jcur, skip);
   }
+  note_launch();
+  OSMPS_LAUNCH_CHECK();
+  return OSMPS_OK;
+}
+
+// One step's orthogonalisation of w (= H v_J, J from the device) against
+// V[0..J] by classical Gram-Schmidt, and its norm: alpha_J, beta_J and J + 1
+// in sc, the remainder in w. nv_max bounds J + 1.
+//
+// Up to 2^18 entries the launches cost more than the traffic: always two
+// passes, each a kernel of block-partial products and one that adds the
+// partial sums up itself (a third kernel does past 64 of them), subtracts and
+// leaves the norm's partials: five launches where there were nine.
+// Beyond, the second pass is taken only where the first removed most of w.
+//
+// (Taking alpha v_J and beta v_(J-1) off first, so that one full pass is
+// enough, halves the traffic of long vectors, 3.5 of 98 ms of a chi = 1024
+// update. It is not done: with w rounded otherwise in its last bit, one
+// value in some runs falls to the other side of a bf16 rounding in the next
+// products, and the Ritz vector moves by up to 7e-7 in 13% of them.)
+osmps_status orthogonalise(osmps_ctx* ctx, const double* V, int64_t ld, int64_t n, int nv_max, double* w,
+                           double* part, double* sc, cudaStream_t s) {
+  const int* state = lz_state(sc);
+  int ub = 0;
+  if (n > ((int64_t)1 << 18)) {
+    int* skip = reinterpret_cast<int*>(sc + OFF_MISC + 6);
+    OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 5, s));
+    OSMPS_TRY(project(ctx, V, ld, n, nv_max, w, part, sc + OFF_C1, s, state));
+    { k_reorth_decide<<<1, 32, 0, s>>>(sc + OFF_C1, sc + OFF_MISC + 5, state, skip); note_launch(); }
+    OSMPS_TRY(project(ctx, V, ld, n, nv_max, w, part, sc + OFF_C2, s, state, skip));
+    OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 3, s));
+  } else {
+    const int nb = dot_blocks(n, ctx->sm_count);
+    const dim3 dgrid(nb, (unsigned)cdiv(nv_max, DOT_GROUP));
+    const bool tiny = n <= ((int64_t)1 << 15);
+    const int ut = tiny ? 64 : DOT_THREADS;
+    ub = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(tiny ? n : n >> 1, ut), DOT_MAX_BLOCKS));
+    const auto update = tiny ? k_lz_update<false> : k_lz_update<true>;
+    for (double* c : {sc + OFF_C1, sc + OFF_C2}) {
+      k_multidot<<<dgrid, DOT_THREADS, 0, s>>>(V, ld, nv_max, w, n, part, state, nullptr);
+      if (nb > 64) {  // too many partial sums for every block to add up
+        k_multidot_final<<<nv_max, 256, 0, s>>>(part, nb, c, state, nullptr);
+        note_launch();
+      }
+      update<<<ub, ut, 0, s>>>(V, ld, w, n, c, part, nb > 64 ? 0 : nb, state);
+      note_launches(2);
+    }
+  }
+  k_lz_norm<<<1, DOT_THREADS, 0, s>>>(sc, part, ub);
   note_launch();
   OSMPS_LAUNCH_CHECK();
   return OSMPS_OK;
@@ -618,13 +897,58 @@ struct SyncOnExit {
   }
 };
 
+// Work beside the main stream, on the context's side stream: fork (after what
+// the main stream holds so far), launches on stream(), mark, join (the main
+// stream waits for the mark). In a capture the same calls make a parallel
+// branch. A failed call leaves nothing running behind it.
+class SideWork {
+ public:
+  explicit SideWork(osmps_ctx* c) : c_(c) {}
+  ~SideWork() {
+    if (open_ && !joined_ && !c_->capturing) cudaStreamSynchronize(c_->side_stream);
+  }
+  osmps_status open() {
+    if (!c_->side_stream) {
+      OSMPS_CUDA(cudaStreamCreateWithFlags(&c_->side_stream, cudaStreamNonBlocking));
+      OSMPS_CUDA(cudaEventCreateWithFlags(&c_->side_ev[0], cudaEventDisableTiming));
+      OSMPS_CUDA(cudaEventCreateWithFlags(&c_->side_ev[1], cudaEventDisableTiming));
+    }
+    open_ = true;
+    return OSMPS_OK;
+  }
+  cudaStream_t stream() const { return c_->side_stream; }
+  osmps_status fork(cudaStream_t q) {
+    joined_ = false;
+    OSMPS_CUDA(cudaEventRecord(c_->side_ev[0], q));
+    OSMPS_CUDA(cudaStreamWaitEvent(c_->side_stream, c_->side_ev[0], 0));
+    return OSMPS_OK;
+  }
+  osmps_status mark() {
+    OSMPS_CUDA(cudaEventRecord(c_->side_ev[1], c_->side_stream));
+    return OSMPS_OK;
+  }
+  osmps_status join(cudaStream_t q) {
+    OSMPS_CUDA(cudaStreamWaitEvent(q, c_->side_ev[1], 0));
+    joined_ = true;
+    return OSMPS_OK;
+  }
+  osmps_status wait() {
+    OSMPS_CUDA(cudaEventSynchronize(c_->side_ev[1]));
+    return OSMPS_OK;
+  }
+
+ private:
+  osmps_ctx* c_;
+  bool open_ = false, joined_ = true;
+};
+
 // Record [k_loop_init] -> while (cond) { step } and instantiate it. The step
 // is recorded by stream capture on the context's capture stream; workspace
 // growth is an error while the capture is open. gr.body_launches: kernels
 // one step launches (the capture's own count is taken back: recording
 // launches nothing).
-osmps_status record_step_graph(osmps_ctx* ctx, const double* sc, const StepRecorder& record,
-                               LzGraph& gr) {
+osmps_status record_step_graph(osmps_ctx* ctx, const double* sc, int max_iter,
+                               const StepRecorder& record, LzGraph& gr) {
   if (!ctx->capture_stream)
     OSMPS_CUDA(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
   cudaStream_t cs = ctx->capture_stream;
@@ -632,7 +956,7 @@ osmps_status record_step_graph(osmps_ctx* ctx, const double* sc, const StepRecor
   cudaGraphConditionalHandle cond;
   OSMPS_CUDA(cudaGraphConditionalHandleCreate(&cond, gr.g, 0, cudaGraphCondAssignDefault));
   cudaKernelNodeParams kn = {};
-  void* args[2] = {(void*)&sc, (void*)&cond};
+  void* args[3] = {(void*)&sc, (void*)&max_iter, (void*)&cond};
   kn.func = (void*)k_loop_init;
   kn.gridDim = dim3(1);
   kn.blockDim = dim3(1);
@@ -682,7 +1006,7 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
   if (!w) return st;
   double* sc = (double*)ws_get(ctx, SLOT_LZ_SCAL, SCAL_COUNT * 8, s, &st);
   if (!sc) return st;
-  double* part = (double*)ws_get(ctx, SLOT_LZ_PART, (size_t)MAXIT * DOT_MAX_BLOCKS * 8, s, &st);
+  double* part = (double*)ws_get(ctx, SLOT_LZ_PART, PART_BYTES, s, &st);
   if (!part) return st;
   const bool graph = use_step_graph(ctx, n, max_iter);
   double* X = nullptr;
@@ -716,34 +1040,46 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
 
   // One step on stream q: w = H_eff V[J] (x is V[J] itself, or the buffer X
   // that the previous step's k_next_vector filled), projected out of the
-  // projector rows and twice out of V[0..J], its norm, the tridiagonal solve
-  // with the stopping decision, and V[J+1] (and its copy in X, when there is
-  // one). final_blocks bounds J + 1.
-  // Krylov vectors of 2^16 entries and more take the second Gram-Schmidt
-  // pass only when the first asks for it; smaller ones, where the launches
-  // and not the vector traffic cost, always take both.
-  const bool twice_if_needed = n >= ((int64_t)1 << 16);
-  auto step = [&](cudaStream_t q, const double* x, int final_blocks,
-                  cudaGraphConditionalHandle cond, int set_cond) -> osmps_status {
+  // projector rows, orthogonalised and normed, the tridiagonal solve with the
+  // stopping decision, and V[J+1] (and its copy in X, when there is one).
+  // nv_max bounds J + 1.
+  //
+  // The tridiagonal solve is one block's chain of dependent float64
+  // operations (20 us at m = 10, 60 at m = 40) that only the decision to stop
+  // waits for. Where a step costs little more than that, it runs beside the
+  // next step's product on a stream of its own (`beside`): a solve that
+  // converges then has run one step for nothing (~50 us at chi = 32), and
+  // every step before it is that much shorter. Larger vectors, whose step
+  // costs ten times the solve, decide before the next product.
+  const bool beside = n < ((int64_t)1 << 20);
+  SideWork side(ctx);
+  if (beside) OSMPS_TRY(side.open());
+  const auto tridiag = [&](cudaStream_t q) -> osmps_status {
+    k_tridiag<<<1, TRI_THREADS, 0, q>>>(sc, max_iter, tol, (long long)n);
+    note_launch();
+    OSMPS_LAUNCH_CHECK();
+    return OSMPS_OK;
+  };
+  auto step = [&](cudaStream_t q, const double* x, int nv_max, cudaGraphConditionalHandle cond,
+                  int set_cond, bool first) -> osmps_status {
+    const bool fork = beside && !first;
+    if (fork) {
+      OSMPS_TRY(side.fork(q));
+      OSMPS_TRY(tridiag(side.stream()));
+      if (!set_cond)
+        OSMPS_CUDA(cudaMemcpyAsync(ctx->host_pinned, sc + OFF_MISC, MISC_READ * 8, cudaMemcpyDeviceToHost,
+                                   side.stream()));
+      OSMPS_TRY(side.mark());
+    }
     OSMPS_TRY(matvec(x, w, q));
     if (kp > 0) {  // the operator restricted to the complement: w <- (1 - P^T P) H v_j
       OSMPS_TRY(project(ctx, P, ldp, n, kp, w, part, sc + OFF_PROJ, q));
       OSMPS_TRY(project(ctx, P, ldp, n, kp, w, part, sc + OFF_PROJ + MAX_PROJ, q));
     }
-    if (twice_if_needed) {  // the second pass only where the first removed most of w
-      int* skip = reinterpret_cast<int*>(sc + OFF_MISC + 6);
-      OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 5, q));
-      OSMPS_TRY(project(ctx, V, ld, n, final_blocks, w, part, sc + OFF_C1, q, state));
-      { k_reorth_decide<<<1, 32, 0, q>>>(sc + OFF_C1, sc + OFF_MISC + 5, state, skip); note_launch(); }
-      OSMPS_TRY(project(ctx, V, ld, n, final_blocks, w, part, sc + OFF_C2, q, state, skip));
-    } else {
-      OSMPS_TRY(project(ctx, V, ld, n, final_blocks, w, part, sc + OFF_C1, q, state));
-      OSMPS_TRY(project(ctx, V, ld, n, final_blocks, w, part, sc + OFF_C2, q, state));
-    }
-    OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 3, q));
-    { k_tridiag<<<1, TRI_THREADS, 0, q>>>(sc, max_iter, tol, (long long)n, cond, set_cond); note_launch(); }
-    OSMPS_LAUNCH_CHECK();
-    { k_next_vector<<<ew_blocks(n), 256, 0, q>>>(V, ld, w, n, sc, X); note_launch(); }
+    OSMPS_TRY(orthogonalise(ctx, V, ld, n, nv_max, w, part, sc, q));
+    if (fork) OSMPS_TRY(side.join(q));
+    if (!beside) OSMPS_TRY(tridiag(q));
+    { k_next_vector<<<ew_blocks(n), 256, 0, q>>>(V, ld, w, n, sc, X, max_iter, cond, set_cond); note_launch(); }
     OSMPS_LAUNCH_CHECK();
     return OSMPS_OK;
   };
@@ -753,17 +1089,22 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
   long long body_launches = 0;
   if (!graph) {
     for (int j = 0; j < max_iter; ++j) {
-      OSMPS_TRY(step(s, V + (int64_t)j * ld, j + 1, 0, 0));
-      OSMPS_CUDA(cudaMemcpyAsync(ctx->host_pinned, sc + OFF_MISC, MISC_READ * 8,
-                                 cudaMemcpyDeviceToHost, s));
-      OSMPS_CUDA(cudaStreamSynchronize(s));
+      OSMPS_TRY(step(s, V + (int64_t)j * ld, j + 1, 0, 0, j == 0));
+      if (beside) {  // the decision on T_j, while step j runs
+        if (j == 0) continue;
+        OSMPS_TRY(side.wait());
+      } else {
+        OSMPS_CUDA(cudaMemcpyAsync(ctx->host_pinned, sc + OFF_MISC, MISC_READ * 8,
+                                   cudaMemcpyDeviceToHost, s));
+        OSMPS_CUDA(cudaStreamSynchronize(s));
+      }
       if (lz_state_in_misc(ctx->host_pinned)[ST_STOP] != STOP_NONE) break;
     }
   } else {
     // Step 0 runs directly: it sizes every workspace slot a step uses, so
     // nothing grows while the step is recorded. The other steps run in the
     // graph loop, recorded now or replayed from the context's cache.
-    OSMPS_TRY(step(s, V, 1, 0, 0));
+    OSMPS_TRY(step(s, V, 1, 0, 0, true));
     std::vector<long long> key(mkey, mkey + (mkey ? nmkey : 0));
     long long tol_bits;
     memcpy(&tol_bits, &tol, sizeof tol_bits);
@@ -776,11 +1117,11 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
         if (c.key == key) gr = &c;
     if (!gr) {
       const StepRecorder rec = [&](cudaStream_t q, cudaGraphConditionalHandle cond) {
-        return step(q, X, max_iter, cond, 1);
+        return step(q, X, max_iter, cond, 1, false);
       };
       LzGraph fresh;
       fresh.key = key;
-      const osmps_status rs = record_step_graph(ctx, sc, rec, fresh);
+      const osmps_status rs = record_step_graph(ctx, sc, max_iter, rec, fresh);
       if (rs != OSMPS_OK) {
         destroy_graph(fresh);
         return rs;
@@ -807,6 +1148,7 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
     OSMPS_CUDA(cudaGraphLaunch(gr->e, s));
     note_launch();  // k_loop_init
   }
+  if (beside) OSMPS_TRY(tridiag(s));  // the last T of a full basis (returns at once after a stop)
   // Ritz vector theta = sum_i s_i v_i, normalised
   { k_combine_scalar<<<ew_blocks(n), 256, 0, s>>>(V, ld, sc, theta, n); note_launch(); }
   OSMPS_LAUNCH_CHECK();
@@ -820,7 +1162,7 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
   const double e = ctx->host_pinned[0], res = ctx->host_pinned[1];
   const int* hs = lz_state_in_misc(ctx->host_pinned);
   const int stop = hs[ST_STOP], m = hs[ST_M];
-  if (graph) note_launches(body_launches * (long long)(m - 1));  // the loop ran m - 1 steps
+  if (graph) note_launches(body_launches * (long long)(hs[ST_J] - 1));  // steps run by the loop
   if (*hflag & 1) {
     cudaMemsetAsync(ctx->dev_flags, 0, sizeof(int), s);
     return set_error(OSMPS_ETIMEOUT, "lanczos: a bounded device wait gave up");
@@ -912,7 +1254,7 @@ extern "C" osmps_status osmps_lanczos_ground_projected(
   if (k > 0) {
     Q = (double*)ws_get(ctx, SLOT_LZ_PROJ, (size_t)k * ld * 8, s, &st);
     if (!Q) return st;
-    double* part = (double*)ws_get(ctx, SLOT_LZ_PART, (size_t)MAXIT * DOT_MAX_BLOCKS * 8, s, &st);
+    double* part = (double*)ws_get(ctx, SLOT_LZ_PART, PART_BYTES, s, &st);
     if (!part) return st;
     double* sc = (double*)ws_get(ctx, SLOT_LZ_SCAL, SCAL_COUNT * 8, s, &st);
     if (!sc) return st;
@@ -979,9 +1321,8 @@ __device__ __forceinline__ double block_max(double v, double* red) {
   return r;
 }
 
-// Step j = state J of the propagator: record alpha_j and beta_j as the
-// ground-state kernel does, then u = exp(-i tau T_m) e_1 for the leading
-// m = j + 1 rows of T. u comes from the Taylor series applied to e_1 in s
+// The propagator's T_{j+1}, j = state ST_T: u = exp(-i tau T_m) e_1 for the
+// leading m = j + 1 rows of T. u comes from the Taylor series applied to e_1 in s
 // substeps of length h = tau / s, s the smallest count with |h| g <= 1 for
 // the Gershgorin bound g of T_m, EXPM_TAYLOR terms each; one thread per
 // coordinate, each term one tridiagonal product. (The float64 eigensolver
@@ -996,7 +1337,7 @@ __global__ void __launch_bounds__(EXPM_THREADS) k_expm_tridiag(double* __restric
   __shared__ double a[EXPM_MAXIT], b[EXPM_MAXIT], tr[EXPM_MAXIT], ti[EXPM_MAXIT];
   __shared__ double red[EXPM_THREADS / 32];
   int* st = lz_state(sc);
-  const int j = st[ST_J];
+  const int j = st[ST_T];
   const int i = threadIdx.x;
   if (j < 0 || j >= max_iter || j >= EXPM_MAXIT) {  // not reachable from the driver below
     if (i == 0) {
@@ -1006,11 +1347,6 @@ __global__ void __launch_bounds__(EXPM_THREADS) k_expm_tridiag(double* __restric
     return;
   }
   const int m = j + 1;
-  if (i == 0) {
-    sc[OFF_ALPHA + j] = sc[OFF_C1 + j] + sc[OFF_C2 + j];
-    sc[OFF_BETA + j] = sqrt(sc[OFF_MISC + 3]);
-  }
-  __syncthreads();
   const bool act = i < m;
   if (act) {
     a[i] = sc[OFF_ALPHA + i];
@@ -1097,8 +1433,8 @@ __global__ void __launch_bounds__(EXPM_THREADS) k_expm_tridiag(double* __restric
     else if (m >= max_iter)
       stop = STOP_CAP;
     st[ST_M] = m;
+    st[ST_T] = j + 1;
     st[ST_STOP] = stop;
-    if (stop == STOP_NONE) st[ST_J] = j + 1;
   }
 }
 
@@ -1192,7 +1528,7 @@ osmps_status expm_core(osmps_ctx* ctx, int64_t n_c, const double* theta_emb, dou
   if (!w) return st;
   double* sc = (double*)ws_get(ctx, SLOT_LZ_SCAL, SCAL_COUNT * 8, s, &st);
   if (!sc) return st;
-  double* part = (double*)ws_get(ctx, SLOT_LZ_PART, (size_t)MAXIT * DOT_MAX_BLOCKS * 8, s, &st);
+  double* part = (double*)ws_get(ctx, SLOT_LZ_PART, PART_BYTES, s, &st);
   if (!part) return st;
   OSMPS_TRY(pinned_reserve(ctx, 16));
   int* state = lz_state(sc);
@@ -1208,12 +1544,10 @@ osmps_status expm_core(osmps_ctx* ctx, int64_t n_c, const double* theta_emb, dou
   OSMPS_CUDA(cudaMemsetAsync(state, 0, 4 * sizeof(int), s));
   for (int j = 0; j < max_iter; ++j) {
     OSMPS_TRY(matvec(V + (int64_t)j * ld, w, s));
-    OSMPS_TRY(project(ctx, V, ld, n, j + 1, w, part, sc + OFF_C1, s, state));
-    OSMPS_TRY(project(ctx, V, ld, n, j + 1, w, part, sc + OFF_C2, s, state));
-    OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 3, s));
+    OSMPS_TRY(orthogonalise(ctx, V, ld, n, j + 1, w, part, sc, s));
     { k_expm_tridiag<<<1, EXPM_THREADS, 0, s>>>(sc, max_iter, tol, tau, (long long)n_c); note_launch(); }
     OSMPS_LAUNCH_CHECK();
-    { k_next_vector<<<ew_blocks(n), 256, 0, s>>>(V, ld, w, n, sc, nullptr); note_launch(); }
+    { k_next_vector<<<ew_blocks(n), 256, 0, s>>>(V, ld, w, n, sc, nullptr, max_iter, 0, 0); note_launch(); }
     OSMPS_LAUNCH_CHECK();
     OSMPS_CUDA(cudaMemcpyAsync(ctx->host_pinned, sc + OFF_MISC, MISC_READ * 8,
                                cudaMemcpyDeviceToHost, s));

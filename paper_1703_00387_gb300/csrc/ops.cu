@@ -149,40 +149,48 @@ struct WTable {
   bool dense;
 };
 
-// Every thread of the block calls it (whole warps): a warp per output, lanes
-// over the inputs, the nonzero ones compacted by ballots.
-template <typename T>
-__device__ __forceinline__ void gather_terms(const double* __restrict__ Mat, int P, int Q,
-                                             WTable<T>& w) {
+// Fill NT tables. Every thread of the block calls it (whole warps): a warp
+// per output, lanes over the inputs, the nonzero ones compacted by ballots.
+// Ends with a barrier.
+template <int NT, typename T>
+__device__ __forceinline__ void gather_terms(const double* const (&Mat)[NT], const int (&P)[NT],
+                                             const int (&Q)[NT], WTable<T>* const (&tab)[NT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  for (int o = warp; o < Q; o += warps) {
-    int n = 0;
-    for (int i0 = 0; i0 < P; i0 += 32) {
-      const double m = i0 + lane < P ? Mat[(i0 + lane) * Q + o] : 0.0;
-      n += __popc(__ballot_sync(0xffffffffu, m != 0.0));
-    }
-    if (lane == 0) w.ptr[o + 1] = n;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    w.ptr[0] = 0;
-    for (int q = 0; q < Q; ++q) w.ptr[q + 1] += w.ptr[q];
-    w.Mat = Mat;
-    w.P = P;
-    w.Q = Q;
-    w.dense = w.ptr[Q] > WT_CAP || P > 32767;
-  }
-  __syncthreads();
-  if (!w.dense)
-    for (int o = warp; o < Q; o += warps) {
-      int n = w.ptr[o];
-      for (int i0 = 0; i0 < P; i0 += 32) {
-        const double m = i0 + lane < P ? Mat[(i0 + lane) * Q + o] : 0.0;
-        const unsigned nz = __ballot_sync(0xffffffffu, m != 0.0);
-        if (m != 0.0) w.terms[n + __popc(nz & ((1u << lane) - 1u))] = WTerm<T>{(T)m, (short)(i0 + lane), (short)(m == 1.0)};
-        n += __popc(nz);
+#pragma unroll
+  for (int k = 0; k < NT; ++k)
+    for (int o = warp; o < Q[k]; o += warps) {
+      int n = 0;
+      for (int i0 = 0; i0 < P[k]; i0 += 32) {
+        const double m = i0 + lane < P[k] ? Mat[k][(i0 + lane) * Q[k] + o] : 0.0;
+        n += __popc(__ballot_sync(0xffffffffu, m != 0.0));
       }
+      if (lane == 0) tab[k]->ptr[o + 1] = n;
     }
+  __syncthreads();
+  if (lane == 0 && warp < NT) {
+    WTable<T>& w = *tab[warp];
+    const int q1 = Q[warp < NT ? warp : 0];
+    w.ptr[0] = 0;
+    for (int q = 0; q < q1; ++q) w.ptr[q + 1] += w.ptr[q];
+    w.Mat = Mat[warp < NT ? warp : 0];
+    w.P = P[warp < NT ? warp : 0];
+    w.Q = q1;
+    w.dense = w.ptr[q1] > WT_CAP || w.P > 32767;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < NT; ++k)
+    if (!tab[k]->dense)
+      for (int o = warp; o < Q[k]; o += warps) {
+        int n = tab[k]->ptr[o];
+        for (int i0 = 0; i0 < P[k]; i0 += 32) {
+          const double m = i0 + lane < P[k] ? Mat[k][(i0 + lane) * Q[k] + o] : 0.0;
+          const unsigned nz = __ballot_sync(0xffffffffu, m != 0.0);
+          if (m != 0.0)
+            tab[k]->terms[n + __popc(nz & ((1u << lane) - 1u))] = WTerm<T>{(T)m, (short)(i0 + lane), (short)(m == 1.0)};
+          n += __popc(nz);
+        }
+      }
   __syncthreads();
 }
 
@@ -316,7 +324,7 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
   const int P = (int)f.P, Q = (int)f.Q;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Pack<T, V>* xs = reinterpret_cast<Pack<T, V>*>(fsm) + lane;
-  gather_terms<T>(Mat, P, Q, tab);
+  bool first = true;  // the table is built while the first fibers' inputs arrive
   const int64_t nc = PACKED ? f.nc / V : f.nc, total = f.n_o1 * f.n_o2 * nc;
   for (int64_t e0 = (int64_t)blockIdx.x * (32 * F::N); e0 < total; e0 += (int64_t)gridDim.x * (32 * F::N)) {
     F fib;
@@ -333,8 +341,10 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
     if (staged) {
 #pragma unroll 4
       for (int i = warp; i < P; i += FIB_WARPS) xs[i * 32] = fib.load(in, (int64_t)i * f.istride);
-      __syncthreads();
     }
+    if (first) gather_terms<1, T>({Mat}, {P}, {Q}, {&tab});
+    else if (staged) __syncthreads();
+    first = false;
     for (int o = warp; o < Q; o += FIB_WARPS) {
       Pack<T, V> acc;
       if (staged) {
@@ -446,8 +456,7 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
     const int t2 = threadIdx.x / wr;
     ooff[threadIdx.x] = t2 * ldo + (int64_t)(threadIdx.x - t2 * wr) * chi_r;
   }
-  gather_terms<T>(Mat1, P1, Q1, tab1);
-  gather_terms<T>(Mat2, P2, Q2, tab2);
+  bool first = true;  // the tables are built while the first fibers' inputs arrive
   const int64_t nc = PACKED ? chi_r / V : chi_r, total = chi_l * nc;
   for (int64_t e0 = (int64_t)blockIdx.x * (32 * F::N); e0 < total; e0 += (int64_t)gridDim.x * (32 * F::N)) {
     F fib;
@@ -462,7 +471,9 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
     }
 #pragma unroll 4
     for (int k = warp; k < P1 * D; k += FIB_WARPS) xs[k * 32] = fib.load(T1, k * chi_r);
-    __syncthreads();
+    if (first) gather_terms<2, T>({Mat1, Mat2}, {P1, P2}, {Q1, Q2}, {&tab1, &tab2});
+    else __syncthreads();
+    first = false;
     for (int o = warp; o < Q1; o += FIB_WARPS)
 #pragma unroll
       for (int s2 = 0; s2 < D; ++s2) ms[(o * D + s2) * 32] = sum_terms<T, V>(tab1, o, xs + s2 * 32, D * 32);

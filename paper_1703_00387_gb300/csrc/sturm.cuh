@@ -54,6 +54,38 @@ __device__ __forceinline__ void sturm_counts(const double* __restrict__ d,
   }
 }
 
+// One point's count together with the last minor p_n = det(T - x I) as
+// value 2^exponent (the scalings taken out are exact).
+__device__ __forceinline__ int sturm_count_minor(const double* __restrict__ d,
+                                                 const double* __restrict__ e2, int n, double x,
+                                                 double* value, int* exponent) {
+  double pm = 0.0, p = 1.0;
+  int c = 0, ex = 0;
+  for (int i = 0; i < n; ++i) {
+    const double ei = i > 0 ? e2[i - 1] : 0.0;
+    double pn = fma(d[i] - x, p, -ei * pm);
+    const bool prev_neg = __double_as_longlong(p) < 0;
+    if ((__double_as_longlong(pn) << 1) == 0) pn = prev_neg ? DBL_MIN : -DBL_MIN;
+    c += (__double_as_longlong(pn) < 0) != prev_neg;
+    pm = p;
+    p = pn;
+    if ((i & 7) == 7) {
+      const long long bp = __double_as_longlong(p) & 0x7FF0000000000000ll;
+      const long long bq = __double_as_longlong(pm) & 0x7FF0000000000000ll;
+      const int e = (int)((bp > bq ? bp : bq) >> 52);
+      if (e < 1023 - 200 || e > 1023 + 200) {
+        const double f = __longlong_as_double((long long)(2046 - e) << 52);
+        p *= f;
+        pm *= f;
+        ex += e - 1023;
+      }
+    }
+  }
+  *value = p;
+  *exponent = ex;
+  return c;
+}
+
 // The same count in float32 (d, e2, x as floats), for narrowing a bracket
 // before the float64 count resolves it: the count is exact for a tridiagonal
 // within a few float32 ulps of T (entrywise), so it can misplace an
