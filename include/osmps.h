@@ -240,9 +240,9 @@ osmps_status osmps_dgemm_emu(osmps_ctx* ctx, const double* A, const double* B, d
  * A[j+2.., j]) stored below the subdiagonal of column j (column-major view;
  * the layout of LAPACK's dsytrd with uplo = L). A: n x n device array
  * holding the full symmetric matrix (both triangles), overwritten. Panels of
- * 32 columns on a cooperative kernel with two grid barriers per column, the
+ * 32 columns on a cooperative kernel whose blocks exchange tagged words, the
  * trailing updates on the float64-accurate emulated tensor-core GEMM.
- * 2 <= n <= 8192, else ESHAPE; ETIMEOUT if a bounded barrier wait gave up. */
+ * 2 <= n <= 8192, else ESHAPE; ETIMEOUT if a bounded wait gave up.       */
 osmps_status osmps_sytrd(osmps_ctx* ctx, double* A, int64_t n, double* d, double* e, double* tau,
                          void* stream);
 
@@ -308,8 +308,8 @@ osmps_status osmps_vec_norm2(osmps_ctx* ctx, const double* x, int64_t n, double*
  * with a limit of limit_us microseconds (1 .. 1e6, else EINVAL):
  *   which = 0: a kernel that holds tensor memory waits on an mbarrier that
  *              no thread arrives at, then frees the tensor memory;
- *   which = 1: a cooperative grid waits at a grid barrier one of its blocks
- *              never reaches.
+ *   which = 1: a cooperative grid polls for a tagged word one of its blocks
+ *              never publishes.
  * Returns OSMPS_ETIMEOUT when the wait gave up (the expected outcome), OK
  * otherwise. Synchronises `stream`.                                          */
 osmps_status osmps_selftest_wait_timeout(osmps_ctx* ctx, int which, double limit_us, void* stream);

@@ -753,8 +753,8 @@ def osmps_sytrd(ctx, A, d, e, tau, stream=None):
 
 def osmps_selftest_wait_timeout(ctx, which, limit_us=2000.0, stream=None):
     """Make one bounded device wait run out on purpose (which = 0: an mbarrier
-    wait in a kernel holding tensor memory; 1: a grid barrier one block never
-    reaches). Raises OsmpsError(ETIMEOUT) when the wait gave up, as it should."""
+    wait in a kernel holding tensor memory; 1: a tagged word one block never
+    publishes). Raises OsmpsError(ETIMEOUT) when the wait gave up, as it should."""
     _check(lib().osmps_selftest_wait_timeout(ctx.ptr, int(which), float(limit_us), _stream(stream)))
 
 

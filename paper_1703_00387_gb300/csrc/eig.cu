@@ -658,7 +658,7 @@ osmps_status eig_top(osmps_ctx* ctx, double* G, int64_t n, int64_t nev, double* 
     OSMPS_CUDA(cudaStreamSynchronize(s));
     if (flag != 0) {
       cudaMemsetAsync(ctx->dev_flags + 3, 0, sizeof(int), s);
-      return set_error(OSMPS_ETIMEOUT, "eigensolver: a grid barrier wait of the reduction gave up");
+      return set_error(OSMPS_ETIMEOUT, "eigensolver: a wait of the panel reduction gave up");
     }
   }
   dim3 grid((unsigned)cdiv(n, 32), (unsigned)cdiv(nev, 32));

@@ -6,12 +6,13 @@
 // short limit, on a barrier that nothing completes:
 //   which = 0: one CTA allocates tensor memory (TMEM) as the tcgen05 kernels
 //              do, waits on an mbarrier no thread arrives at, frees the TMEM;
-//   which = 1: a cooperative grid whose last block leaves without arriving at
-//              the grid barrier the others wait at.
+//   which = 1: a cooperative grid whose last block leaves without publishing
+//              the tagged word the others poll for (as the panel reduction's
+//              blocks do).
 // Nothing faults, traps or spins without a bound; the context stays usable.
 #include "common.cuh"
-#include "gridsync.cuh"
 #include "ieee.cuh"
+#include "tagged.cuh"
 #include "tcgen05.cuh"
 
 namespace osmps {
@@ -49,10 +50,14 @@ __global__ void __launch_bounds__(64, 1) k_selftest_mbarrier(uint64_t limit_ns, 
   }
 }
 
-__global__ void k_selftest_grid(unsigned* bar, uint64_t limit_ns, int* __restrict__ err) {
-  __shared__ int s_ok;
-  if (blockIdx.x == gridDim.x - 1) return;  // this block never arrives
-  grid_barrier(bar, gridDim.x, err, &s_ok, limit_ns);
+// Every block but the last publishes its tagged word and waits for all of
+// them; the last never publishes.
+__global__ void k_selftest_words(ulonglong2* words, uint64_t limit_ns, int* __restrict__ err) {
+  if (blockIdx.x == gridDim.x - 1) return;
+  if (threadIdx.x == 0) put_word(words + blockIdx.x, 1.0, 1);
+  const ulonglong2* p[1] = {threadIdx.x < gridDim.x ? words + threadIdx.x : nullptr};
+  double v[1];
+  if (!get_words<1>(p, 1, v, limit_ns)) atomicOr(err, 1);
 }
 
 __global__ void k_selftest_convert(const double* __restrict__ x64, float* __restrict__ y32,
@@ -124,8 +129,7 @@ extern "C" osmps_status osmps_selftest_wait_timeout(osmps_ctx* ctx, int which, d
   CtxScope scope_(ctx);
   cudaStream_t s = (cudaStream_t)stream;
   int* flag = ctx->dev_flags + SELFTEST_FLAG;
-  unsigned* bar = reinterpret_cast<unsigned*>(ctx->dev_flags + SELFTEST_FLAG + 1);
-  OSMPS_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), s));
+  OSMPS_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
   const uint64_t limit_ns = (uint64_t)(limit_us * 1e3);
   if (which == 0) {
     k_selftest_mbarrier<<<1, 64, 0, s>>>(limit_ns, flag);
@@ -133,8 +137,12 @@ extern "C" osmps_status osmps_selftest_wait_timeout(osmps_ctx* ctx, int which, d
     OSMPS_LAUNCH_CHECK();
   } else {
     const int G = std::max(2, std::min(ctx->sm_count, 8));
-    void* args[] = {&bar, (void*)&limit_ns, &flag};
-    OSMPS_CUDA(cudaLaunchCooperativeKernel((void*)k_selftest_grid, dim3(G), dim3(64), args, 0, s));
+    osmps_status st = OSMPS_OK;
+    auto* words = (ulonglong2*)ws_get(ctx, SLOT_TRD, 8 * sizeof(ulonglong2), s, &st);
+    if (!words) return st;
+    OSMPS_CUDA(cudaMemsetAsync(words, 0, 8 * sizeof(ulonglong2), s));
+    void* args[] = {&words, (void*)&limit_ns, &flag};
+    OSMPS_CUDA(cudaLaunchCooperativeKernel((void*)k_selftest_words, dim3(G), dim3(64), args, 0, s));
     note_launch();
   }
   int h = 0;
@@ -142,6 +150,6 @@ extern "C" osmps_status osmps_selftest_wait_timeout(osmps_ctx* ctx, int which, d
   OSMPS_CUDA(cudaStreamSynchronize(s));
   if (h & 1)
     return set_error(OSMPS_ETIMEOUT, "osmps_selftest_wait_timeout: the %s wait gave up after %g us",
-                     which == 0 ? "mbarrier" : "grid barrier", limit_us);
+                     which == 0 ? "mbarrier" : "tagged word", limit_us);
   return OSMPS_OK;
 }

@@ -5,45 +5,65 @@
 // v_j = (0, .., 0, 1 at j+1, A[j+2.., j]).
 //
 // Blocked as in LAPACK's dlatrd: panels of NB columns. Inside a panel, column
-// j is first brought up to date with the panel's earlier reflectors
-// (A - V W^T - W V^T), its reflector is formed, and
+// j is brought up to date with the panel's earlier reflectors
+// (x = A e_j - V W^T e_j - W V^T e_j), its reflector is formed, and
 //   w = tau (A22 v - W y - V z) + alpha2 v,   y = V^T v,  z = W^T v,
-//   alpha2 = -(tau/2) tau (A22 v - W y - V z)^T v
-// with A22 the trailing matrix as it stood at the start of the panel. Since
-// y and z are V^T v and W^T v, (W y + V z)^T v = 2 y^T z, so the scalar
-// needs only t^T v (t = A22 v) besides y and z: it comes out of the same
-// reduction as y and z, and a column costs two grid-wide reductions:
-//   1. the squared norm of the updated column below the subdiagonal;
-//   2. t = A22 v on every row (the float64 work, spread over all SMs), with
-//      the partial sums of y, z and t^T v.
-// The kernel is one cooperative launch per panel; its grid barriers are a
-// counter in global memory with bounded waits (after ~2 s a block records
-// the failure in the error flag and leaves). Rows are dealt to the blocks
-// round robin (row r to block r mod G), and each block keeps its rows of V
-// and W in shared memory, so only v (every block needs all of it) and the
-// reductions cross the grid. After each panel the trailing block is updated,
-// A22 -= V W^T + W V^T, by the float64-accurate emulated tensor-core GEMM,
-// subtracting in its epilogue. The matrix is kept full (both triangles), so
-// row r of the trailing block is contiguous; the reflectors overwrite column
-// j below the subdiagonal (row j of the row-major view), which later
-// columns never read.
+//   alpha2 = -(tau^2/2) (v^T A22 v - 2 y^T z)
+// with A22 the trailing matrix as it stood at the start of the panel. After
+// the panel the trailing block is updated, A22 -= V W^T + W V^T, by the
+// float64-accurate emulated tensor-core GEMM, subtracting in its epilogue.
+// The matrix is kept full (both triangles), so row r of the trailing block is
+// contiguous; the reflectors overwrite column j below the subdiagonal (row j
+// of the row-major view), which later columns never read.
+//
+// A panel is one cooperative launch, its rows dealt to the blocks round robin;
+// each block keeps its rows of V and W in shared memory. What bounds a column
+// is not its float64 work (A22 v: 13 us at m = 2048, under 2 below m = 700) but
+// the way of its numbers between the blocks and the dependent float64 chains
+// around it, so the column is arranged for few exchanges off the critical
+// path and none through a barrier:
+//   * v = e_(j+1) + inv u with u the column below j + 1 and inv known only
+//     after sigma = u^T u, a square root and two divisions (2000 clocks, formed
+//     by one warp of every block from its own copy of u beside the rest):
+//     everything linear in v is formed from u. A22 v = A e_(j+1) + inv A22 u,
+//     y = V^T e_(j+1) + inv V^T u, v^T A22 v = A_(j+1)(j+1) + 2 inv s1 + inv^2 s2
+//     with s1 = e_(j+1)^T A u and s2 = u^T A22 u. Only s2 needs the product
+//     A22 u; the other 2 jj + 1 sums are on their way while it runs, and what
+//     is left to do when s2 arrives is four operations per row.
+//   * every number crosses the GPU as a 16-byte word of value and column
+//     number, written and read in one access; a reader polls for the number,
+//     so an exchange is one store and one load, not a fence, an atomic, a wait
+//     and a load. Words alternate between two buffers: a block can publish
+//     column j + 2 only after it has read every block's column j + 1, which a
+//     block publishes after its last read of column j.
+//   * the 2 jj + 1 sums: up to 32 blocks, every block adds up all partial
+//     sums itself; beyond, one warp per sum adds it up and publishes it.
+//   * row j + 1 of W (needed by every block for the next column) is published
+//     by its owner a column ahead; row j + 1 of V every block has.
+// Polls are bounded: after ~2 s a block records the failure in the error
+// flag and leaves, and later panels leave at once.
+// Measured per column, averaged over a reduction, against two grid barriers
+// per column with every block adding up all partial sums: n = 128 12.4 -> 5.7
+// us, 512 13.8 -> 7.8, 1024 15.0 -> 8.0, 2048 18.9 -> 11.2.
 #include <cooperative_groups.h>
 
 #include <cfloat>
 #include <cmath>
 
 #include "common.cuh"
-#include "gridsync.cuh"
+#include "tagged.cuh"
 
 namespace osmps {
 namespace {
 
 constexpr int NB = 32;            // panel width (one lane per earlier reflector)
-constexpr int ST_THREADS = 256;
-constexpr int ST_WARPS = ST_THREADS / 32;
+constexpr int ROW_WARPS = 8;      // warps that share the block's rows
+constexpr int ROW_THREADS = 32 * ROW_WARPS;
+constexpr int ST_THREADS = ROW_THREADS + 64;  // and one warp each for sums and scalars
 constexpr int MAXLOC = 64;        // rows per block at most
-constexpr int PW = 2 * NB + 2;    // partial sums per block: y | z | t^T v | ssq
-constexpr int P_TV = 2 * NB, P_SSQ = 2 * NB + 1;
+constexpr int MAXSUM = 64;        // 2 jj + 1 < 64 sums
+constexpr int LINE = 8;             // words per 128-byte line
+constexpr int DIRECT_G = 32;      // blocks up to which every block adds up all partial sums
 
 struct SytrdArgs {
   double* A;         // n x n, full symmetric (row r contiguous)
@@ -53,12 +73,18 @@ struct SytrdArgs {
   double* tau;       // reflector scalars
   double* Vp;        // panel reflectors, column-major NB x n: Vp[q * n + r]
   double* Wp;        // panel w vectors, same layout
-  double* col;       // updated column (n)
-  double* t;         // A22 v, only row j+1 is read by other blocks
-  double* part;      // per-block partial sums: G x PW
-  unsigned* bar;     // grid barrier counter
-  unsigned bar_base; // counter value at the start of this launch
-  int* err;          // bit 0: a barrier wait gave up
+  // tagged words, two buffers each (column parity), laid out so that no
+  // 128-byte line holds words of two blocks (a line that several blocks write
+  // while all poll it moves between the two dies' caches: gathering a column
+  // of 1024 entries from 152 blocks took 4 us in row order)
+  ulonglong2* X;     // [2][G][lw] column entries, block by block
+  ulonglong2* Wn;    // [2][NB] row j + 1 of W
+  ulonglong2* part;  // [2][G][MAXSUM] partial sums
+  ulonglong2* R;     // [2][MAXSUM][LINE] sums (G > DIRECT_G)
+  ulonglong2* T2;    // [2][G][LINE] partial u^T A22 u
+  int lw;            // words per block in X: its rows, rounded up to whole lines
+  int sa;            // row stride of the block's rows in shared memory (0: they stay in L2)
+  int* err;          // bit 0: a poll gave up
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -66,310 +92,343 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sum over the G blocks' partials part[b * PW + off] by one warp (lanes over
-// blocks, fixed order, then a fixed shuffle tree): the same value in every
-// block and every lane.
-__device__ __forceinline__ double sum_parts(const double* __restrict__ part, int G, int off) {
-  const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  for (int b = lane; b < G; b += 32) s += part[(size_t)b * PW + off];
-  return warp_sum(s);
-}
-
-// Four threads of a quad share one row: sum over q < jj with q = sub (mod 4)
-// of a[q] bs[q] + c[q] ds[q] in two interleaved partial sums, then two xor
-// shuffles, so every thread of the quad gets the total. GB300's float64
-// pipe is narrow: a warp-wide tree would spend five additions of 32 lanes on
-// each row's sum, the quad two of four. Every lane of the warp must call it.
-__device__ __forceinline__ double quad_dot2(const double* __restrict__ a,
-                                            const double* __restrict__ bs,
-                                            const double* __restrict__ c,
-                                            const double* __restrict__ ds, int jj, int sub) {
-  double p0 = 0.0, p1 = 0.0;
-  int q = sub;
-  for (; q + 4 < jj; q += 8) {
-    p0 = fma(a[q], bs[q], fma(c[q], ds[q], p0));
-    p1 = fma(a[q + 4], bs[q + 4], fma(c[q + 4], ds[q + 4], p1));
-  }
-  if (q < jj) p0 = fma(a[q], bs[q], fma(c[q], ds[q], p0));
-  double x = p0 + p1;
-  x += __shfl_xor_sync(0xffffffffu, x, 1);
-  x += __shfl_xor_sync(0xffffffffu, x, 2);
-  return x;
-}
-
+// SA: the block's rows of A22 are kept in shared memory for the whole panel
+// (loaded once; a column then waits for no L2 round trip). VEC: rows in global
+// memory start on 16-byte boundaries.
+template <bool VEC, bool SA>
 __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
-  extern __shared__ double sv[];            // v over rows [0, n) (entries up to j are 0)
+  extern __shared__ __align__(16) double su[];  // u over rows [0, n + 64): zero up to j + 1 and past n
+  double* sA = su + ((a.n + 64 + 1) & ~1);      // (SA) rows of A, columns k0 ..
   __shared__ double sV[MAXLOC][NB];         // this block's rows of V and W
   __shared__ double sW[MAXLOC][NB];
-  __shared__ double st[MAXLOC];             // this block's rows of t = A22 v
-  __shared__ double sVs[NB], sWs[NB];       // V_q[j], W_q[j] of the current column
-  __shared__ double scoef[2 * NB + 1];      // y | z | t^T v of the current column
-  __shared__ double sq[MAXLOC];             // squares of this block's column entries
-  __shared__ double sc[4];                  // tau, 1/(alpha - beta), alpha2, row j+1 sum
-  __shared__ int s_ok;
-  const int n = a.n, G = gridDim.x, b = blockIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int cnt = b < n ? (n - b + G - 1) / G : 0;  // rows b, b + G, ...
-  double* part = a.part + (size_t)b * PW;
-  unsigned target = a.bar_base;
-  // per-row work: the quad of threads 4 loc .. 4 loc + 3 takes row r = b + G loc
-  const int qloc = threadIdx.x >> 2, qsub = threadIdx.x & 3;
-  const int qrow = b + G * qloc;
-  const bool qmine = qloc < cnt;
-  // A[j][qrow], loaded one column ahead by the quad's first thread (row j of A
-  // is not written before column j reads it)
-  auto load_arow = [&](int jrow) {
-    return (qsub == 0 && qmine && jrow < n) ? a.A[(size_t)jrow * n + qrow] : 0.0;
-  };
-  double arow = load_arow(a.k0);
-
+  __shared__ double sVp[NB][NB + 1];        // V_q[k0 + 1 + i]
+  __shared__ double spart[ROW_WARPS][MAXLOC];
+  __shared__ double st[MAXLOC];             // this block's rows of A22 u
+  __shared__ double sAc[MAXLOC];            // A[r][j + 1]
+  __shared__ double sR[MAXSUM];             // V^T u | W^T u | s1
+  __shared__ double sVn[NB], sWn[NB];       // V_q[j + 1], W_q[j + 1]
+  __shared__ double sa0, sAd, ss2;          // x[j + 1], A[j + 1][j + 1], s2
+  __shared__ double sti[2];                 // tau, inv
+  __shared__ double sc[3];                  // alpha2 = sc[0] + sc[1] s2, w[j + 1] = sc[2] + alpha2
+  const int n = a.n, k0 = a.k0, G = gridDim.x, b = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool direct = G <= DIRECT_G;
+  const int cnt = k0 + b < n ? (n - k0 - b + G - 1) / G : 0;  // rows k0 + b, k0 + b + G, ...
+  if (__syncthreads_or(tid == 0 ? *(volatile int*)a.err & 1 : 0)) return;  // an earlier panel failed
+  // per-row work: eight or four neighbouring threads per row, so that up to 32
+  // rows lie in warps 0-3, one per sub-partition (a float64 instruction takes
+  // 64 clocks of its sub-partition whatever number of its lanes is active)
+  const int lg = cnt <= 16 ? 3 : 2, tpr = 1 << lg;
+  const int rloc = tid >> lg, sub = tid & (tpr - 1);
+  const bool row_warp = tid < ROW_THREADS && ((warp * 32) >> lg) < cnt;
+  const bool has_row = tid < ROW_THREADS && rloc < cnt;
+  const int row = k0 + b + G * rloc;
+  for (int k = tid; k < n + 64; k += ST_THREADS) su[k] = 0.0;
+  if (SA) {
+    for (int loc = warp; loc < cnt; loc += ST_THREADS / 32) {
+      const double* src = a.A + (size_t)(k0 + b + G * loc) * n + k0;
+      for (int k = lane; k < a.sa; k += 32) sA[loc * a.sa + k] = k0 + k < n ? src[k] : 0.0;
+    }
+    __syncthreads();
+  }
+  double xv = 0.0, ac = 0.0;  // x[row] and A[row][j + 1]
+  if (has_row) {
+    xv = a.A[(size_t)k0 * n + row];
+    if (k0 + 1 < n) ac = a.A[(size_t)row * n + k0 + 1];
+  }
   for (int jj = 0; jj < a.nbp; ++jj) {
-    const int j = a.k0 + jj;
-    // ---- A: column j brought up to date with the panel's earlier reflectors
-    // x_r = A[j][r] - sum_q (V_q[r] W_q[j] + W_q[r] V_q[j])
-    {
-      double sq_r = 0.0;
-      if (warp * 8 < cnt) {  // warps without rows keep off the float64 pipe
-        const double x = quad_dot2(&sV[qloc][0], sWs, &sW[qloc][0], sVs, jj, qsub);
-        if (qsub == 0 && qmine && qrow >= j) {
-          const double xv = arow - x;
-          a.col[qrow] = xv;
-          if (qrow == j) a.d[j] = xv;
-          if (qrow >= j + 2) sq_r = xv * xv;
-        }
+    const int j = k0 + jj, NV = 2 * jj + 1;
+    const uint64_t tag = (uint64_t)j + 1;
+    ulonglong2* X = a.X + (size_t)(j & 1) * G * a.lw;
+    ulonglong2* Wn = a.Wn + (j & 1) * NB;
+    ulonglong2* part = a.part + (size_t)(j & 1) * MAXSUM * G;
+    ulonglong2* R = a.R + (j & 1) * MAXSUM * LINE;
+    ulonglong2* T2 = a.T2 + (size_t)(j & 1) * G * LINE;
+    // ---- publish this block's rows of the column, and row j + 1 of W
+    if (has_row && row >= j) {
+      if (sub == 0) {
+        if (jj == 0) put_word(X + b * a.lw + rloc, xv, tag);  // (else published as soon as it was known)
+        if (row == j) a.d[j] = xv;
+        sAc[rloc] = ac;
       }
-      if (qsub == 0) sq[qloc] = sq_r;
+      if (row == j + 1)
+        for (int q = sub; q < jj; q += tpr) put_word(Wn + q, sW[rloc][q], tag);
     }
-    __syncthreads();
-    if (warp == 0) {
-      const double s = warp_sum(sq[lane] + sq[lane + 32]);
-      if (lane == 0) part[P_SSQ] = s;
-    }
-    target += G;
-    if (!grid_barrier(a.bar, target, a.err, &s_ok)) return;
-
-    // ---- B: the reflector (every block the same), v staged in shared memory
-    if (warp == 0) {
-      const double sigma = sum_parts(a.part, G, P_SSQ);
-      if (lane == 0) {
-        double tau = 0.0, inv = 0.0, beta = 0.0;
-        if (j < n - 1) {
-          const double alpha = a.col[j + 1];
-          if (sigma == 0.0) {
-            beta = alpha;  // nothing below the subdiagonal: H = I
-          } else {
-            const double nrm = sqrt(fma(alpha, alpha, sigma));
-            beta = alpha >= 0.0 ? -nrm : nrm;
-            tau = (beta - alpha) / beta;
-            inv = 1.0 / (alpha - beta);
-          }
-          if (b == 0) {
-            a.e[j] = beta;
-            a.tau[j] = tau;
-          }
-        }
-        sc[0] = tau;
-        sc[1] = inv;
+    if (j == n - 1) break;  // the last column has nothing below its diagonal
+    // ---- gather the whole column
+    bool bad = false;
+    for (int w0 = tid; w0 < G * a.lw; w0 += 4 * ST_THREADS) {
+      const ulonglong2* p[4];
+      double v[4];
+      int r[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int w = w0 + i * ST_THREADS, bb = w / a.lw;
+        r[i] = k0 + bb + G * (w - bb * a.lw);
+        p[i] = bb < G && r[i] > j && r[i] < n ? X + w : nullptr;
       }
-    }
-    for (int r = threadIdx.x; r < n; r += ST_THREADS)
-      sv[r] = r > j + 1 ? a.col[r] : (r == j + 1 ? 1.0 : 0.0);
-    __syncthreads();
-    const double tau = sc[0], inv = sc[1];
-    for (int r = j + 2 + threadIdx.x; r < n; r += ST_THREADS) sv[r] *= inv;
-    __syncthreads();
-    // reflector storage (row j of the row-major view) and this block's V rows
-    for (int loc = threadIdx.x; loc < cnt; loc += ST_THREADS) {
-      const int r = b + G * loc;
-      const double v = sv[r];
-      if (r >= j + 2) a.A[(size_t)j * n + r] = v;
-      a.Vp[(size_t)jj * n + r] = v;
-      sV[loc][jj] = v;
-    }
-    // t = A22 v on this block's rows, one warp per row. The row is read from
-    // L2 in 16-byte pairs, eight per lane in flight (the loop is bound by the
-    // latency of these loads, not by the float64 pipe): element j+1 alone when
-    // its address is not 16-byte aligned, then pairs, then a last odd element.
-    if (j < n - 1) {
-      for (int loc = warp; loc < cnt; loc += ST_WARPS) {
-        const int r = b + G * loc;
-        if (r < j + 1) continue;
-        const double* row = a.A + (size_t)r * n;
-        const int k1 = j + 1;
-        const int ka = k1 + (int)((reinterpret_cast<uintptr_t>(row + k1) >> 3) & 1);  // 16-byte aligned
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        if (lane == 0 && ka > k1) s0 = row[k1] * sv[k1];
-        const int np2 = ka < n ? (n - ka) >> 1 : 0;  // pairs (ka + 2p, ka + 2p + 1)
-        const double2* row2 = reinterpret_cast<const double2*>(row + ka);
-        const double* svp = sv + ka;
-        int p = lane;
-        for (; p + 224 < np2; p += 256) {
-          double2 x[8];
+      bad |= !get_words<4>(p, tag, v);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) x[u] = row2[p + 32 * u];
-#pragma unroll
-          for (int u = 0; u < 8; u += 2) {
-            const int k = 2 * (p + 32 * u);
-            s0 = fma(x[u].x, svp[k], s0);
-            s1 = fma(x[u].y, svp[k + 1], s1);
-            s2 = fma(x[u + 1].x, svp[k + 64], s2);
-            s3 = fma(x[u + 1].y, svp[k + 65], s3);
-          }
+      for (int i = 0; i < 4; ++i)
+        if (p[i]) {
+          if (r[i] == j + 1) sa0 = v[i];
+          else su[r[i]] = v[i];
         }
-        for (; p < np2; p += 32) {
-          const double2 x = row2[p];
-          s0 = fma(x.x, svp[2 * p], s0);
-          s1 = fma(x.y, svp[2 * p + 1], s1);
+    }
+    if (tid == 0) su[j + 1] = 0.0;
+    double vpan = 0.0;  // (warp 9) V row of lane's panel row, before scaling
+    if (warp == 9) {
+      const ulonglong2* p[1] = {lane < jj ? Wn + lane : nullptr};
+      double v[1];
+      bad |= !get_words<1>(p, tag, v);
+      sWn[lane] = lane < jj ? v[0] : 0.0;
+      sVn[lane] = lane < jj ? sVp[lane][jj] : 0.0;
+      if (lane == 0) sAd = a.A[(size_t)(j + 1) * n + j + 1];
+    }
+    if (__syncthreads_or(bad)) {
+      if (bad) atomicOr(a.err, 1);
+      return;
+    }
+    const double ur = has_row && row > j + 1 ? su[row] : 0.0;
+    if (warp == 9 && k0 + 1 + lane < n) vpan = su[k0 + 1 + lane];
+    const int loc0 = j + 1 > k0 + b ? (j + 1 - k0 - b + G - 1) / G : 0;  // first row >= j + 1
+    double Cr = 0.0, acn = 0.0;
+    if (tid < ROW_THREADS) {
+      // ---- partial sums over this block's rows, four threads to a sum
+      {
+        const int c = tid >> 2, s4 = tid & 3;
+        double p = 0.0;
+        if (c < NV) {
+          const double* f = c < jj ? &sV[0][c] : c < 2 * jj ? &sW[0][c - jj] : sAc;
+          const int fs = c < 2 * jj ? NB : 1;
+#pragma unroll 4
+          for (int loc = loc0 + s4; loc < cnt; loc += 4) p = fma(f[loc * fs], su[k0 + b + G * loc], p);
         }
-        if (lane == 1 && ka < n && ((n - ka) & 1)) s2 = fma(row[n - 1], sv[n - 1], s2);
-        const double tr = warp_sum((s0 + s1) + (s2 + s3));
-        if (lane == 0) {
-          st[loc] = tr;
-          if (r == j + 1) a.t[r] = tr;
-        }
+        p += __shfl_xor_sync(0xffffffffu, p, 1);
+        p += __shfl_xor_sync(0xffffffffu, p, 2);
+        if (c < NV && s4 == 0) put_word(part + (size_t)b * MAXSUM + c, p, tag);
       }
-    }
-    __syncthreads();
-    // partial y_q = V_q^T v, z_q = W_q^T v (q < jj) and t^T v over this block's rows
-    if (threadIdx.x < 2 * NB + 1) {
-      const int c = threadIdx.x;
-      double p0 = 0.0, p1 = 0.0;
-      if (j < n - 1 && (c == 2 * NB || (c % NB) < jj)) {
-        const int q = c % NB;
-        int loc = 0;
-        for (; loc < cnt; ++loc) {
-          const int r = b + G * loc;
-          if (r < j + 1) continue;
-          const double x = c == 2 * NB ? st[loc] : (c < NB ? sV[loc][q] : sW[loc][q]);
-          if (loc & 1) p1 = fma(x, sv[r], p1);
-          else p0 = fma(x, sv[r], p0);
-        }
-      }
-      part[c] = p0 + p1;
-    }
-    target += G;
-    if (!grid_barrier(a.bar, target, a.err, &s_ok)) return;
-
-    // ---- C: y, z, t^T v summed over the blocks; w on this block's rows
-    // (loads that do not depend on the sums are issued first)
-    double vq_next = 0.0, wq_next = 0.0;  // V_q[j+1], W_q[j+1] for the next column
-    if (warp == 1 && j + 1 < n && lane < jj) {
-      vq_next = a.Vp[(size_t)lane * n + j + 1];
-      wq_next = a.Wp[(size_t)lane * n + j + 1];
-    }
-    arow = load_arow(j + 1);
-    double t_next = 0.0;  // t[j+1], written before the barrier by its owner
-    if (warp == 0 && lane == 0 && j + 1 < n) t_next = a.t[j + 1];
-    {
-      // y_q, z_q: warp w sums coefficients 8w .. 8w+7 (y for w < 4, z after)
-      // over the blocks: lane l loads them (two 16-byte loads per four) from
-      // blocks l, l + 32, ...; the lanes then combine by a butterfly that
-      // halves the live values at each of the first three steps, so lane l
-      // ends with coefficient (l >> 2) & 7 summed over all lanes. Warp 0 also
-      // sums t^T v. Every load is issued before the first addition.
-      const int c0 = 8 * warp;
-      const bool live = j < n - 1 && (c0 % NB) < jj;   // this warp's coefficients
-      const bool with_tv = warp == 0 && j < n - 1;      // t^T v is needed from jj = 0 on
-      if (live || with_tv) {
-        constexpr int MAXB = 5;  // blocks per lane: G <= 160
-        double2 v[MAXB][4];
-        double tvp[MAXB];
-#pragma unroll
-        for (int i = 0; i < MAXB; ++i) {
-          const int bb = lane + 32 * i;
-          const bool ok = bb < G;
-          const double2* src = reinterpret_cast<const double2*>(a.part + (size_t)bb * PW + c0);
-#pragma unroll
-          for (int u = 0; u < 4; ++u) v[i][u] = (ok && live) ? src[u] : make_double2(0.0, 0.0);
-          tvp[i] = (ok && with_tv) ? a.part[(size_t)bb * PW + P_TV] : 0.0;
-        }
+      if (has_row && j + 2 < n)  // the next column's
+        acn = SA ? sA[rloc * a.sa + j + 2 - k0] : a.A[(size_t)row * n + j + 2];
+      // ---- A22 u: each warp takes every eighth chunk of 64 columns for all
+      // rows (so the warps, and the four float64 pipes behind them, have
+      // equal shares), eight rows at a time
+      const int kbeg = (j + 2) & ~1, nch = (n - kbeg + 63) >> 6;
+      for (int g0 = loc0; g0 < cnt; g0 += 8) {
         double acc[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          acc[2 * u] = v[0][u].x;
-          acc[2 * u + 1] = v[0][u].y;
-        }
+        for (int i = 0; i < 8; ++i) acc[i] = 0.0;
+        const double* rp = SA ? sA + g0 * a.sa - k0 : a.A + (size_t)(k0 + b + G * g0) * n;
+        const size_t rs = SA ? (size_t)a.sa : (size_t)G * n;
+        const int rows = cnt - g0;  // (the same for the whole block)
+#pragma unroll 2
+        for (int ch = warp; ch < nch; ch += ROW_WARPS) {
+          const int k = kbeg + 64 * ch + 2 * lane;
+          const double u0 = su[k], u1 = su[k + 1];
+          double2 x[8];
 #pragma unroll
-        for (int i = 1; i < MAXB; ++i)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            acc[2 * u] += v[i][u].x;
-            acc[2 * u + 1] += v[i][u].y;
+          for (int i = 0; i < 8; ++i) {
+            x[i] = make_double2(0.0, 0.0);
+            if (i < rows) {
+              if (VEC || SA) {
+                if (k < n) x[i] = *reinterpret_cast<const double2*>(rp + i * rs + k);
+              } else {
+                if (k < n) x[i].x = rp[i * rs + k];
+                if (k + 1 < n) x[i].y = rp[i * rs + k + 1];
+              }
+            }
           }
-        // butterfly: keep the half of the values selected by the lane bit
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (i < rows) acc[i] = fma(x[i].x, u0, fma(x[i].y, u1, acc[i]));
+        }
+        if (warp >= nch) {  // no columns left for this warp
+          if (lane < 8 && lane < rows) spart[warp][g0 + lane] = 0.0;
+          continue;
+        }
+        // eight sums by a butterfly that halves the live values
+        const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
         double h4[4], h2[2], h1;
-        {
-          const bool up = lane & 16;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const double send = up ? acc[i] : acc[i + 4];
-            const double keep = up ? acc[i + 4] : acc[i];
-            h4[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-          }
-        }
-        {
-          const bool up = lane & 8;
+        for (int i = 0; i < 4; ++i)
+          h4[i] = (b16 ? acc[i + 4] : acc[i]) + __shfl_xor_sync(0xffffffffu, b16 ? acc[i] : acc[i + 4], 16);
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const double send = up ? h4[i] : h4[i + 2];
-            const double keep = up ? h4[i + 2] : h4[i];
-            h2[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-          }
-        }
-        {
-          const bool up = lane & 4;
-          const double send = up ? h2[0] : h2[1];
-          const double keep = up ? h2[1] : h2[0];
-          h1 = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
+        for (int i = 0; i < 2; ++i)
+          h2[i] = (b8 ? h4[i + 2] : h4[i]) + __shfl_xor_sync(0xffffffffu, b8 ? h4[i] : h4[i + 2], 8);
+        h1 = (b4 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, b4 ? h2[0] : h2[1], 4);
         h1 += __shfl_xor_sync(0xffffffffu, h1, 2);
         h1 += __shfl_xor_sync(0xffffffffu, h1, 1);
-        if ((lane & 3) == 0)
-          scoef[c0 + ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0)] = h1;
-        if (with_tv) {
-          double tv = tvp[0];
-#pragma unroll
-          for (int i = 1; i < MAXB; ++i) tv += tvp[i];
-          tv = warp_sum(tv);
-          if (lane == 0) scoef[P_TV] = tv;
+        const int loc = g0 + (b16 ? 4 : 0) + (b8 ? 2 : 0) + (b4 ? 1 : 0);
+        if ((lane & 3) == 0 && loc < cnt) spart[warp][loc] = h1;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(ROW_THREADS) : "memory");
+      if (warp == 0) {
+        double s2 = 0.0;
+        for (int loc = loc0 + lane; loc < cnt; loc += 32) {
+          double t0 = spart[0][loc] + spart[1][loc], t1 = spart[2][loc] + spart[3][loc];
+          t0 += spart[4][loc] + spart[5][loc];
+          t1 += spart[6][loc] + spart[7][loc];
+          st[loc] = t0 + t1;
+          s2 = fma(t0 + t1, su[k0 + b + G * loc], s2);
         }
-      } else {
-        if (lane < 8) scoef[c0 + lane] = 0.0;
-        if (warp == 0 && lane == 0) scoef[P_TV] = 0.0;
+        for (int o = cnt <= 16 ? 8 : 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        if (lane == 0) put_word(T2 + b * LINE, s2, tag);
       }
-      if (warp == 1 && lane < jj) {
-        sVs[lane] = vq_next;
-        sWs[lane] = wq_next;
+      // ---- C_r = sum_q V_q[r] W_q[j+1] + W_q[r] V_q[j+1]
+      if (row_warp) {  // warps without rows keep off the float64 pipe
+        double c2 = 0.0;
+#pragma unroll 4
+        for (int q = sub; q < jj; q += tpr) {
+          Cr = fma(sV[rloc][q], sWn[q], Cr);
+          c2 = fma(sW[rloc][q], sVn[q], c2);
+        }
+        Cr += c2;
+        for (int o = tpr >> 1; o > 0; o >>= 1) Cr += __shfl_xor_sync(0xffffffffu, Cr, o);
+      }
+      if (direct && warp >= 4) {  // all sums from the partial sums, two threads to a sum
+        const int c = (tid - 128) >> 1, s2 = tid & 1;
+        double p = 0.0;
+        for (int b0 = s2; b0 < G; b0 += 16) {
+          const ulonglong2* w[8];
+          double v[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) w[i] = c < NV && b0 + 2 * i < G ? part + (size_t)(b0 + 2 * i) * MAXSUM + c : nullptr;
+          bad |= !get_words<8>(w, tag, v);
+          p += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+        }
+        p += __shfl_xor_sync(0xffffffffu, p, 1);
+        if (s2 == 0) sR[c] = p;
+      }
+    } else if (warp == 8) {
+      if (!direct)  // this block's sums, added up for everybody
+        for (int c = b; c < NV; c += G) {
+          const ulonglong2* w[5];
+          double v[5];
+#pragma unroll
+          for (int i = 0; i < 5; ++i) w[i] = lane + 32 * i < G ? part + (size_t)(lane + 32 * i) * MAXSUM + c : nullptr;
+          bad |= !get_words<5>(w, tag, v);
+          const double s = warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + v[4]);
+          if (lane == 0) put_word(R + c * LINE, s, tag);
+        }
+    } else {
+      // sigma from this block's own copy of u, and what follows from it
+      double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
+      for (int r = j + 2 + lane; r < n; r += 128) {  // (su is zero past n; 64 entries of it exist)
+        const double x0 = su[r], x1 = r + 32 < n ? su[r + 32] : 0.0, x2 = r + 64 < n ? su[r + 64] : 0.0,
+                     x3 = r + 96 < n ? su[r + 96] : 0.0;
+        q0 = fma(x0, x0, q0);
+        q1 = fma(x1, x1, q1);
+        q2 = fma(x2, x2, q2);
+        q3 = fma(x3, x3, q3);
+      }
+      const double sigma = warp_sum((q0 + q1) + (q2 + q3)), a0 = sa0;
+      double tau = 0.0, inv = 0.0, beta = a0;  // sigma = 0: nothing below the subdiagonal, H = I
+      if (sigma != 0.0) {
+        const double q = fma(a0, a0, sigma), rn = rsqrt(q), nrm = q * rn;
+        if (nrm > 0.0 && rn < 1e308) {  // |beta| = nrm, tau = 1 + |a0| / nrm: one division on the way
+          beta = a0 >= 0.0 ? -nrm : nrm;
+          tau = fma(fabs(a0), rn, 1.0);
+        } else {  // out of range of the reciprocal root, or not finite
+          const double root = sqrt(q);
+          beta = a0 >= 0.0 ? -root : root;
+          tau = (beta - a0) / beta;
+        }
+        inv = 1.0 / (a0 - beta);
+      }
+      if (lane == 0) {
+        sti[0] = tau;
+        sti[1] = inv;
+        if (b == 0) {
+          a.e[j] = beta;
+          a.tau[j] = tau;
+        }
+      }
+      // row jj of V on the panel's rows (k0 + 1 + lane)
+      const int r = k0 + 1 + lane;
+      sVp[jj][lane] = r == j + 1 ? 1.0 : r > j + 1 ? inv * vpan : 0.0;
+    }
+    if (warp == 9 && !direct) {
+      const ulonglong2* w[2] = {lane < NV ? R + lane * LINE : nullptr,
+                                lane + 32 < NV ? R + (lane + 32) * LINE : nullptr};
+      double v[2];
+      bad |= !get_words<2>(w, tag, v);
+      sR[lane] = v[0];
+      sR[lane + 32] = v[1];
+    }
+    if (__syncthreads_or(bad)) {
+      if (bad) atomicOr(a.err, 1);
+      return;
+    }
+    // ---- D_r = sum_q W_q[r] (V^T u)_q + V_q[r] (W^T u)_q on the row threads,
+    // s2 on warp 8, the scalars on warp 9
+    const double tau = sti[0], inv = sti[1];
+    double v = 0.0, B = 0.0, E = 0.0;  // w = B + alpha2 v, the next column's entry E - v w[j+1] - w
+    if (tid < ROW_THREADS) {
+      if (row_warp) {
+        double d1 = 0.0, d2 = 0.0;
+#pragma unroll 4
+        for (int q = sub; q < jj; q += tpr) {
+          d1 = fma(sW[rloc][q], sR[q], d1);
+          d2 = fma(sV[rloc][q], sR[jj + q], d2);
+        }
+        d1 += d2;
+        for (int o = tpr >> 1; o > 0; o >>= 1) d1 += __shfl_xor_sync(0xffffffffu, d1, o);
+        if (has_row && sub == 0) {
+          E = ac - Cr;
+          if (row == j + 1) {
+            v = 1.0;
+          } else if (row > j + 1) {
+            v = inv * ur;
+            B = tau * fma(inv, st[rloc] - d1, E);
+          }
+        }
+      }
+    } else if (warp == 8) {
+      const ulonglong2* w[5];
+      double x[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) w[i] = lane + 32 * i < G ? T2 + (lane + 32 * i) * LINE : nullptr;
+      bad |= !get_words<5>(w, tag, x);
+      const double s = direct ? warp_sum(x[0]) : warp_sum(((x[0] + x[1]) + (x[2] + x[3])) + x[4]);
+      if (lane == 0) ss2 = s;
+    } else {
+      const double s1 = sR[2 * jj], vn = sVn[lane], wn = sWn[lane];
+      const double y = lane < jj ? fma(inv, sR[lane], vn) : 0.0;
+      const double z = lane < jj ? fma(inv, sR[jj + lane], wn) : 0.0;
+      // sum of y z (lower half-warp) and of w_n y + v_n z (upper) together
+      const double p = y * z, q = fma(wn, y, vn * z);
+      const bool up = lane & 16;
+      double h = (up ? q : p) + __shfl_xor_sync(0xffffffffu, up ? p : q, 16);
+      for (int o = 8; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+      const double yz = __shfl_sync(0xffffffffu, h, 0), sj = __shfl_sync(0xffffffffu, h, 16);
+      const double at = fma(inv, s1, sAd), f = -0.5 * tau * tau;
+      if (lane == 0) {
+        sc[0] = f * fma(-2.0, yz, fma(inv, s1, at));
+        sc[1] = f * (inv * inv);
+        sc[2] = tau * (at - sj);
       }
     }
-    __syncthreads();
-    if (warp == 0) {
-      // alpha2 = -(tau/2) tau (t^T v - 2 y^T z)
-      double yz = lane < jj ? scoef[lane] * scoef[NB + lane] : 0.0;
-      yz = warp_sum(yz);
-      if (lane == 0) sc[2] = -0.5 * tau * (tau * (scoef[P_TV] - 2.0 * yz));
-    } else if (warp == 1) {
-      // the quad sum of row j+1 exactly as its owner's quad forms it below
-      const double x = quad_dot2(sWs, scoef, sVs, scoef + NB, jj, lane & 3);
-      if (lane == 0) sc[3] = x;
+    if (__syncthreads_or(bad)) {
+      if (bad) atomicOr(a.err, 1);
+      return;
     }
-    __syncthreads();
-    const double alpha2 = sc[2];
-    if (threadIdx.x == 0 && j + 1 < n) {  // the next column's V_jj[j+1], W_jj[j+1]
-      sVs[jj] = 1.0;
-      sWs[jj] = j < n - 1 ? fma(tau, t_next - sc[3], alpha2) : 0.0;
+    // ---- v, w and the next column on this block's rows
+    if (has_row && sub == 0) {
+      const double alpha2 = fma(sc[1], ss2, sc[0]), w1 = sc[2] + alpha2;
+      double w = 0.0;
+      if (row == j + 1) w = w1;
+      else if (row > j + 1) w = fma(alpha2, v, B);
+      xv = fma(-v, w1, E - w);
+      sV[rloc][jj] = v;
+      sW[rloc][jj] = w;
+      // (published before the slower stores below)
+      if (row >= j + 1 && jj + 1 < a.nbp) put_word(a.X + ((size_t)((j + 1) & 1) * G + b) * a.lw + rloc, xv, tag + 1);
+      if (row > j + 1) a.A[(size_t)j * n + row] = v;
+      a.Vp[(size_t)jj * n + row] = v;
+      a.Wp[(size_t)jj * n + row] = w;
     }
-    if (warp * 8 < cnt) {
-      const double x = quad_dot2(&sW[qloc][0], scoef, &sV[qloc][0], scoef + NB, jj, qsub);
-      if (qsub == 0 && qmine) {
-        double w = 0.0;
-        if (j < n - 1 && qrow >= j + 1) w = fma(tau, st[qloc] - x, alpha2 * sv[qrow]);
-        sW[qloc][jj] = w;
-        a.Wp[(size_t)jj * n + qrow] = w;
-      }
-    }
-    __syncthreads();  // sv, sc and the shared scalars are rewritten by the next column
+    ac = acn;
+    __syncwarp();  // (the row's other threads read this column's w when they publish its row)
   }
 }
 
@@ -405,40 +464,57 @@ osmps_status sytrd_tc(osmps_ctx* ctx, double* A, int64_t n, double* d, double* e
                       cudaStream_t s) {
   osmps_status st = OSMPS_OK;
   if (!sytrd_supported(n)) return set_error(OSMPS_EUNSUPPORTED, "sytrd: n=%lld", (long long)n);
-  const size_t smem = (size_t)n * 8;
-  static const cudaError_t cfg = cudaFuncSetAttribute(
-      k_sytrd_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * 8);
-  OSMPS_CUDA(cfg);
+  const size_t smem = (size_t)((n + 64 + 1) & ~(int64_t)1) * 8;
+  const bool vec = n % 2 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;  // 16-byte rows
+  const auto in_l2 = vec ? k_sytrd_panel<true, false> : k_sytrd_panel<false, false>;
+  const auto in_smem = k_sytrd_panel<false, true>;
+  // dynamic shared memory beside the kernels' 48 KB
+  constexpr size_t SMEM_MOST = (size_t)(227 - 48) * 1024;
+  OSMPS_CUDA(cudaFuncSetAttribute(in_l2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MOST));
+  OSMPS_CUDA(cudaFuncSetAttribute(in_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MOST));
   int per_sm = 0;
-  OSMPS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sytrd_panel, ST_THREADS, smem));
+  OSMPS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, in_smem, ST_THREADS, SMEM_MOST));
   if (per_sm < 1) return set_error(OSMPS_EUNSUPPORTED, "sytrd: panel kernel does not fit an SM");
-  // about 8 rows per block, at most one block per SM (all blocks co-resident)
-  const int G = (int)std::max<int64_t>(
-      1, std::min<int64_t>(std::min<int64_t>(ctx->sm_count, 160), cdiv(n, 8)));
-  if (cdiv(n, G) > MAXLOC)
+  // Blocks of a panel with m trailing rows: about 8 rows each, at most one
+  // block per SM (all co-resident). Up to SMALL_M rows, no more than DIRECT_G:
+  // the product A22 v (m^2 / 64 clocks on 32 SMs, 2.3 us at 544) costs less
+  // there than the second exchange of the sums (line at 768: n = 1024 9.3
+  // instead of 8.0 us a column, n = 768 9.8 instead of 8.0).
+  constexpr int64_t SMALL_M = 544;
+  const auto blocks_for = [&](int64_t m) {
+    const int64_t most = m <= SMALL_M ? (m <= 256 ? DIRECT_G / 2 : DIRECT_G) : 160;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(ctx->sm_count, most), cdiv(m, 8)));
+  };
+  const int Gmax = (int)std::max<int64_t>(std::min<int64_t>(ctx->sm_count, 160), DIRECT_G);
+  if (cdiv(n, blocks_for(n)) > MAXLOC)
     return set_error(OSMPS_EUNSUPPORTED, "sytrd: n=%lld needs more than %d rows per block",
                      (long long)n, MAXLOC);
-  double* buf = (double*)ws_get(ctx, SLOT_TRD, (size_t)(2 * NB * n + 2 * n + (size_t)G * PW +
-                                                        2 * n * 2 * NB + 64) * 8, s, &st);
+  // panel vectors, GEMM operands, then the tagged words (cleared: tags start at 1)
+  const size_t xwords = (size_t)n + (size_t)LINE * Gmax;  // rows of every block rounded up to lines
+  const size_t words = 2 * xwords + 2 * NB + 2 * (size_t)MAXSUM * Gmax + 2 * MAXSUM * LINE + 2 * (size_t)Gmax * LINE;
+  const size_t vecs = (size_t)(2 * NB * n + 2 * n * 2 * NB);
+  double* buf = (double*)ws_get(ctx, SLOT_TRD, (vecs + 2 * words + 64) * 8, s, &st);
   if (!buf) return st;
   double* Vp = buf;
   double* Wp = Vp + NB * n;
-  double* col = Wp + NB * n;
-  double* t = col + n;
-  double* part = t + n;
-  double* X = part + (size_t)G * PW;
+  double* X = Wp + NB * n;
   double* Y = X + 2 * NB * n;
-  unsigned* bar = reinterpret_cast<unsigned*>(ctx->dev_flags + 8);
+  ulonglong2* word = reinterpret_cast<ulonglong2*>(buf + vecs);
+  OSMPS_CUDA(cudaMemsetAsync(word, 0, words * sizeof(ulonglong2), s));
   int* err = ctx->dev_flags + 3;
-  OSMPS_CUDA(cudaMemsetAsync(bar, 0, sizeof(unsigned), s));
-  unsigned base = 0;
   for (int64_t k0 = 0; k0 < n; k0 += NB) {
     const int nbp = (int)std::min<int64_t>(NB, n - k0);
+    const int G = blocks_for(n - k0);
     SytrdArgs a;
     a.A = A; a.n = (int)n; a.k0 = (int)k0; a.nbp = nbp;
     a.d = d; a.e = e; a.tau = tau; a.Vp = Vp; a.Wp = Wp;
-    a.col = col; a.t = t; a.part = part;
-    a.bar = bar; a.bar_base = base; a.err = err;
+    a.X = word; a.Wn = a.X + 2 * xwords; a.part = a.Wn + 2 * NB; a.R = a.part + 2 * (size_t)MAXSUM * Gmax;
+    a.T2 = a.R + 2 * MAXSUM * LINE; a.err = err;
+    const int64_t rows = cdiv(n - k0, G);
+    a.lw = (int)round_up(rows, LINE);
+    const int64_t stride = round_up(n - k0, 2);
+    const size_t with_rows = smem + (size_t)(rows * stride) * 8;
+    a.sa = with_rows <= SMEM_MOST ? (int)stride : 0;
     void* args[] = {&a};
     // algorithmic float64 work of the panel: per column j (i columns of the
     // panel before it, m = n - j - 1 trailing rows) the product A22 v
@@ -449,11 +525,10 @@ osmps_status sytrd_tc(osmps_ctx* ctx, double* A, int64_t n, double* d, double* e
       pf += 2.0 * mm * mm + 8.0 * mm * i;
     }
     const int ph = prof_begin(s);
-    OSMPS_CUDA(cudaLaunchCooperativeKernel((void*)k_sytrd_panel, dim3(G), dim3(ST_THREADS), args,
-                                           smem, s));
+    OSMPS_CUDA(cudaLaunchCooperativeKernel((void*)(a.sa ? in_smem : in_l2), dim3(G), dim3(ST_THREADS), args,
+                                           a.sa ? with_rows : smem, s));
     note_launch();
     prof_end(ph, s, OSMPS_KERNEL_SYTRD_PANEL, pf, 0.0);
-    base += 2u * (unsigned)nbp * (unsigned)G;
     const int64_t k = k0 + nbp, m = n - k;
     if (m <= 0) break;
     { k_pack_vw<<<grid_1d(m * 2 * NB), 256, 0, s>>>(Vp, Wp, n, k, m, nbp, X, Y); note_launch(); }
@@ -484,7 +559,7 @@ extern "C" osmps_status osmps_sytrd(osmps_ctx* ctx, double* A, int64_t n, double
   OSMPS_CUDA(cudaStreamSynchronize(s));
   if (flag) {
     cudaMemsetAsync(ctx->dev_flags + 3, 0, sizeof(int), s);
-    return set_error(OSMPS_ETIMEOUT, "osmps_sytrd: a grid barrier wait gave up");
+    return set_error(OSMPS_ETIMEOUT, "osmps_sytrd: a wait of the panel reduction gave up");
   }
   return OSMPS_OK;
 }
