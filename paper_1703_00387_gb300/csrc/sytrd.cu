@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
   __shared__ double sVn[NB], sWn[NB];       // V_q[j + 1], W_q[j + 1]
   __shared__ double sa0, sAd, ss2;          // x[j + 1], A[j + 1][j + 1], s2
   __shared__ double sti[2];                 // tau, inv
+  __shared__ int sE[2];                     // largest biased exponent of the column, by parity
   __shared__ double sc[3];                  // alpha2 = sc[0] + sc[1] s2, w[j + 1] = sc[2] + alpha2
   const int n = a.n, k0 = a.k0, G = gridDim.x, b = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -124,6 +125,8 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
   const bool has_row = tid < ROW_THREADS && rloc < cnt;
   const int row = k0 + b + G * rloc;
   for (int k = tid; k < n + 64; k += ST_THREADS) su[k] = 0.0;
+  if (tid < 2) sE[tid] = 0;
+  __syncthreads();
   if (SA) {
     for (int loc = warp; loc < cnt; loc += ST_THREADS / 32) {
       const double* src = a.A + (size_t)(k0 + b + G * loc) * n + k0;
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
     if (j == n - 1) break;  // the last column has nothing below its diagonal
     // ---- gather the whole column
     bool bad = false;
+    int em = 0;
     for (int w0 = tid; w0 < G * a.lw; w0 += 4 * ST_THREADS) {
       const ulonglong2* p[4];
       double v[4];
@@ -171,11 +175,14 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (p[i]) {
+          em = max(em, (__double2hiint(v[i]) >> 20) & 0x7FF);
           if (r[i] == j + 1) sa0 = v[i];
           else su[r[i]] = v[i];
         }
     }
     if (tid == 0) su[j + 1] = 0.0;
+    em = __reduce_max_sync(0xffffffffu, em);
+    if (lane == 0) atomicMax(&sE[j & 1], em);
     double vpan = 0.0;  // (warp 9) V row of lane's panel row, before scaling
     if (warp == 9) {
       const ulonglong2* p[1] = {lane < jj ? Wn + lane : nullptr};
@@ -189,6 +196,17 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
       if (bad) atomicOr(a.err, 1);
       return;
     }
+    // u is not scaled, so s2 holds |A| |u|^2: a column far from 1 is brought
+    // there by a power of two (v, tau and everything below stay as they are,
+    // inv absorbs it, beta gets it back)
+    const int ex = sE[j & 1] - 1023;
+    const bool scaled = (ex > 100 || ex < -200) && ex > -1023 && ex < 1024;  // the same in every block
+    if (scaled) {
+      for (int r = j + 2 + tid; r < n; r += ST_THREADS) su[r] = scalbn(su[r], -ex);
+      if (tid == 0) sa0 = scalbn(sa0, -ex);
+      __syncthreads();
+    }
+    if (tid == 0) sE[(j + 1) & 1] = 0;
     const double ur = has_row && row > j + 1 ? su[row] : 0.0;
     if (warp == 9 && k0 + 1 + lane < n) vpan = su[k0 + 1 + lane];
     const int loc0 = j + 1 > k0 + b ? (j + 1 - k0 - b + G - 1) / G : 0;  // first row >= j + 1
@@ -339,7 +357,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
         sti[0] = tau;
         sti[1] = inv;
         if (b == 0) {
-          a.e[j] = beta;
+          a.e[j] = scaled ? scalbn(beta, ex) : beta;
           a.tau[j] = tau;
         }
       }
