@@ -113,6 +113,7 @@ enum Slot {
   SLOT_CX_R,
   SLOT_CX_THETA,
   SLOT_HEFF_IDDEV,
+  SLOT_EMU_PART,
   SLOT_COUNT
 };
 

@@ -16,24 +16,32 @@
 //     i + j (same unit 2^(-7(i+j+2))), over the 36 pairs with i + j <= 7
 //     (the dropped pairs are below 2^-56 of the row scales);
 //   * pairs on one diagonal share the unit, so a TMEM partial sum runs over
-//     up to 16 K blocks of 64 across the pairs of a diagonal (at K = 64 the
-//     36 pairs take 8 epilogue rounds, not 36);
-//   * the diagonals are combined exactly in int64, Horner fashion in steps
-//     of 2^7, within groups of consecutive diagonals (two groups of four
-//     while K <= 2^17, whose sums stay below 2^53); each group sum becomes
+//     several K blocks of 64 and all pairs of its diagonal: 16 block products
+//     on diagonal 0, 32 on the others;
+//   * the diagonals are taken in groups of four (two while K > 2^17), one TMEM
+//     accumulator of 128 columns each. Their partial sums are combined exactly
+//     in int64 at weights 2^7 apart and stay below 2^53; a group sum becomes
 //     a float64 by integer operations on the IEEE bits, the row and column
 //     scales 2^(e_A + e_B) folded into its exponent, and the group values
-//     are added in float64 in a second TMEM region. One float64 addition per
-//     output element and tile remains: GB300's float64 pipe is what limits
-//     this kind of kernel otherwise. The result is stored, or subtracted
-//     from C.
-// The kernel reuses the persistent, warp-specialised structure of gemm_tc:
-// 128 x 128 tiles, a 6-stage TMA ring, two 128-column TMEM buffers, 16
-// epilogue warps each holding 32 float64 accumulators per row.
+//     are added in float64. One float64 addition per output element and group
+//     after the first remains: GB300's float64 pipe is what limits this kind
+//     of kernel otherwise. The result is stored, or subtracted from C.
+// What bounds it: the MMAs, 64 clocks per 128 x 128 x 16. A group walks K once
+// and forms all its pairs from one copy of the slices in shared memory: 24
+// slice tiles per K block and output tile where a pass over K for each pair
+// took 72, which the 60 bytes per clock that an SM takes in from L2 allowed one
+// pair in 570 clocks; now 380, the rest being the single issuing warp and the
+// drains. 2048 x 2048 x 2048: kernel 764 -> 481 us (1280 TFLOP/s of bf16), 2560 x
+// 2048 x 512: 348 -> 211, 2048 x 512 x 2560 with K in shares: 475 -> 178, 381 x 1905
+// x 1000: 201 -> 74.
+// The kernel is persistent and warp-specialised: a TMA producer with a ring
+// of 13 slice tiles, a warp that issues the MMAs, and 16 epilogue warps each
+// holding 32 exact sums per row in registers.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "tcgen05.cuh"
@@ -47,26 +55,37 @@ using namespace tc;
 constexpr int SLICES = 8;
 constexpr int SLICE_BITS = 7;
 constexpr int EBM = 128, EBN = 128;
-constexpr int ESTAGES = 6;
-constexpr int E_A_STAGE = EBM * 128, E_B_STAGE = EBN * 128;
-constexpr int E_STAGE = E_A_STAGE + E_B_STAGE;
+constexpr int E_SLOTS = 13;                // ring of 128-row, 64-element slice tiles
+constexpr int E_TILE = 128 * 128;          // bytes of one
+constexpr int E_BUFS = 4;                  // TMEM accumulators: one per diagonal of a group
 constexpr int E_EPI_WARPS = 16;
 constexpr int E_EPI_COLS = EBN / 4;
 constexpr int E_THREADS = 64 + 32 * E_EPI_WARPS;
-// 64-element K slices per exact partial sum: products are at most 2^14 (the
-// pair of top digits, |d_0| <= 128), so 16 slices (1024 products) stay
-// within 2^24. (Diagonals other than 0 could run 32 slices, their products
-// being at most 2^13; measured slightly slower, the epilogue then drains in
-// longer, fewer bursts.)
-constexpr int E_CHUNK = 16;
-constexpr uint32_t E_TMEM_COLS = 512;   // 2 x 128 accumulator columns, then the float64 sums
-constexpr uint32_t E_ACC_COL0 = 256;    // float64 group sums: two 32-bit columns per tile column
-constexpr size_t E_SMEM = (size_t)ESTAGES * E_STAGE + 1024 + 256;
+constexpr uint32_t E_TMEM_COLS = E_BUFS * EBN;
+constexpr size_t E_SMEM = (size_t)E_SLOTS * E_TILE + 1024 + 512;
+static_assert(EBM == 128 && EBN == 128 && E_SMEM <= 227 * 1024, "slice tile ring");
 
-struct PairList {
-  int n;
-  unsigned char a[64], b[64];
-};
+// 64-element K blocks per exact partial sum of diagonal d, whose d + 1 pairs
+// share one accumulator: digit products are at most 2^14 in size on diagonal 0
+// (|d_0| <= 128) and 2^13 on the others, so 16 and 32 of their 64-term sums
+// stay within 2^24.
+__host__ __device__ constexpr int chunk_blocks(int d) { return d == 0 ? 16 : 32 / (d + 1); }
+// the same as bytes of a word (a division costs the drains more than a shift)
+constexpr uint64_t chunk_bytes() {
+  uint64_t w = 0;
+  for (int d = 0; d < SLICES; ++d) w |= (uint64_t)chunk_blocks(d) << (8 * d);
+  return w;
+}
+
+// The slices' order of arrival within a K block of diagonals d0..d1: first
+// A_d1 .. A_d0 and B_0, then before each further b the slice A_(d0-b), if
+// there is one, and B_b. Position in that order:
+__host__ __device__ constexpr int a_pos(int a, int d0, int d1) {
+  return a >= d0 ? d1 - a : d1 - d0 + 2 * (d0 - a);
+}
+__host__ __device__ constexpr int b_pos(int b, int d0, int d1) {
+  return d1 - d0 + 1 + (b <= d0 ? 2 * b : d0 + b);
+}
 
 // x 2^k as a float64 for an integer |x| < 2^53, built from the IEEE-754 bit
 // layout (sign, biased exponent, 52 fraction bits) with integer operations
@@ -85,7 +104,7 @@ __device__ __forceinline__ double i64_ldexp(long long x, int k) {
 // Tile t -> (m0, n0) in groups of E_GROUP_M tile rows, columns walked within
 // a group: the tiles that run at the same time then share E_GROUP_M A row
 // slabs and fewer B column slabs than a row-major walk, so more of the slice
-// operands stay in L2 between the pairs' passes.
+// operands stay in L2.
 constexpr int E_GROUP_M = 8;
 __device__ __forceinline__ void emu_tile(int tile, int tiles_m, int tiles_n, int& m0, int& n0) {
   const int per_group = E_GROUP_M * tiles_n;
@@ -96,71 +115,163 @@ __device__ __forceinline__ void emu_tile(int tile, int tiles_m, int tiles_n, int
   n0 = (local / rows) * EBN;
 }
 
-// Close a diagonal group of the epilogue: its sums H (the last diagonal `cur`
-// at weight 1) become float64 with the scales folded in and are added to the
-// float64 sums of the earlier groups kept in TMEM (acc_t); after the last
-// group the total is stored to C (or subtracted from it). H is zeroed.
-__device__ __forceinline__ void close_group(long long (&H)[E_EPI_COLS], int& groups, bool last,
-                                            uint32_t acc_t, int cur, int ea,
-                                            const int* __restrict__ eB, int64_t col0, int64_t N,
-                                            int64_t row, int64_t M, double* __restrict__ C,
-                                            int64_t ldc, int subtract) {
-  const int k0 = -SLICE_BITS * (cur + 2) + ea;
+// Four float64 values of a row, at columns c .. c+3 of N; two per access where
+// `vec` says that rows and base are 16-byte aligned.
+__device__ __forceinline__ void load_row4(const double* p, int64_t c, int64_t N, int vec, double (&v)[4]) {
+  if (vec && c + 4 <= N) {
 #pragma unroll
-  for (int h = 0; h < E_EPI_COLS / 8; ++h) {  // 8 values = 16 TMEM words at a time
-    uint32_t w[16];
-    if (groups > 0) tmem_ld16(acc_t + 16 * h, w);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = 8 * h + i;
-      const int eb = (col0 + j < N) ? eB[col0 + j] : 0;
-      double v = i64_ldexp(H[j], k0 + eb);
-      if (groups > 0) v += __hiloint2double((int)w[2 * i + 1], (int)w[2 * i]);
-      if (last) {
-        if (row < M && col0 + j < N) {
-          double* dst = C + row * ldc + col0 + j;
-          if (subtract) *dst -= v;
-          else *dst = v;
-        }
-      } else {
-        w[2 * i] = (uint32_t)__double2loint(v);
-        w[2 * i + 1] = (uint32_t)__double2hiint(v);
-      }
-      H[j] = 0;
+    for (int i = 0; i < 4; i += 2) {
+      const double2 t = *reinterpret_cast<const double2*>(p + c + i);
+      v[i] = t.x;
+      v[i + 1] = t.y;
     }
-    if (!last) tmem_st16(acc_t + 16 * h, w);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = c + i < N ? p[c + i] : 0.0;
   }
-  if (!last) tmem_st_wait();
-  ++groups;
+}
+__device__ __forceinline__ void store_row4(double* p, int64_t c, int64_t N, int vec, const double (&v)[4]) {
+  if (vec && c + 4 <= N) {
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) *reinterpret_cast<double2*>(p + c + i) = make_double2(v[i], v[i + 1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (c + i < N) p[c + i] = v[i];
+  }
 }
 
+// What the kernel writes: C[r][c] (subtract: C -= the product), rows of ldc
+// values, two per access where `vec`; share s of K writes at s * slab. G holds
+// the sums of the diagonal groups before the last, in an order of the threads'
+// own (128 KB for each CTA, [column pair][thread], so that a warp's accesses
+// are whole lines: in C itself they took a line for each lane).
+struct EmuOut {
+  double* C;
+  double2* G;
+  int64_t ldc, slab;
+  int subtract, vec;
+};
+
+// Warp-wide forms: the whole warp runs the issuing loop, one elected thread
+// issues. The loop's values are then uniform and stay in uniform registers,
+// where the instruction wants its operands.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+__device__ __forceinline__ void umma_elect(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
+                                           uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(id), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_elect(uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+
+// The MMA issuer's place in the ring: slot and phase of the next K block's
+// first slice; blocks in each buffer's partial sum, and the buffers' phases.
+struct EmuIssue {
+  uint32_t slot = 0, phase = 0, used = 0;
+  int count[E_BUFS] = {};
+};
+
+// Issue the pairs of diagonals D0 .. D0 + GD - 1 over one K block, B slice by
+// B slice; false when a wait ran out. One thread issues everything, at one
+// instruction per several clocks, and has 256 clocks per pair: positions in the
+// ring and partial-sum lengths are constants of the unrolled loops (computed,
+// they cost 1040 clocks a pair).
+template <int D0, int GD>
+__device__ __forceinline__ bool emu_issue_block(EmuIssue& st, uint32_t ring, uint32_t tmem,
+                                                uint64_t* full, uint64_t* empty, uint64_t* tfull,
+                                                uint64_t* tempty, bool last_block) {
+  constexpr int D1 = D0 + GD - 1;
+  const uint32_t id = idesc<TC_BF16, EBM, EBN>();
+  const uint64_t desc0 = sdesc(ring);
+  const auto slot_of = [&](int pos) {
+    const uint32_t t = st.slot + (uint32_t)pos;  // at most 12 + 16
+    return t >= 2 * E_SLOTS ? t - 2 * E_SLOTS : t >= E_SLOTS ? t - E_SLOTS : t;
+  };
+  const auto phase_of = [&](int pos) {
+    const uint32_t t = st.slot + (uint32_t)pos;
+    return st.phase ^ (t >= 2 * E_SLOTS ? 0u : t >= E_SLOTS ? 1u : 0u);
+  };
+#pragma unroll
+  for (int b = 0; b <= D1; ++b) {
+    // the slices that this b is the first to use: in order of arrival they end with B_b
+    const int from = b == 0 ? 0 : b_pos(b - 1, D0, D1) + 1;
+    const int to = b_pos(b, D0, D1);
+#pragma unroll
+    for (int p = 0; p <= GD; ++p)
+      if (from + p <= to && !mbar_wait_warp(&full[slot_of(from + p)], phase_of(from + p))) return false;
+    tc_fence_after();
+    const uint32_t sb = slot_of(to);
+    const uint64_t bd = desc0 + (uint64_t)(sb * (E_TILE >> 4));
+#pragma unroll
+    for (int d = (D0 > b ? D0 : b); d <= D1; ++d) {
+      const int buf = d - D0;
+      const bool first = b == 0 && st.count[buf] == 0;
+      if (first) {
+        if (!mbar_wait_warp(&tempty[buf], ((st.used >> buf) & 1u) ^ 1u)) return false;
+        st.used ^= 1u << buf;
+        tc_fence_after();
+      }
+      const uint64_t ad = desc0 + (uint64_t)(slot_of(a_pos(d - b, D0, D1)) * (E_TILE >> 4));
+      const uint32_t dt = tmem + (uint32_t)(buf * EBN);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        umma_elect(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
+      if (d == b) {  // a = 0: the diagonal's last pair
+        if (++st.count[buf] == chunk_blocks(d) || last_block) {
+          umma_commit_elect(&tfull[buf]);
+          st.count[buf] = 0;
+        }
+      }
+    }
+    // A_(D1-b) and B_b were used for the last time
+    umma_commit_elect(&empty[slot_of(a_pos(D1 - b, D0, D1))]);
+    umma_commit_elect(&empty[sb]);
+  }
+  constexpr uint32_t LOADS = 2 * (D1 + 1);
+  const uint32_t phase = phase_of(LOADS);
+  st.slot = slot_of(LOADS);
+  st.phase = phase;
+  return true;
+}
+
+template <int GD>
 __global__ void __launch_bounds__(E_THREADS, 1)
     k_gemm_emu(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               double* __restrict__ C, int64_t M, int64_t N, int64_t ldc, int nkb, int Kp,
-               int tiles_n, int n_tiles, const int* __restrict__ eA, const int* __restrict__ eB,
-               const __grid_constant__ PairList pl, int* __restrict__ err, int subtract,
-               int group_diags) {
+               const __grid_constant__ EmuOut out, int64_t M, int64_t N, int nkb, int Kp, int tiles_n,
+               int n_tiles, int splits, const int* __restrict__ eA, const int* __restrict__ eB,
+               int* __restrict__ err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + ESTAGES * E_A_STAGE;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + ESTAGES * E_STAGE);
-  uint64_t* empty = full + ESTAGES;
-  uint64_t* tfull = empty + ESTAGES;
-  uint64_t* tempty = tfull + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + E_SLOTS * E_TILE);
+  uint64_t* empty = full + E_SLOTS;
+  uint64_t* tfull = empty + E_SLOTS;
+  uint64_t* tempty = tfull + E_BUFS;
+  uint64_t* done = tempty + E_BUFS;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < ESTAGES; ++s) {
+    for (int s = 0; s < E_SLOTS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < E_BUFS; ++b) {
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], E_EPI_WARPS);
     }
+    mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -173,138 +284,158 @@ __global__ void __launch_bounds__(E_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int npairs = pl.n;
-  // the K block kb of pair q is the last of its TMEM partial sum when the
-  // sum holds E_CHUNK blocks or the next block belongs to another diagonal
-  auto chunk_ends = [&](int q, int kb, int inchunk) {
-    return inchunk == E_CHUNK ||
-           (kb == nkb - 1 && (q == npairs - 1 || pl.a[q + 1] + pl.b[q + 1] != pl.a[q] + pl.b[q]));
+  // work item -> output tile and its share [kb0, kb1) of the K blocks
+  const auto item_of = [&](int item, int& m0, int& n0, int& kb0, int& kb1) {
+    const int tile = item / splits, s = item - tile * splits;
+    emu_tile(tile, n_tiles / tiles_n, tiles_n, m0, n0);
+    kb0 = (int)((int64_t)nkb * s / splits);
+    kb1 = (int)((int64_t)nkb * (s + 1) / splits);
+    return s;
   };
+  const int n_items = n_tiles * splits;
 
   if (warp == 0 && lane == 0) {
-    uint32_t g = 0, issued = 0;
+    uint32_t g = 0, s = 0, phase = 1;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-      int m0, n0;
-      emu_tile(tile, n_tiles / tiles_n, tiles_n, m0, n0);
-      for (int q = 0; q < npairs && ok; ++q) {
-        const int xa = pl.a[q] * Kp, xb = pl.b[q] * Kp;
-        for (int kb = 0; kb < nkb; ++kb, ++g) {
-          const int s = g % ESTAGES;
-          if (!mbar_wait(&empty[s], ((g / ESTAGES) & 1u) ^ 1u)) {
-            ok = false;
-            break;
-          }
-          mbar_expect_tx(&full[s], E_STAGE);
-          tma_load_2d(sA + s * E_A_STAGE, &tmA, xa + kb * 64, m0, &full[s]);
-          tma_load_2d(sB + s * E_B_STAGE, &tmB, xb + kb * 64, n0, &full[s]);
-          issued = g + 1;
-        }
+    const auto load = [&](const CUtensorMap* map, int x, int y) {
+      if (!ok || !mbar_wait(&empty[s], phase)) {
+        ok = false;
+        return;
       }
-    }
-    if (!ok) atomicOr(err, 1);
-    for (uint32_t q = (issued > ESTAGES ? issued - ESTAGES : 0); q < issued; ++q)
-      if (!mbar_wait(&full[q % ESTAGES], (q / ESTAGES) & 1u)) atomicOr(err, 1);
-  } else if (warp == 1 && lane == 0) {
-    const uint32_t id = idesc<TC_BF16, EBM, EBN>();
-    uint32_t g = 0, gc = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-      int inchunk = 0;
-      for (int q = 0; q < npairs && ok; ++q) {
-        for (int kb = 0; kb < nkb && ok; ++kb, ++g) {
-          const bool first = inchunk == 0;
-          const uint32_t buf = gc & 1u;
-          if (first) {
-            if (!mbar_wait(&tempty[buf], ((gc >> 1) & 1u) ^ 1u)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-          }
-          const int s = g % ESTAGES;
-          if (!mbar_wait(&full[s], (g / ESTAGES) & 1u)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint64_t ad = sdesc(smem_u32(sA + s * E_A_STAGE));
-          const uint64_t bd = sdesc(smem_u32(sB + s * E_B_STAGE));
-          const uint32_t dt = tmem + buf * (uint32_t)EBN;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            umma<TC_BF16>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
-          umma_commit(&empty[s]);
-          if (chunk_ends(q, kb, ++inchunk)) {
-            umma_commit(&tfull[buf]);
-            ++gc;
-            inchunk = 0;
+      mbar_expect_tx(&full[s], E_TILE);
+      tma_load_2d(smem + s * E_TILE, map, x, y, &full[s]);
+      ++g;
+      if (++s == E_SLOTS) {
+        s = 0;
+        phase ^= 1u;
+      }
+    };
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      int m0, n0, kb0, kb1;
+      item_of(item, m0, n0, kb0, kb1);
+      for (int d0 = 0; d0 < SLICES && ok; d0 += GD) {
+        const int d1 = d0 + GD - 1;
+        for (int kb = kb0; kb < kb1 && ok; ++kb) {
+          for (int a = d1; a > d0; --a) load(&tmA, a * Kp + kb * 64, m0);
+          for (int b = 0; b <= d1; ++b) {
+            if (b <= d0) load(&tmA, (d0 - b) * Kp + kb * 64, m0);
+            load(&tmB, b * Kp + kb * 64, n0);
           }
         }
       }
     }
     if (!ok) atomicOr(err, 1);
-    if (gc > 0 && !mbar_wait(&tfull[(gc - 1) & 1u], ((gc - 1) >> 1) & 1u)) atomicOr(err, 1);
+    for (uint32_t q = (g > E_SLOTS ? g - E_SLOTS : 0); q < g; ++q)
+      if (!mbar_wait(&full[q % E_SLOTS], (q / E_SLOTS) & 1u)) atomicOr(err, 1);
+  } else if (warp == 1) {
+    EmuIssue st;
+    const uint32_t ring = smem_u32(smem);
+    bool ok = true;
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      int m0, n0, kb0, kb1;
+      item_of(item, m0, n0, kb0, kb1);
+      const auto group = [&](auto d0) {
+        for (int kb = kb0; kb < kb1 && ok; ++kb)
+          ok = emu_issue_block<decltype(d0)::value, GD>(st, ring, tmem, full, empty, tfull, tempty,
+                                                        kb == kb1 - 1);
+      };
+      group(std::integral_constant<int, 0>());
+      if constexpr (GD == 2) group(std::integral_constant<int, 2>());
+      group(std::integral_constant<int, 4>());
+      if constexpr (GD == 2) group(std::integral_constant<int, 6>());
+    }
+    umma_commit_elect(done);
+    ok = mbar_wait_warp(done, 0) && ok;
+    if (!ok && lane == 0) atomicOr(err, 1);
   } else if (warp >= 2) {
     const int qd = warp & 3;
     const int part = (warp - 2) >> 2;
-    // this thread's float64 group sums: TMEM lane of its row, two columns per value
-    const uint32_t acc_t = tmem + ((uint32_t)(qd * 32) << 16) + E_ACC_COL0 + part * 2 * E_EPI_COLS;
-    uint32_t gc = 0;
+    const uint32_t lane_t = tmem + ((uint32_t)(qd * 32) << 16) + part * E_EPI_COLS;
+    uint32_t used = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-      int m0, n0;
-      emu_tile(tile, n_tiles / tiles_n, tiles_n, m0, n0);
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      int m0, n0, kb0, kb1;
+      const int64_t off = (int64_t)item_of(item, m0, n0, kb0, kb1) * out.slab;
       const int64_t row = (int64_t)m0 + qd * 32 + lane;
       const int64_t col0 = (int64_t)n0 + part * E_EPI_COLS;
-      const int ea = row < M ? eA[row] : 0;
-      long long H[E_EPI_COLS];  // exact group sum, the current diagonal at weight 1
+      for (int d0 = 0; d0 < SLICES && ok; d0 += GD) {
+        const int d1 = d0 + GD - 1;
+        long long H[E_EPI_COLS];  // exact group sum, diagonal d1 at weight 1
 #pragma unroll
-      for (int j = 0; j < E_EPI_COLS; ++j) H[j] = 0;
-      int cur = pl.a[0] + pl.b[0];
-      int inchunk = 0, groups = 0;
-      for (int q = 0; q < npairs && ok; ++q) {
-        const int diag = pl.a[q] + pl.b[q];
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-          if (!chunk_ends(q, kb, ++inchunk)) continue;
-          inchunk = 0;
-          if (diag != cur) {
-            if (diag / group_diags != cur / group_diags) {
-              close_group(H, groups, false, acc_t, cur, ea, eB, col0, N, row, M, C, ldc,
-                          subtract);
+        for (int j = 0; j < E_EPI_COLS; ++j) H[j] = 0;
+        uint32_t count = 0;  // blocks in each buffer's partial sum, a byte each
+        for (int kb = kb0; kb < kb1 && ok; ++kb) {
+          for (int d = d0; d <= d1; ++d) {
+            const int buf = d - d0;
+            count += 1u << (8 * buf);
+            if (((count >> (8 * buf)) & 255u) != ((uint32_t)(chunk_bytes() >> (8 * d)) & 255u) &&
+                kb != kb1 - 1)
+              continue;
+            count &= ~(255u << (8 * buf));
+            if (!mbar_wait(&tfull[buf], (used >> buf) & 1u)) {
+              ok = false;
+              break;
+            }
+            used ^= 1u << buf;
+            tc_fence_after();
+            const int weight = 1 << (SLICE_BITS * (d1 - d));
+#pragma unroll
+            for (int j = 0; j < E_EPI_COLS / 16; ++j) {
+              uint32_t r[16];
+              tmem_ld16(lane_t + buf * EBN + 16 * j, r);
+              if (j == E_EPI_COLS / 16 - 1) {
+                // the words are in registers: the buffer may be written again
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[buf]);
+              }
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                // an exact integer of magnitude <= 2^24: converted exactly
+                H[16 * j + i] += (long long)__float2int_rn(__uint_as_float(r[i])) * weight;
+              }
+            }
+          }
+        }
+        if (!ok) break;
+        // close the group: its sums become float64 with the scales folded in,
+        // added to those of the groups before
+        if (row < M) {
+          const bool final = d1 == SLICES - 1;
+          const int k0 = -SLICE_BITS * (d1 + 2) + eA[row];
+          double* c = out.C + off + row * out.ldc;
+          double2* g = out.G + (size_t)blockIdx.x * (EBM * EBN / 2) + (threadIdx.x - 64);
+#pragma unroll
+          for (int h = 0; h < E_EPI_COLS / 4; ++h) {
+            const int64_t col = col0 + 4 * h;
+            const int4 eb = *reinterpret_cast<const int4*>(eB + col);
+            double v[4], t[4];
+            double2* gh = g + 2 * h * (32 * E_EPI_WARPS);
+            v[0] = i64_ldexp(H[4 * h], k0 + eb.x);
+            v[1] = i64_ldexp(H[4 * h + 1], k0 + eb.y);
+            v[2] = i64_ldexp(H[4 * h + 2], k0 + eb.z);
+            v[3] = i64_ldexp(H[4 * h + 3], k0 + eb.w);
+            if (d0 > 0) {
+              const double2 x = gh[0], y = gh[32 * E_EPI_WARPS];
+              v[0] += x.x;
+              v[1] += x.y;
+              v[2] += y.x;
+              v[3] += y.y;
+            }
+            if (!final) {
+              gh[0] = make_double2(v[0], v[1]);
+              gh[32 * E_EPI_WARPS] = make_double2(v[2], v[3]);
             } else {
-              const int sh = SLICE_BITS * (diag - cur);
+              if (out.subtract) {
+                load_row4(c, col, N, out.vec, t);
 #pragma unroll
-              for (int j = 0; j < E_EPI_COLS; ++j) H[j] <<= sh;
-            }
-            cur = diag;
-          }
-          const uint32_t buf = gc & 1u;
-          if (!mbar_wait(&tfull[buf], (gc >> 1) & 1u)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t base =
-              tmem + ((uint32_t)(qd * 32) << 16) + buf * (uint32_t)EBN + part * E_EPI_COLS;
-#pragma unroll
-          for (int j = 0; j < E_EPI_COLS / 16; ++j) {
-            uint32_t r[16];
-            tmem_ld16(base + 16 * j, r);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              // an exact integer of magnitude <= 2^24: converted exactly
-              H[16 * j + i] += (long long)__float2int_rn(__uint_as_float(r[i]));
+                for (int i = 0; i < 4; ++i) v[i] = t[i] - v[i];
+              }
+              store_row4(c, col, N, out.vec, v);
             }
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty[buf]);
-          ++gc;
         }
       }
-      if (!ok) break;
-      close_group(H, groups, true, acc_t, cur, ea, eB, col0, N, row, M, C, ldc, subtract);
     }
     if (!ok) atomicOr(err, 1);
   }
@@ -314,6 +445,18 @@ __global__ void __launch_bounds__(E_THREADS, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(E_TMEM_COLS));
+  }
+}
+
+// C = sum of the partial products (or C -= it), its slabs in order.
+__global__ void k_emu_combine(const double* __restrict__ P, int splits, int64_t slab, int64_t ldp,
+                              int64_t N, double* __restrict__ C, int64_t ldc, int subtract) {
+  const int64_t r = blockIdx.y;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < N; c += (int64_t)gridDim.x * blockDim.x) {
+    double t = 0.0;
+    for (int s = 0; s < splits; ++s) t += P[s * slab + r * ldp + c];
+    double* dst = C + r * ldc + c;
+    *dst = subtract ? *dst - t : t;
   }
 }
 
@@ -517,16 +660,26 @@ osmps_status slice_operand(osmps_ctx* ctx, const SplitView& v, int64_t Kp, int* 
   return OSMPS_OK;
 }
 
-PairList make_pairs() {
-  PairList pl{};
-  pl.n = 0;
-  for (int sum = 0; sum < SLICES; ++sum)
-    for (int i = 0; i <= sum; ++i) {
-      pl.a[pl.n] = (unsigned char)i;
-      pl.b[pl.n] = (unsigned char)(sum - i);
-      ++pl.n;
+// Shares of K per output tile. A tile takes its K blocks one after the other
+// on one SM, so a product of few tiles leaves SMs idle; its K blocks are then
+// shared out, the partial products going to slabs that are added in order.
+// Taken by estimated clocks: 36 slice pairs of about 300 per K block, 8000 per
+// tile for its drains and sums, and for the slabs 2600 bytes a clock and
+// one launch. With one share 512 x 512 x 2048 took 381 us and 1024 x 1024 x 2048
+// 385 (a pass over K per pair), with eight and two shares 64 and 150.
+int emu_splits(int64_t M, int64_t N, int64_t n_tiles, int64_t nkb, int sms) {
+  if (M > 65535) return 1;
+  int best = 1;
+  double t_best = 0;
+  for (int s = 1; s <= 8 && (s == 1 || nkb / s >= 2); ++s) {
+    double t = (double)cdiv(n_tiles * s, sms) * ((double)cdiv(nkb, s) * 36 * 300 + 8000);
+    if (s > 1) t += (double)s * M * N * 16 / 2600 + 6000;
+    if (s == 1 || t < t_best) {
+      best = s;
+      t_best = t;
     }
-  return pl;
+  }
+  return best;
 }
 
 }  // namespace
@@ -538,8 +691,9 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   if (K <= 0 || a.rows != M || b.rows != N || a.K != K || b.K != K)
     return set_error(OSMPS_ESHAPE, "gemm_emu: inconsistent operand views");
   // Small products go to the float64 DMMA kernel, which is float64-accurate
-  // too: the emulation costs about 56 us even for one tile (slicing passes,
-  // 36 slice pairs), so whatever the DMMA kernel finishes sooner runs there.
+  // too: the emulation costs 52 to 62 us even for a few tiles (three launches,
+  // 36 slice pairs; 128x128x64: 53, 300x300x340: 62), so whatever the DMMA
+  // kernel finishes sooner runs there.
   if (small_on_dmma && a.n1 == 1 && b.n1 == 1 && !a.src_f32 && !b.src_f32 && gemm_f64_us(M, N, K) < 56.0) {
     GemmF64 g;
     g.M = M; g.N = N; g.K = K;
@@ -560,7 +714,7 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   if (!sa) return st;
   auto* sb = (__nv_bfloat16*)ws_get(ctx, SLOT_EMU_B, (size_t)N * SLICES * Kp * 2, s, &st);
   if (!sb) return st;
-  int* ex = (int*)ws_get(ctx, SLOT_EMU_EXP, (size_t)(M + N + 64) * sizeof(int), s, &st);
+  int* ex = (int*)ws_get(ctx, SLOT_EMU_EXP, (size_t)(M + N + 64 + EBN) * sizeof(int), s, &st);
   if (!ex) return st;
   int* eA = ex;
   int* eB = ex + ((M + 63) / 64) * 64;
@@ -569,28 +723,50 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   CUtensorMap ma, mb;
   OSMPS_TRY(tc_make_map(&ma, sa, TC_BF16, M, SLICES * Kp, EBM));
   OSMPS_TRY(tc_make_map(&mb, sb, TC_BF16, N, SLICES * Kp, EBN));
-  // thread-safe one-time setup (function-local static initialisation)
-  static const cudaError_t configured =
-      cudaFuncSetAttribute(k_gemm_emu, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)E_SMEM);
-  OSMPS_CUDA(configured);
-  static const PairList pl = make_pairs();
   const int tiles_n = (int)cdiv(N, EBN);
   const int n_tiles = tiles_n * (int)cdiv(M, EBM);
-  const int grid = std::min(n_tiles, ctx->sm_count);
   const int nkb = (int)(Kp / 64);
+  const int splits = emu_splits(M, N, n_tiles, nkb, ctx->sm_count);
+  const int grid = std::min(n_tiles * splits, ctx->sm_count);
+  EmuOut out{C, nullptr, ldc, 0, subtract && splits == 1 ? 1 : 0, 0};
+  if (splits > 1) {
+    out.ldc = round_up(N, 2);
+    out.slab = M * out.ldc;
+  }
+  auto* scratch = (double*)ws_get(ctx, SLOT_EMU_PART,
+                                  ((size_t)grid * EBM * EBN + (splits > 1 ? (size_t)splits * out.slab : 0)) * 8, s, &st);
+  if (!scratch) return st;
+  out.G = reinterpret_cast<double2*>(scratch);
+  if (splits > 1) out.C = scratch + (size_t)grid * EBM * EBN;
+  out.vec = (reinterpret_cast<uintptr_t>(out.C) & 15) == 0 && out.ldc % 2 == 0;
   // diagonals per exact int64 group: four while a group sum stays below 2^53
   // (|I_d| < (d + 1) K 2^14 with slice digits of at most 2^7 and 2^6), else two
-  const int group_diags = Kp <= ((int64_t)1 << 17) ? 4 : 2;
+  const auto run = [&](auto kernel, cudaError_t configured) -> osmps_status {
+    OSMPS_CUDA(configured);
+    kernel<<<grid, E_THREADS, E_SMEM, s>>>(ma, mb, out, M, N, nkb, (int)Kp, tiles_n, n_tiles, splits, eA, eB,
+                                           ctx->dev_flags);
+    note_launch();
+    return OSMPS_OK;
+  };
   const int ph = prof_begin(s);
-  {
-    k_gemm_emu<<<grid, E_THREADS, E_SMEM, s>>>(ma, mb, C, M, N, ldc, nkb, (int)Kp, tiles_n,
-                                               n_tiles, eA, eB, pl, ctx->dev_flags,
-                                               subtract ? 1 : 0, group_diags);
+  // thread-safe one-time setups (function-local static initialisation)
+  if (Kp <= ((int64_t)1 << 17)) {
+    static const cudaError_t configured =
+        cudaFuncSetAttribute(k_gemm_emu<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)E_SMEM);
+    OSMPS_TRY(run(k_gemm_emu<4>, configured));
+  } else {
+    static const cudaError_t configured =
+        cudaFuncSetAttribute(k_gemm_emu<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)E_SMEM);
+    OSMPS_TRY(run(k_gemm_emu<2>, configured));
+  }
+  if (splits > 1) {
+    const dim3 cg((unsigned)std::min<int64_t>(cdiv(N, 256), 64), (unsigned)M);
+    k_emu_combine<<<cg, 256, 0, s>>>(out.C, splits, out.slab, out.ldc, N, C, ldc, subtract ? 1 : 0);
     note_launch();
   }
   OSMPS_LAUNCH_CHECK();
   const double logical = 2.0 * (double)M * (double)N * (double)K;
-  prof_end(ph, s, OSMPS_KERNEL_GEMM_EMU, logical, (double)pl.n * logical);
+  prof_end(ph, s, OSMPS_KERNEL_GEMM_EMU, logical, (double)(SLICES * (SLICES + 1) / 2) * logical);
   return OSMPS_OK;
 }
 
