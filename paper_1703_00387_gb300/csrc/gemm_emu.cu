@@ -153,28 +153,6 @@ struct EmuOut {
   int subtract, vec;
 };
 
-// Warp-wide forms: the whole warp runs the issuing loop, one elected thread
-// issues. The loop's values are then uniform and stay in uniform registers,
-// where the instruction wants its operands.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
-}
-__device__ __forceinline__ void umma_elect(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t id,
-                                           uint32_t accumulate) {
-  asm volatile(
-      "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
-      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(id), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit_elect(uint64_t* bar) {
-  asm volatile(
-      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
-
 // The MMA issuer's place in the ring: slot and phase of the next K block's
 // first slice; blocks in each buffer's partial sum, and the buffers' phases.
 struct EmuIssue {
@@ -226,7 +204,7 @@ __device__ __forceinline__ bool emu_issue_block(EmuIssue& st, uint32_t ring, uin
       const uint32_t dt = tmem + (uint32_t)(buf * EBN);
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        umma_elect(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
+        umma_elect<TC_BF16>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
       if (d == b) {  // a = 0: the diagonal's last pair
         if (++st.count[buf] == chunk_blocks(d) || last_block) {
           umma_commit_elect(&tfull[buf]);
@@ -660,6 +638,11 @@ osmps_status slice_operand(osmps_ctx* ctx, const SplitView& v, int64_t Kp, int* 
   return OSMPS_OK;
 }
 
+// Tiles of partial products at most, per SM: the scratch of the kernel then has
+// one size for all products and never grows after the first (a growing one
+// would be refused inside a graph capture).
+constexpr int E_SLAB_WAVES = 2;
+
 // Shares of K per output tile. A tile takes its K blocks one after the other
 // on one SM, so a product of few tiles leaves SMs idle; its K blocks are then
 // shared out, the partial products going to slabs that are added in order.
@@ -671,7 +654,7 @@ int emu_splits(int64_t M, int64_t N, int64_t n_tiles, int64_t nkb, int sms) {
   if (M > 65535) return 1;
   int best = 1;
   double t_best = 0;
-  for (int s = 1; s <= 8 && (s == 1 || nkb / s >= 2); ++s) {
+  for (int s = 1; s <= 8 && (s == 1 || (nkb / s >= 2 && n_tiles * s <= E_SLAB_WAVES * sms)); ++s) {
     double t = (double)cdiv(n_tiles * s, sms) * ((double)cdiv(nkb, s) * 36 * 300 + 8000);
     if (s > 1) t += (double)s * M * N * 16 / 2600 + 6000;
     if (s == 1 || t < t_best) {
@@ -733,11 +716,11 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
     out.ldc = round_up(N, 2);
     out.slab = M * out.ldc;
   }
-  auto* scratch = (double*)ws_get(ctx, SLOT_EMU_PART,
-                                  ((size_t)grid * EBM * EBN + (splits > 1 ? (size_t)splits * out.slab : 0)) * 8, s, &st);
+  const size_t tile_sums = (size_t)ctx->sm_count * EBM * EBN;
+  auto* scratch = (double*)ws_get(ctx, SLOT_EMU_PART, (1 + E_SLAB_WAVES) * tile_sums * 8, s, &st);
   if (!scratch) return st;
   out.G = reinterpret_cast<double2*>(scratch);
-  if (splits > 1) out.C = scratch + (size_t)grid * EBM * EBN;
+  if (splits > 1) out.C = scratch + tile_sums;
   out.vec = (reinterpret_cast<uintptr_t>(out.C) & 15) == 0 && out.ldc % 2 == 0;
   // diagonals per exact int64 group: four while a group sum stays below 2^53
   // (|I_d| < (d + 1) K 2^14 with slice digits of at most 2^7 and 2^6), else two

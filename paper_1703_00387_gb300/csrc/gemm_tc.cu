@@ -193,18 +193,21 @@ __global__ void __launch_bounds__(THREADS, 1)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sA = smem;
   uint8_t* sB = smem + STAGES * A_STAGE;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* tfull = empty + STAGES;   // 2: chunk in TMEM buffer ready
+  // ring of DEPTH K blocks, each with the hi and lo tiles of A and B
+  constexpr int DEPTH = STAGES / 2;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);  // hi tiles have landed
+  uint64_t* full_lo = full + DEPTH;                                           // lo tiles
+  uint64_t* empty = full_lo + DEPTH;     // A hi and B lo read by their last MMA
+  uint64_t* empty_x = empty + DEPTH;     // A lo and B hi
+  uint64_t* tfull = empty_x + DEPTH;  // 2: chunk in TMEM buffer ready
   uint64_t* tempty = tfull + 2;       // 2: TMEM buffer drained by the epilogue
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  uint64_t* done = tempty + 2;        // every MMA of this CTA
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
+    for (int s = 0; s < 4 * DEPTH; ++s) mbar_init(&full[s], 1);
+    mbar_init(done, 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], EPI_WARPS);
@@ -223,70 +226,95 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    // Producer. Slice it of a tile covers K slice kb = it / 3 of product
-    // p = it % 3: p = 0 (hi, hi), 1 (hi, lo), 2 (lo, hi).
-    uint32_t g = 0;  // slices issued by this CTA (ring position)
-    uint32_t issued = 0;
+    // Producer: A hi and B hi of a K block, then its lo tiles. B lo is free one
+    // product before B hi, so the next hi tile takes the slot of the lo tile
+    // that was there and the next lo tile that of the hi tile.
+    uint32_t hi = 0, lo = 0;  // K blocks whose hi / lo tiles were requested
+    uint32_t x = 0, round = 0;  // place in the ring, parity of the turns round it
     bool ok = true;
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       const TileJob job = tile_job<OUT, BN>(tile, C, M, N, ldc, nkb, tiles_n, probs, n_prob);
-      const int total = 3 * job.nkb;  // K slices over the three products
-      for (int it = 0; it < total; ++it, ++g) {
-        const int s = g % STAGES;
-        const uint32_t ph = (g / STAGES) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u)) {
+      for (int kb = 0; kb < job.nkb; ++kb) {
+        const int k = kb * kelem;
+        const uint32_t bh = 2 * x + round, bl = bh ^ 1u;
+        if (!mbar_wait(&empty[x], round ^ 1u)) {
           ok = false;
           break;
         }
-        const int kb = it / 3, p = it % 3;
-        mbar_expect_tx(&full[s], STAGE_BYTES);
-        tma_load_2d(sA + s * A_STAGE, &tmA, kb * kelem + (p == 2 ? Kp : 0), job.a_row, &full[s]);
-        tma_load_2d(sB + s * B_STAGE, &tmB, kb * kelem + (p == 1 ? Kp : 0), job.b_row, &full[s]);
-        issued = g + 1;
+        mbar_expect_tx(&full[x], STAGE_BYTES);
+        tma_load_2d(sA + 2 * x * A_STAGE, &tmA, k, job.a_row, &full[x]);
+        tma_load_2d(sB + bh * B_STAGE, &tmB, k, job.b_row, &full[x]);
+        ++hi;
+        if (!mbar_wait(&empty_x[x], round ^ 1u)) {
+          ok = false;
+          break;
+        }
+        mbar_expect_tx(&full_lo[x], STAGE_BYTES);
+        tma_load_2d(sB + bl * B_STAGE, &tmB, k + Kp, job.b_row, &full_lo[x]);
+        tma_load_2d(sA + (2 * x + 1) * A_STAGE, &tmA, k + Kp, job.a_row, &full_lo[x]);
+        ++lo;
+        if (++x == DEPTH) {
+          x = 0;
+          round ^= 1u;
+        }
       }
     }
     if (!ok) atomicOr(err, 1);
-    // Drain: the last copy issued into each stage has landed before exit.
-    for (uint32_t q = (issued > STAGES ? issued - STAGES : 0); q < issued; ++q)
-      if (!mbar_wait(&full[q % STAGES], (q / STAGES) & 1u)) atomicOr(err, 1);
-  } else if (warp == 1 && lane == 0) {
+    // Drain: the last copies issued into each place have landed before exit.
+    for (uint32_t q = (hi > DEPTH ? hi - DEPTH : 0); q < hi; ++q)
+      if (!mbar_wait(&full[q % DEPTH], (q / DEPTH) & 1u)) atomicOr(err, 1);
+    for (uint32_t q = (lo > DEPTH ? lo - DEPTH : 0); q < lo; ++q)
+      if (!mbar_wait(&full_lo[q % DEPTH], (q / DEPTH) & 1u)) atomicOr(err, 1);
+  } else if (warp == 1) {
     const uint32_t id = idesc<KIND, BM, BN>();
-    uint32_t g = 0, gc = 0;  // slices / chunks consumed by this CTA
+    const uint64_t descA = sdesc(smem_u32(sA)), descB = sdesc(smem_u32(sB));
+    uint32_t gc = 0;            // chunks issued by this CTA
+    uint32_t x = 0, round = 0;  // as in the producer
     bool ok = true;
     for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
       const int total = 3 * tile_job<OUT, BN>(tile, C, M, N, ldc, nkb, tiles_n, probs, n_prob).nkb;
-      for (int it = 0; it < total && ok; ++it, ++g) {
-        const bool first = (it % CHUNK) == 0;
-        const uint32_t buf = gc & 1u;
-        if (first) {
-          if (!mbar_wait(&tempty[buf], ((gc >> 1) & 1u) ^ 1u)) {
+      int in_chunk = 0;
+      // K slice it of a tile is block kb = it / 3 of product p = it % 3:
+      // p = 0 (hi, hi), 1 (hi, lo), 2 (lo, hi)
+      for (int it = 0; it < total && ok;) {
+        const uint32_t bh = 2 * x + round;
+#pragma unroll
+        for (int p = 0; p < 3; ++p, ++it) {
+          const bool first = in_chunk == 0;
+          const uint32_t buf = gc & 1u;
+          if (first && !mbar_wait_warp(&tempty[buf], ((gc >> 1) & 1u) ^ 1u)) {
+            ok = false;
+            break;
+          }
+          if (p < 2 && !mbar_wait_warp(p == 0 ? &full[x] : &full_lo[x], round)) {
             ok = false;
             break;
           }
           tc_fence_after();
-        }
-        const int s = g % STAGES;
-        if (!mbar_wait(&full[s], (g / STAGES) & 1u)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint64_t ad = sdesc(smem_u32(sA + s * A_STAGE));
-        const uint64_t bd = sdesc(smem_u32(sB + s * B_STAGE));
-        const uint32_t dt = tmem + buf * (uint32_t)BN;
+          const uint64_t ad = descA + (uint64_t)((2 * x + (p == 2 ? 1u : 0u)) * (A_STAGE >> 4));
+          const uint64_t bd = descB + (uint64_t)((p == 1 ? bh ^ 1u : bh) * (B_STAGE >> 4));
+          const uint32_t dt = tmem + buf * (uint32_t)BN;
 #pragma unroll
-        for (int k = 0; k < KSLICE_BYTES / 32; ++k)  // 32 bytes of K per MMA: +2 in the address field
-          umma<KIND>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
-        umma_commit(&empty[s]);
-        if ((it % CHUNK) == CHUNK - 1 || it == total - 1) {
-          umma_commit(&tfull[buf]);
-          ++gc;
+          for (int k = 0; k < KSLICE_BYTES / 32; ++k)  // 32 bytes of K per MMA: +2 in the address field
+            umma_elect<KIND>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
+          if (p == 1) umma_commit_elect(&empty[x]);
+          if (p == 2) umma_commit_elect(&empty_x[x]);
+          if (++in_chunk == CHUNK || it == total - 1) {
+            umma_commit_elect(&tfull[buf]);
+            in_chunk = 0;
+            ++gc;
+          }
+        }
+        if (++x == DEPTH) {
+          x = 0;
+          round ^= 1u;
         }
       }
     }
-    if (!ok) atomicOr(err, 1);
-    // No MMA may still be running when TMEM is released: wait for the last chunk.
-    if (gc > 0 && !mbar_wait(&tfull[(gc - 1) & 1u], ((gc - 1) >> 1) & 1u)) atomicOr(err, 1);
+    // No MMA may still be running when TMEM is released.
+    umma_commit_elect(done);
+    ok = mbar_wait_warp(done, 0) && ok;
+    if (!ok && lane == 0) atomicOr(err, 1);
   } else if (warp >= 2) {
     const int q = warp & 3;                 // TMEM lane quarter this warp may access
     const int part = (warp - 2) >> 2;       // which 64-column quarter of the tile
