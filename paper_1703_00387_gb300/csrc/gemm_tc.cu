@@ -10,14 +10,22 @@
 // each, so a product is just a K-range of the same two TMA tensors.
 //
 // Kernel structure (persistent, 128 x 256 output tiles, 576 threads):
-//   warp 0, one lane : TMA producer, 4-stage ring of 128B-swizzled tiles
-//   warp 1           : allocates all 512 TMEM columns; one lane issues the
-//                      MMAs (M=128, N=256, 4 instructions per 128-byte K slice),
-//                      commits each stage back to the producer and each
-//                      16-MMA partial sum to the epilogue
+//   warp 0, one lane : TMA producer, ring of 128B-swizzled tiles: per 128-byte
+//                      K block the hi and lo tiles of A and B, each loaded once
+//                      for the block's three products
+//   warp 1           : allocates all 512 TMEM columns; issues the MMAs (M=128,
+//                      N=256, 4 instructions per 128-byte K slice) through one
+//                      elected lane, commits the tiles back to the producer
+//                      after their last product and each 16-MMA partial sum
+//                      to the epilogue
 //   warps 2..17      : epilogue, TMEM partial sums -> float32 registers
 //                      (round-to-nearest adds) -> shared-memory staging ->
 //                      row-contiguous global stores (f32 or f64)
+// What bounds it: the tiles' way from L2 into the SM, about 60 bytes per clock
+// (a K block of 96 KB takes 1600 clocks, its 12 MMAs 1536). With the hi tiles
+// loaded again for the second and third product it was 144 KB: chi = 1024 XXZ
+// product in bf16x3 325 -> 291 us, AKLT 301 x 257 in tf32x3 275 -> 225, left
+// environment update at chi = 1024 264 -> 240.
 // Every mbarrier wait is bounded by %globaltimer (2 s); on expiry the kernel
 // records bit 0 in the context's error flag, drains its own copies (bounded),
 // frees TMEM and returns.
