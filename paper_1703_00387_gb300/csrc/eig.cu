@@ -6,8 +6,8 @@
 //      on a cooperative kernel, trailing updates on the emulated GEMM; cuSOLVER
 //      dsytrd above n = 8192).
 //   2. The wanted eigenvalues of T by multisection on Sturm counts (sign
-//      changes of the leading principal minors of T - x I), eight points per
-//      eigenvalue on eight lanes: float32 counts on T / ||T|| narrow the
+//      changes of the leading principal minors of T - x I), sixteen points per
+//      eigenvalue on sixteen lanes: float32 counts on T / ||T|| narrow the
 //      bracket to ~1e-5 ||T||; the padded bracket is checked at both ends
 //      with float64 counts (the Gershgorin interval again if the check
 //      fails) and narrowed to eps ||T|| with float64 counts.
