@@ -204,17 +204,17 @@ __device__ __forceinline__ bool emu_issue_block(EmuIssue& st, uint32_t ring, uin
       const uint32_t dt = tmem + (uint32_t)(buf * EBN);
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        umma_elect<TC_BF16>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
+        umma<TC_BF16>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
       if (d == b) {  // a = 0: the diagonal's last pair
         if (++st.count[buf] == chunk_blocks(d) || last_block) {
-          umma_commit_elect(&tfull[buf]);
+          umma_commit(&tfull[buf]);
           st.count[buf] = 0;
         }
       }
     }
     // A_(D1-b) and B_b were used for the last time
-    umma_commit_elect(&empty[slot_of(a_pos(D1 - b, D0, D1))]);
-    umma_commit_elect(&empty[sb]);
+    umma_commit(&empty[slot_of(a_pos(D1 - b, D0, D1))]);
+    umma_commit(&empty[sb]);
   }
   constexpr uint32_t LOADS = 2 * (D1 + 1);
   const uint32_t phase = phase_of(LOADS);
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(E_THREADS, 1)
       group(std::integral_constant<int, 4>());
       if constexpr (GD == 2) group(std::integral_constant<int, 6>());
     }
-    umma_commit_elect(done);
+    umma_commit(done);
     ok = mbar_wait_warp(done, 0) && ok;
     if (!ok && lane == 0) atomicOr(err, 1);
   } else if (warp >= 2) {

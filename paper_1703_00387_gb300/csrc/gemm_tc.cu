@@ -304,11 +304,11 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t dt = tmem + buf * (uint32_t)BN;
 #pragma unroll
           for (int k = 0; k < KSLICE_BYTES / 32; ++k)  // 32 bytes of K per MMA: +2 in the address field
-            umma_elect<KIND>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
-          if (p == 1) umma_commit_elect(&empty[x]);
-          if (p == 2) umma_commit_elect(&empty_x[x]);
+            umma<KIND>(dt, ad + 2u * k, bd + 2u * k, id, (!first || k > 0) ? 1u : 0u);
+          if (p == 1) umma_commit(&empty[x]);
+          if (p == 2) umma_commit(&empty_x[x]);
           if (++in_chunk == CHUNK || it == total - 1) {
-            umma_commit_elect(&tfull[buf]);
+            umma_commit(&tfull[buf]);
             in_chunk = 0;
             ++gc;
           }
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
     // No MMA may still be running when TMEM is released.
-    umma_commit_elect(done);
+    umma_commit(done);
     ok = mbar_wait_warp(done, 0) && ok;
     if (!ok && lane == 0) atomicOr(err, 1);
   } else if (warp >= 2) {
