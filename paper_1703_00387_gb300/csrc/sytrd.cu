@@ -83,6 +83,7 @@ struct SytrdArgs {
   ulonglong2* R;     // [2][MAXSUM][LINE] sums (G > DIRECT_G)
   ulonglong2* T2;    // [2][G][LINE] partial u^T A22 u
   int lw;            // words per block in X: its rows, rounded up to whole lines
+  const int* emax;   // largest biased exponent of the whole matrix
   int sa;            // row stride of the block's rows in shared memory (0: they stay in L2)
   int* err;          // bit 0: a poll gave up
 };
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
   const int n = a.n, k0 = a.k0, G = gridDim.x, b = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool direct = G <= DIRECT_G;
+  const int amax = *a.emax - 1023;
   const int cnt = k0 + b < n ? (n - k0 - b + G - 1) / G : 0;  // rows k0 + b, k0 + b + G, ...
   if (__syncthreads_or(tid == 0 ? *(volatile int*)a.err & 1 : 0)) return;  // an earlier panel failed
   // per-row work: eight or four neighbouring threads per row, so that up to 32
@@ -196,11 +198,16 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
       if (bad) atomicOr(a.err, 1);
       return;
     }
-    // u is not scaled, so s2 holds |A| |u|^2: a column far from 1 is brought
-    // there by a power of two (v, tau and everything below stay as they are,
-    // inv absorbs it, beta gets it back)
-    const int ex = sE[j & 1] - 1023;
-    const bool scaled = (ex > 100 || ex < -200) && ex > -1023 && ex < 1024;  // the same in every block
+    // u is not scaled, so A22 u and s2 hold |A| |u| and |A| |u|^2, which can leave
+    // the float64 range where |A| does not. A column is brought under 2^-7 (|u| < 1
+    // up to 8192 rows) by a power of two where its largest entry 2^ec and the
+    // matrix's 2^amax (|A22| <= n 2^(amax + 1) throughout, the reduction being
+    // orthogonal) say 2 ec + amax > 960, i.e. n^2 |u|^2 |A| could pass 2^1023, and
+    // where ec < -200. v, tau and everything below stay as they are, inv absorbs
+    // the factor, beta gets it back. (Always scaling costs 6% to 11% a column on
+    // random matrices: 2048 13.0 -> 14.5 us.)
+    const int em_all = sE[j & 1], ec = em_all - 1023, ex = ec + 8;
+    const bool scaled = (2 * ec + amax > 960 || ec < -200) && em_all > 0 && em_all < 0x7FF;  // the same in every block
     if (scaled) {
       for (int r = j + 2 + tid; r < n; r += ST_THREADS) su[r] = scalbn(su[r], -ex);
       if (tid == 0) sa0 = scalbn(sa0, -ex);
@@ -450,6 +457,15 @@ __global__ void __launch_bounds__(ST_THREADS, 1) k_sytrd_panel(SytrdArgs a) {
   }
 }
 
+// Largest biased exponent field of x[0..n) into *emax (cleared before).
+__global__ void k_max_exponent(const double* __restrict__ x, int64_t n, int* __restrict__ emax) {
+  int m = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, (__double2hiint(x[i]) >> 20) & 0x7FF);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(emax, m);
+}
+
 // [V | W] and [W | V] as m x 2 NB row-major operands for the trailing update
 // (rows k.. of the panel's column-major V, W).
 __global__ void k_pack_vw(const double* __restrict__ Vp, const double* __restrict__ Wp,
@@ -518,7 +534,10 @@ osmps_status sytrd_tc(osmps_ctx* ctx, double* A, int64_t n, double* d, double* e
   double* X = Wp + NB * n;
   double* Y = X + 2 * NB * n;
   ulonglong2* word = reinterpret_cast<ulonglong2*>(buf + vecs);
-  OSMPS_CUDA(cudaMemsetAsync(word, 0, words * sizeof(ulonglong2), s));
+  int* emax = reinterpret_cast<int*>(word + words);
+  OSMPS_CUDA(cudaMemsetAsync(word, 0, (words + 1) * sizeof(ulonglong2), s));
+  { k_max_exponent<<<(int)std::min<int64_t>(cdiv(n * n, 1024), 1216), 256, 0, s>>>(A, n * n, emax); note_launch(); }
+  OSMPS_LAUNCH_CHECK();
   int* err = ctx->dev_flags + 3;
   for (int64_t k0 = 0; k0 < n; k0 += NB) {
     const int nbp = (int)std::min<int64_t>(NB, n - k0);
@@ -527,7 +546,7 @@ osmps_status sytrd_tc(osmps_ctx* ctx, double* A, int64_t n, double* d, double* e
     a.A = A; a.n = (int)n; a.k0 = (int)k0; a.nbp = nbp;
     a.d = d; a.e = e; a.tau = tau; a.Vp = Vp; a.Wp = Wp;
     a.X = word; a.Wn = a.X + 2 * xwords; a.part = a.Wn + 2 * NB; a.R = a.part + 2 * (size_t)MAXSUM * Gmax;
-    a.T2 = a.R + 2 * MAXSUM * LINE; a.err = err;
+    a.T2 = a.R + 2 * MAXSUM * LINE; a.err = err; a.emax = emax;
     const int64_t rows = cdiv(n - k0, G);
     a.lw = (int)round_up(rows, LINE);
     const int64_t stride = round_up(n - k0, 2);
