@@ -8,8 +8,7 @@
 //   M^[k] (few entries, Eq. MPOdef) act on the small (w, s) index pair of an
 //   intermediate, for every (outer, inner) fiber. These are bandwidth-bound:
 //   one coalesced pass over the input and the output, summing only over the
-//   nonzero MPO entries (an Inf or NaN input reaches the outputs it is
-//   connected to).
+//   nonzero MPO entries while every input is finite.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -140,22 +139,53 @@ struct WTerm {
 // them is read entry by entry instead (dense).
 constexpr int WT_CAP = 640;
 constexpr int WT_QMAX = 64;
+// how outputs are summed: from the terms; over the matrix, nonzero entries; over
+// the matrix, all entries (note_top)
+constexpr int W_TERMS = 0, W_NONZERO = 1, W_ALL = 2;
 template <typename T>
 struct WTable {
   WTerm<T> terms[WT_CAP];
   int ptr[WT_QMAX + 1];
   const double* Mat;
   int P, Q;
-  bool dense;
+  int dense;
 };
+
+// V fibers of one thread.
+template <typename T, int V>
+struct alignas(sizeof(T) * V) Pack {
+  T a[V];
+};
+
+// The largest magnitude met so far, as (upper) float bits. Where a fiber's
+// inputs are below 2^63 in float32 or 2^511 in float64 and the MPO entries
+// below 2^50, all that a W-step and the one fused behind it sum is finite (at
+// most 2^11 terms each) and zero entries can be left out. Else (one comparison
+// for all values of a block) they are summed like the others, because 0 x Inf =
+// NaN has to reach every output; finite sums have the same bits either way.
+template <typename T, int V>
+__device__ __forceinline__ void note_top(int& top, const Pack<T, V>& x) {
+#pragma unroll
+  for (int v = 0; v < V; ++v) {
+    if constexpr (sizeof(T) == 8) top = max(top, __double2hiint(x.a[v]) & 0x7FFFFFFF);
+    else top = max(top, __float_as_int(x.a[v]) & 0x7FFFFFFF);
+  }
+}
+template <typename T>
+__device__ __forceinline__ bool wild(int top) {
+  return top >= (sizeof(T) == 8 ? 0x5FE00000 : 0x5F000000);
+}
+__device__ __forceinline__ bool wild_entry(double m) { return (__double2hiint(m) & 0x7FFFFFFF) >= 0x43100000; }
 
 // Fill NT tables. Every thread of the block calls it (whole warps): a warp
 // per output, lanes over the inputs, the nonzero ones compacted by ballots.
-// Ends with a barrier.
+// Ends with a barrier, which also says whether any thread met wild values, in
+// its inputs (top) or in the tables.
 template <int NT, typename T>
-__device__ __forceinline__ void gather_terms(const double* const (&Mat)[NT], const int (&P)[NT],
+__device__ __forceinline__ bool gather_terms(int top, const double* const (&Mat)[NT], const int (&P)[NT],
                                              const int (&Q)[NT], WTable<T>* const (&tab)[NT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  bool all = wild<T>(top);
 #pragma unroll
   for (int k = 0; k < NT; ++k)
     for (int o = warp; o < Q[k]; o += warps) {
@@ -163,6 +193,7 @@ __device__ __forceinline__ void gather_terms(const double* const (&Mat)[NT], con
       for (int i0 = 0; i0 < P[k]; i0 += 32) {
         const double m = i0 + lane < P[k] ? Mat[k][(i0 + lane) * Q[k] + o] : 0.0;
         n += __popc(__ballot_sync(0xffffffffu, m != 0.0));
+        all |= wild_entry(m);
       }
       if (lane == 0) tab[k]->ptr[o + 1] = n;
     }
@@ -175,7 +206,7 @@ __device__ __forceinline__ void gather_terms(const double* const (&Mat)[NT], con
     w.Mat = Mat[warp < NT ? warp : 0];
     w.P = P[warp < NT ? warp : 0];
     w.Q = q1;
-    w.dense = w.ptr[q1] > WT_CAP || w.P > 32767;
+    w.dense = w.ptr[q1] > WT_CAP || w.P > 32767 ? W_NONZERO : W_TERMS;
   }
   __syncthreads();
 #pragma unroll
@@ -191,14 +222,8 @@ __device__ __forceinline__ void gather_terms(const double* const (&Mat)[NT], con
           n += __popc(nz);
         }
       }
-  __syncthreads();
+  return __syncthreads_or(all);
 }
-
-// V fibers of one thread.
-template <typename T, int V>
-struct alignas(sizeof(T) * V) Pack {
-  T a[V];
-};
 
 // Output o of a W-step: sum over its nonzero entries of v x_i, inputs in
 // ascending order; x_i is at xs[i stride]. A first entry of 1 is taken over
@@ -216,7 +241,7 @@ __device__ __forceinline__ Pack<T, V> sum_terms(const WTable<T>& w, int o,
   if (w.dense) {
     for (int i = 0; i < w.P; ++i) {
       const T m = (T)w.Mat[i * w.Q + o];
-      if (m != (T)0) add(m, xs[i * stride]);
+      if (w.dense == W_ALL || m != (T)0) add(m, xs[i * stride]);
     }
     return acc;
   }
@@ -338,13 +363,21 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
       fib.at[v] = o1 * f.is1 + o2 * f.is2 + c;
       ob[v] = o1 * f.os1 + o2 * f.os2 + c;
     }
-    if (staged) {
+    int top = 0;
 #pragma unroll 4
-      for (int i = warp; i < P; i += FIB_WARPS) xs[i * 32] = fib.load(in, (int64_t)i * f.istride);
+    for (int i = warp; i < P; i += FIB_WARPS) {
+      const Pack<T, V> x = fib.load(in, (int64_t)i * f.istride);
+      if (staged) xs[i * 32] = x;
+      note_top<T, V>(top, x);
     }
-    if (first) gather_terms<1, T>({Mat}, {P}, {Q}, {&tab});
-    else if (staged) __syncthreads();
+    bool all = false;
+    if (first) all = gather_terms<1, T>(top, {Mat}, {P}, {Q}, {&tab});
+    else all = __syncthreads_or(wild<T>(top));
     first = false;
+    if (all) {  // from here on
+      if (threadIdx.x == 0) tab.dense = W_ALL;
+      __syncthreads();
+    }
     for (int o = warp; o < Q; o += FIB_WARPS) {
       Pack<T, V> acc;
       if (staged) {
@@ -354,7 +387,7 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
         for (int v = 0; v < V; ++v) acc.a[v] = (T)0;
         for (int i = 0; i < P; ++i) {
           const T m = (T)Mat[i * Q + o];
-          if (m == (T)0) continue;
+          if (tab.dense != W_ALL && m == (T)0) continue;
           const Pack<T, V> x = fib.load(in, (int64_t)i * f.istride);
 #pragma unroll
           for (int v = 0; v < V; ++v) acc.a[v] = fma(m, x.a[v], acc.a[v]);
@@ -436,9 +469,12 @@ osmps_status fiber_dispatch(const Fiber& f, const double* Mat, const T* in, T* o
 // separate passes, term by term. Traffic: one read of T1, one write of T3; in
 // float64 the ~36 FMAs per fiber come next (XXZ chi = 512: 55 us, float64 pipe
 // 44% active, against 158 + 158 us for two dense passes); AKLT 301x257 in
-// float32 61 us against 152 + 147.
+// float32 61 us against 152 + 147. Blocks per SM: for packed float64 fibers the
+// five that the tables and XXZ's columns leave room for (with four, 71 us), else
+// four (left to itself the compiler takes 48 registers: AKLT 2 us slower, a
+// 33 x 31 float64 product 1 us).
 template <typename T, int MODE, int D, int V, bool PACKED>
-__global__ void __launch_bounds__(32 * FIB_WARPS)
+__global__ void __launch_bounds__(32 * FIB_WARPS, sizeof(T) == 8 && PACKED ? 5 : 4)
     k_wsteps(const T* __restrict__ T1, const double* __restrict__ Mat1,
              const double* __restrict__ Mat2, int wl, int wm, int wr, T* __restrict__ out,
              void* __restrict__ sdst, int64_t Kp, int64_t chi_l, int64_t chi_r, FastDiv by_c,
@@ -469,11 +505,21 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
       fib.at[v] = a2 * (P1 * D) * chi_r + c;
       ob[v] = a2 * (D * D) * ldo + c;
     }
+    int top = 0;
 #pragma unroll 4
-    for (int k = warp; k < P1 * D; k += FIB_WARPS) xs[k * 32] = fib.load(T1, k * chi_r);
-    if (first) gather_terms<2, T>({Mat1, Mat2}, {P1, P2}, {Q1, Q2}, {&tab1, &tab2});
-    else __syncthreads();
+    for (int k = warp; k < P1 * D; k += FIB_WARPS) {
+      const Pack<T, V> x = fib.load(T1, k * chi_r);
+      xs[k * 32] = x;
+      note_top<T, V>(top, x);
+    }
+    bool all = false;
+    if (first) all = gather_terms<2, T>(top, {Mat1, Mat2}, {P1, P2}, {Q1, Q2}, {&tab1, &tab2});
+    else all = __syncthreads_or(wild<T>(top));
     first = false;
+    if (all) {  // from here on
+      if (threadIdx.x == 0) tab1.dense = tab2.dense = W_ALL;
+      __syncthreads();
+    }
     for (int o = warp; o < Q1; o += FIB_WARPS)
 #pragma unroll
       for (int s2 = 0; s2 < D; ++s2) ms[(o * D + s2) * 32] = sum_terms<T, V>(tab1, o, xs + s2 * 32, D * 32);
