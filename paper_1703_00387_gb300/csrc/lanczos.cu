@@ -820,7 +820,10 @@ osmps_status project(osmps_ctx* ctx, const double* V, int64_t ld, int64_t n, int
 // passes, each a kernel of block-partial products and one that adds the
 // partial sums up itself (a third kernel does past 64 of them), subtracts and
 // leaves the norm's partials: five launches where there were nine.
-// Beyond, the second pass is taken only where the first removed most of w.
+// Beyond, the ground-state solver takes the second pass only where the first
+// removed most of w (a pass reads the whole basis twice); with `twice` (the
+// propagator, whose few vectors enter the result with equal weight) it is
+// always taken.
 //
 // (Taking alpha v_J and beta v_(J-1) off first, so that one full pass is
 // enough, halves the traffic of long vectors, 3.5 of 98 ms of a chi = 1024
@@ -828,10 +831,14 @@ osmps_status project(osmps_ctx* ctx, const double* V, int64_t ld, int64_t n, int
 // value in some runs falls to the other side of a bf16 rounding in the next
 // products, and the Ritz vector moves by up to 7e-7 in 13% of them.)
 osmps_status orthogonalise(osmps_ctx* ctx, const double* V, int64_t ld, int64_t n, int nv_max, double* w,
-                           double* part, double* sc, cudaStream_t s) {
+                           double* part, double* sc, bool twice, cudaStream_t s) {
   const int* state = lz_state(sc);
   int ub = 0;
-  if (n > ((int64_t)1 << 18)) {
+  if (n > ((int64_t)1 << 18) && twice) {
+    OSMPS_TRY(project(ctx, V, ld, n, nv_max, w, part, sc + OFF_C1, s, state));
+    OSMPS_TRY(project(ctx, V, ld, n, nv_max, w, part, sc + OFF_C2, s, state));
+    OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 3, s));
+  } else if (n > ((int64_t)1 << 18)) {
     int* skip = reinterpret_cast<int*>(sc + OFF_MISC + 6);
     OSMPS_TRY(vec_norm2(ctx, w, n, sc + OFF_MISC + 5, s));
     OSMPS_TRY(project(ctx, V, ld, n, nv_max, w, part, sc + OFF_C1, s, state));
@@ -1076,7 +1083,7 @@ osmps_status lanczos_core(osmps_ctx* ctx, int64_t n, double* theta, int max_iter
       OSMPS_TRY(project(ctx, P, ldp, n, kp, w, part, sc + OFF_PROJ, q));
       OSMPS_TRY(project(ctx, P, ldp, n, kp, w, part, sc + OFF_PROJ + MAX_PROJ, q));
     }
-    OSMPS_TRY(orthogonalise(ctx, V, ld, n, nv_max, w, part, sc, q));
+    OSMPS_TRY(orthogonalise(ctx, V, ld, n, nv_max, w, part, sc, false, q));
     if (fork) OSMPS_TRY(side.join(q));
     if (!beside) OSMPS_TRY(tridiag(q));
     { k_next_vector<<<ew_blocks(n), 256, 0, q>>>(V, ld, w, n, sc, X, max_iter, cond, set_cond); note_launch(); }
@@ -1544,7 +1551,7 @@ osmps_status expm_core(osmps_ctx* ctx, int64_t n_c, const double* theta_emb, dou
   OSMPS_CUDA(cudaMemsetAsync(state, 0, 4 * sizeof(int), s));
   for (int j = 0; j < max_iter; ++j) {
     OSMPS_TRY(matvec(V + (int64_t)j * ld, w, s));
-    OSMPS_TRY(orthogonalise(ctx, V, ld, n, j + 1, w, part, sc, s));
+    OSMPS_TRY(orthogonalise(ctx, V, ld, n, j + 1, w, part, sc, true, s));
     { k_expm_tridiag<<<1, EXPM_THREADS, 0, s>>>(sc, max_iter, tol, tau, (long long)n_c); note_launch(); }
     OSMPS_LAUNCH_CHECK();
     { k_next_vector<<<ew_blocks(n), 256, 0, s>>>(V, ld, w, n, sc, nullptr, max_iter, 0, 0); note_launch(); }
