@@ -44,6 +44,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "operand.cuh"
 #include "tcgen05.cuh"
 
 namespace osmps {
@@ -510,11 +511,8 @@ __global__ void __launch_bounds__(256) k_slice_rows(SplitView v, int* __restrict
   const S* src = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1;
   const auto load = [&](int64_t k, double (&x)[8]) {
     if (vec && k + 8 <= v.K) {
-      constexpr int PER = 16 / sizeof(S);
       S q[8];
-#pragma unroll
-      for (int i = 0; i < 8; i += PER)
-        *reinterpret_cast<uint4*>(q + i) = *reinterpret_cast<const uint4*>(src + k + i);
+      load_eight(src + k, q);
 #pragma unroll
       for (int i = 0; i < 8; ++i) x[i] = (double)q[i];
     } else {

@@ -34,6 +34,26 @@ __device__ __forceinline__ typename SplitWord<KIND>::T split_word(S x) {
   }
 }
 
+// Eight consecutive values from a 16-byte boundary, in 16-byte loads.
+__device__ __forceinline__ void load_eight(const double* p, double (&x)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    const double2 q = *reinterpret_cast<const double2*>(p + i);
+    x[i] = q.x;
+    x[i + 1] = q.y;
+  }
+}
+__device__ __forceinline__ void load_eight(const float* p, float (&x)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; i += 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p + i);
+    x[i] = q.x;
+    x[i + 1] = q.y;
+    x[i + 2] = q.z;
+    x[i + 3] = q.w;
+  }
+}
+
 // Eight consecutive columns of an operand row (off_hi a multiple of 8) in
 // 16-byte stores.
 __device__ __forceinline__ void store_words(void* dst, int64_t off_hi, int64_t Kp, const uint32_t (&w)[8]) {

@@ -69,12 +69,7 @@ __global__ void __launch_bounds__(256) k_split_direct(SplitView v, void* __restr
     const S* p = reinterpret_cast<const S*>(v.src) + r0 * v.s0 + r1 * v.s1 + k * v.sk;
     S x[8];
     if (vec && k + 8 <= v.K) {
-      constexpr int PER = 16 / sizeof(S);
-#pragma unroll
-      for (int i = 0; i < 8; i += PER) {
-        const uint4 q = *reinterpret_cast<const uint4*>(p + i);
-        *reinterpret_cast<uint4*>(x + i) = q;
-      }
+      load_eight(p, x);
     } else {
 #pragma unroll
       for (int i = 0; i < 8; ++i) x[i] = k + i < v.K ? p[i * v.sk] : (S)0;

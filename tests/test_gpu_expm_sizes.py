@@ -1,8 +1,9 @@
 """The propagator at the vector length where the orthogonalisation changes its
 form (2^18 entries of the embedded vector): against the oracle's Krylov space,
-and projected twice in every step on both sides of it. Below it two projections and the norm are seven launches, beyond it nine
-(twice three and two for the norm, one for alpha and beta); deciding whether to
-project again would add a norm and the decision.
+and projected twice in every step on both sides of it. Below it two projections
+and the norm are seven launches, beyond it nine (twice three and two for the
+norm, one for alpha and beta); deciding whether to project again would add a norm
+and the decision.
 """
 import numpy as np
 import pytest
