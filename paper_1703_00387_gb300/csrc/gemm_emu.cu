@@ -31,9 +31,11 @@
 // slice tiles per K block and output tile where a pass over K for each pair
 // took 72, which the 60 bytes per clock that an SM takes in from L2 allowed one
 // pair in 570 clocks; now 380, the rest being the single issuing warp and the
-// drains. 2048 x 2048 x 2048: kernel 764 -> 481 us (1280 TFLOP/s of bf16), 2560 x
-// 2048 x 512: 348 -> 211, 2048 x 512 x 2560 with K in shares: 475 -> 178, 381 x 1905
-// x 1000: 201 -> 74.
+// drains. 2048 x 2048 x 2048: kernel 764 -> 479 us (1290 TFLOP/s of bf16), 2560 x
+// 2048 x 512: 348 -> 208, 2048 x 512 x 2560 with K in shares: 475 -> 168, 381 x 1905
+// x 1000: 201 -> 68. (Shares are added as integers: rounded to float64 first they
+// cost 177 and 75 us and seven more roundings, 1.3e-16 instead of 8e-17 against
+// 113-bit arithmetic at 128 x 128 x 2048.)
 // The kernel is persistent and warp-specialised: a TMA producer with a ring
 // of 13 slice tiles, a warp that issues the MMAs, and 16 epilogue warps each
 // holding 32 exact sums per row in registers.
@@ -143,13 +145,17 @@ __device__ __forceinline__ void store_row4(double* p, int64_t c, int64_t N, int 
 }
 
 // What the kernel writes: C[r][c] (subtract: C -= the product), rows of ldc
-// values, two per access where `vec`; share s of K writes at s * slab. G holds
-// the sums of the diagonal groups before the last, in an order of the threads'
-// own (128 KB for each CTA, [column pair][thread], so that a warp's accesses
-// are whole lines: in C itself they took a line for each lane).
+// values, two per access where `vec`. G holds the sums of the diagonal groups
+// before the last, in an order of the threads' own (128 KB for each CTA,
+// [column pair][thread], so that a warp's accesses are whole lines: in C itself
+// they took a line for each lane).
+// With K in shares (H set) nothing is rounded here: group g of share s goes to
+// H[s][g][r][c] as the exact integer, planes of `slab` and rows of ldc integers
+// (ldc a multiple of four), and k_emu_combine adds the shares.
 struct EmuOut {
   double* C;
   double2* G;
+  long long* H;
   int64_t ldc, slab;
   int subtract, vec;
 };
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(E_THREADS, 1)
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       int m0, n0, kb0, kb1;
-      const int64_t off = (int64_t)item_of(item, m0, n0, kb0, kb1) * out.slab;
+      const int share = item_of(item, m0, n0, kb0, kb1);
       const int64_t row = (int64_t)m0 + qd * 32 + lane;
       const int64_t col0 = (int64_t)n0 + part * E_EPI_COLS;
       for (int d0 = 0; d0 < SLICES && ok; d0 += GD) {
@@ -379,10 +385,18 @@ __global__ void __launch_bounds__(E_THREADS, 1)
         if (!ok) break;
         // close the group: its sums become float64 with the scales folded in,
         // added to those of the groups before
-        if (row < M) {
+        if (out.H) {
+          long long* h = out.H + ((int64_t)share * (SLICES / GD) + d0 / GD) * out.slab + row * out.ldc;
+#pragma unroll
+          for (int j = 0; j < E_EPI_COLS; j += 4)
+            if (row < M && col0 + j < N) {
+              *reinterpret_cast<longlong2*>(h + col0 + j) = make_longlong2(H[j], H[j + 1]);
+              *reinterpret_cast<longlong2*>(h + col0 + j + 2) = make_longlong2(H[j + 2], H[j + 3]);
+            }
+        } else if (row < M) {
           const bool final = d1 == SLICES - 1;
           const int k0 = -SLICE_BITS * (d1 + 2) + eA[row];
-          double* c = out.C + off + row * out.ldc;
+          double* c = out.C + row * out.ldc;
           double2* g = out.G + (size_t)blockIdx.x * (EBM * EBN / 2) + (threadIdx.x - 64);
 #pragma unroll
           for (int h = 0; h < E_EPI_COLS / 4; ++h) {
@@ -427,13 +441,26 @@ __global__ void __launch_bounds__(E_THREADS, 1)
   }
 }
 
-// C = sum of the partial products (or C -= it), its slabs in order.
-__global__ void k_emu_combine(const double* __restrict__ P, int splits, int64_t slab, int64_t ldp,
-                              int64_t N, double* __restrict__ C, int64_t ldc, int subtract) {
+// C = (or -=) the product whose group sums lie in `splits` shares: the shares
+// are added as integers, exactly, so the bits do not depend on their number.
+template <int GD>
+__global__ void k_emu_combine(const long long* __restrict__ H, int splits, int64_t slab, int64_t ldh,
+                              int64_t N, const int* __restrict__ eA, const int* __restrict__ eB,
+                              double* __restrict__ C, int64_t ldc, int subtract) {
+  constexpr int GROUPS = SLICES / GD;
   const int64_t r = blockIdx.y;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < N; c += (int64_t)gridDim.x * blockDim.x) {
+    long long h[GROUPS] = {};
+#pragma unroll 4
+    for (int s = 0; s < splits; ++s)
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g) h[g] += H[((int64_t)s * GROUPS + g) * slab + r * ldh + c];
     double t = 0.0;
-    for (int s = 0; s < splits; ++s) t += P[s * slab + r * ldp + c];
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) {
+      const double v = i64_ldexp(h[g], -SLICE_BITS * (GD * (g + 1) + 1) + eA[r] + eB[c]);
+      t = g == 0 ? v : v + t;
+    }
     double* dst = C + r * ldc + c;
     *dst = subtract ? *dst - t : t;
   }
@@ -636,25 +663,27 @@ osmps_status slice_operand(osmps_ctx* ctx, const SplitView& v, int64_t Kp, int* 
   return OSMPS_OK;
 }
 
-// Tiles of partial products at most, per SM: the scratch of the kernel then has
-// one size for all products and never grows after the first (a growing one
-// would be refused inside a graph capture).
+// Tiles of shares at most, per SM: the scratch of the kernel then has one size
+// for all products up to K = 2^17 (two planes of two tiles for each SM, 80 MB)
+// and never grows after the first (a growing one would be refused inside a
+// graph capture).
 constexpr int E_SLAB_WAVES = 2;
 
 // Shares of K per output tile. A tile takes its K blocks one after the other
 // on one SM, so a product of few tiles leaves SMs idle; its K blocks are then
-// shared out, the partial products going to slabs that are added in order.
-// Taken by estimated clocks: 36 slice pairs of about 300 per K block, 8000 per
-// tile for its drains and sums, and for the slabs 2600 bytes a clock and
-// one launch. With one share 512 x 512 x 2048 took 381 us and 1024 x 1024 x 2048
-// 385 (a pass over K per pair), with eight and two shares 64 and 150.
-int emu_splits(int64_t M, int64_t N, int64_t n_tiles, int64_t nkb, int sms) {
+// shared out, the shares' integer sums added by a second kernel.
+// Taken by estimated clocks: 36 slice pairs of 380 per K block, 8000 per tile for
+// its drains and sums, and for the shares one more launch and 16 bytes per group
+// and element at 2600 bytes a clock. Kernels with one share and with the shares
+// taken: 128 x 128 x 2048 234 and 49 us, 512 x 512 x 2048 231 and 56, 1024 x 1024
+// x 2048 240 and 140, 381 x 1905 x 1000 130 and 68.
+int emu_splits(int64_t M, int64_t N, int64_t n_tiles, int64_t nkb, int groups, int sms) {
   if (M > 65535) return 1;
   int best = 1;
   double t_best = 0;
   for (int s = 1; s <= 8 && (s == 1 || (nkb / s >= 2 && n_tiles * s <= E_SLAB_WAVES * sms)); ++s) {
-    double t = (double)cdiv(n_tiles * s, sms) * ((double)cdiv(nkb, s) * 36 * 300 + 8000);
-    if (s > 1) t += (double)s * M * N * 16 / 2600 + 6000;
+    double t = (double)cdiv(n_tiles * s, sms) * ((double)cdiv(nkb, s) * 36 * 380 + 8000);
+    if (s > 1) t += (double)s * M * N * 16 * groups / 2600 + 6000;
     if (s == 1 || t < t_best) {
       best = s;
       t_best = t;
@@ -707,21 +736,23 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   const int tiles_n = (int)cdiv(N, EBN);
   const int n_tiles = tiles_n * (int)cdiv(M, EBM);
   const int nkb = (int)(Kp / 64);
-  const int splits = emu_splits(M, N, n_tiles, nkb, ctx->sm_count);
-  const int grid = std::min(n_tiles * splits, ctx->sm_count);
-  EmuOut out{C, nullptr, ldc, 0, subtract && splits == 1 ? 1 : 0, 0};
-  if (splits > 1) {
-    out.ldc = round_up(N, 2);
-    out.slab = M * out.ldc;
-  }
-  const size_t tile_sums = (size_t)ctx->sm_count * EBM * EBN;
-  auto* scratch = (double*)ws_get(ctx, SLOT_EMU_PART, (1 + E_SLAB_WAVES) * tile_sums * 8, s, &st);
-  if (!scratch) return st;
-  out.G = reinterpret_cast<double2*>(scratch);
-  if (splits > 1) out.C = scratch + tile_sums;
-  out.vec = (reinterpret_cast<uintptr_t>(out.C) & 15) == 0 && out.ldc % 2 == 0;
   // diagonals per exact int64 group: four while a group sum stays below 2^53
   // (|I_d| < (d + 1) K 2^14 with slice digits of at most 2^7 and 2^6), else two
+  const int groups = Kp <= ((int64_t)1 << 17) ? 2 : 4;
+  const int splits = emu_splits(M, N, n_tiles, nkb, groups, ctx->sm_count);
+  const int grid = std::min(n_tiles * splits, ctx->sm_count);
+  EmuOut out{C, nullptr, nullptr, ldc, 0, subtract ? 1 : 0, 0};
+  const size_t tile_sums = (size_t)ctx->sm_count * EBM * EBN;
+  void* scratch = ws_get(ctx, SLOT_EMU_PART, groups * E_SLAB_WAVES * tile_sums * 8, s, &st);
+  if (!scratch) return st;
+  if (splits > 1) {
+    out.H = static_cast<long long*>(scratch);
+    out.ldc = round_up(N, 4);
+    out.slab = M * out.ldc;
+  } else {
+    out.G = static_cast<double2*>(scratch);
+    out.vec = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ldc % 2 == 0;
+  }
   const auto run = [&](auto kernel, cudaError_t configured) -> osmps_status {
     OSMPS_CUDA(configured);
     kernel<<<grid, E_THREADS, E_SMEM, s>>>(ma, mb, out, M, N, nkb, (int)Kp, tiles_n, n_tiles, splits, eA, eB,
@@ -731,7 +762,7 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   };
   const int ph = prof_begin(s);
   // thread-safe one-time setups (function-local static initialisation)
-  if (Kp <= ((int64_t)1 << 17)) {
+  if (groups == 2) {
     static const cudaError_t configured =
         cudaFuncSetAttribute(k_gemm_emu<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)E_SMEM);
     OSMPS_TRY(run(k_gemm_emu<4>, configured));
@@ -742,7 +773,8 @@ osmps_status gemm_emu(osmps_ctx* ctx, const SplitView& a, const SplitView& b, in
   }
   if (splits > 1) {
     const dim3 cg((unsigned)std::min<int64_t>(cdiv(N, 256), 64), (unsigned)M);
-    k_emu_combine<<<cg, 256, 0, s>>>(out.C, splits, out.slab, out.ldc, N, C, ldc, subtract ? 1 : 0);
+    const auto combine = groups == 2 ? k_emu_combine<4> : k_emu_combine<2>;
+    combine<<<cg, 256, 0, s>>>(out.H, splits, out.slab, out.ldc, N, eA, eB, C, ldc, subtract ? 1 : 0);
     note_launch();
   }
   OSMPS_LAUNCH_CHECK();
