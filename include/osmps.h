@@ -319,12 +319,19 @@ osmps_status osmps_selftest_wait_timeout(osmps_ctx* ctx, int which, double limit
  * of n elements). Results must equal the IEEE conversions bit for bit.    */
 osmps_status osmps_selftest_convert(osmps_ctx* ctx, const double* x64, float* y32,
                                     const float* x32, double* y64, int64_t n, void* stream);
-/* Test support: the bf16 rounding of n doubles (device arrays) by the
- * integer-field route the U(1) operand split uses (y_int) and by CUDA's
+/* Test support: the bf16 rounding of n doubles (device arrays) as the operand
+ * splits form it with integer operations (the hi word, y_int) and by CUDA's
  * __double2bfloat16 (y_hw), as raw 16-bit patterns. EINVAL for a null
  * pointer with n > 0 or n < 0.                                              */
 osmps_status osmps_selftest_bf16(osmps_ctx* ctx, const double* x, uint16_t* y_int, uint16_t* y_hw,
                                  int64_t n, void* stream);
+/* Test support: both words of the hi / lo split of n doubles for `precision`
+ * (OSMPS_PREC_BF16X3 or TF32X3; others EINVAL) as the operand passes form it
+ * (got) and by the hardware conversions h = cvt(x), l = cvt(x - h) (ref):
+ * device arrays of 2 n raw words, hi then lo of each value (bf16 in the lower
+ * half), 8-byte aligned. EINVAL as above.                                    */
+osmps_status osmps_selftest_split(osmps_ctx* ctx, const double* x, int precision, uint32_t* got,
+                                  uint32_t* ref, int64_t n, void* stream);
 
 /* Environment update (Sec. 3.4: the fixed sites are contracted into L and R
  * one site at a time).

@@ -111,6 +111,7 @@ _SIGS = {
     "osmps_selftest_wait_timeout": (_c.c_int, [_vp, _c.c_int, _c.c_double, _vp]),
     "osmps_selftest_convert": (_c.c_int, [_vp, _vp, _vp, _vp, _vp, _i64, _vp]),
     "osmps_selftest_bf16": (_c.c_int, [_vp, _vp, _vp, _vp, _i64, _vp]),
+    "osmps_selftest_split": (_c.c_int, [_vp, _vp, _c.c_int, _vp, _vp, _i64, _vp]),
     "osmps_gemm_grouped": (_c.c_int, [_vp, _vp, _i64, _vp, _i64, _vp]),
     "osmps_copy_list": (_c.c_int, [_vp, _c.POINTER(CopyDesc), _i64, _vp]),
     "osmps_sym_eig_top": (_c.c_int, [_vp, _vp, _i64, _i64, _dp, _vp, _vp]),
@@ -782,6 +783,16 @@ def osmps_selftest_bf16(ctx, x, stream=None):
     _check(lib().osmps_selftest_bf16(ctx.ptr, _dev(x, "x"), _vp(yi.data_ptr()), _vp(yh.data_ptr()),
                                      x.numel(), _stream(stream)))
     return yi, yh
+
+
+def osmps_selftest_split(ctx, x, precision, stream=None):
+    """(operand passes', hardware's) hi / lo splits of the float64 device tensor
+    x as int32 tensors (n, 2) of raw words."""
+    import torch
+    got, ref = (torch.empty(x.numel(), 2, dtype=torch.int32, device=x.device) for _ in range(2))
+    _check(lib().osmps_selftest_split(ctx.ptr, _dev(x, "x"), _prec(precision), _vp(got.data_ptr()),
+                                      _vp(ref.data_ptr()), x.numel(), _stream(stream)))
+    return got, ref
 
 
 def osmps_gemm_grouped(ctx, outs, terms, stream=None):

@@ -11,7 +11,7 @@
 //              blocks do).
 // Nothing faults, traps or spins without a bound; the context stays usable.
 #include "common.cuh"
-#include "ieee.cuh"
+#include "operand.cuh"
 #include "tagged.cuh"
 #include "tcgen05.cuh"
 
@@ -78,6 +78,27 @@ __global__ void k_selftest_bf16(const double* __restrict__ x, uint16_t* __restri
   }
 }
 
+// Both words of the hi / lo split of float64 values as the operand passes form
+// them, beside the hardware conversions: h = cvt(x), l = cvt(x - h).
+template <int KIND>
+__global__ void k_selftest_split(const double* __restrict__ x, uint2* __restrict__ got,
+                                 uint2* __restrict__ ref, int64_t n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if constexpr (KIND == TC_BF16) {
+      const uint32_t w = split_word<KIND, double>(x[i]);
+      got[i] = make_uint2(w & 0xFFFFu, w >> 16);
+      const __nv_bfloat16 h = __double2bfloat16(x[i]);
+      const __nv_bfloat16 l = __double2bfloat16(x[i] - (double)__bfloat162float(h));
+      ref[i] = make_uint2(__bfloat16_as_ushort(h), __bfloat16_as_ushort(l));
+    } else {
+      got[i] = split_word<KIND, double>(x[i]);
+      const uint32_t h = to_tf32((float)x[i]);
+      ref[i] = make_uint2(h, to_tf32((float)(x[i] - (double)__uint_as_float(h))));
+    }
+  }
+}
+
 }  // namespace
 }  // namespace osmps
 
@@ -95,6 +116,29 @@ extern "C" osmps_status osmps_selftest_bf16(osmps_ctx* ctx, const double* x, uin
   cudaStream_t s = (cudaStream_t)stream;
   const int blocks = (int)std::min<int64_t>((n + 255) / 256, 4096);
   k_selftest_bf16<<<blocks, 256, 0, s>>>(x, y_int, y_hw, n);
+  note_launch();
+  OSMPS_LAUNCH_CHECK();
+  return OSMPS_OK;
+}
+
+extern "C" osmps_status osmps_selftest_split(osmps_ctx* ctx, const double* x, int precision, uint32_t* got,
+                                             uint32_t* ref, int64_t n, void* stream) {
+  clear_error();
+  if (!ctx || (n > 0 && (!x || !got || !ref)))
+    return set_error(OSMPS_EINVAL, "osmps_selftest_split: null argument");
+  if (n < 0) return set_error(OSMPS_EINVAL, "osmps_selftest_split: n=%lld", (long long)n);
+  if (precision != OSMPS_PREC_BF16X3 && precision != OSMPS_PREC_TF32X3)
+    return set_error(OSMPS_EINVAL, "osmps_selftest_split: precision %d", precision);
+  for (const uint32_t* p : {got, ref})
+    if ((reinterpret_cast<uintptr_t>(p) & 7) != 0)
+      return set_error(OSMPS_EINVAL, "osmps_selftest_split: outputs must be 8-byte aligned");
+  if (n == 0) return OSMPS_OK;
+  OSMPS_CUDA(cudaSetDevice(ctx->device));
+  CtxScope scope_(ctx);
+  cudaStream_t s = (cudaStream_t)stream;
+  const int blocks = (int)std::min<int64_t>((n + 255) / 256, 4096);
+  const auto kernel = precision == OSMPS_PREC_BF16X3 ? k_selftest_split<TC_BF16> : k_selftest_split<TC_TF32>;
+  kernel<<<blocks, 256, 0, s>>>(x, reinterpret_cast<uint2*>(got), reinterpret_cast<uint2*>(ref), n);
   note_launch();
   OSMPS_LAUNCH_CHECK();
   return OSMPS_OK;
