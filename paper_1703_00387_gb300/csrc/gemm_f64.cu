@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(128) k_gemm_f64(Args p, int tiles_n) {
 // FMA: with several rounds of tiles it measured 2% (300x300x340) to 40%
 // (256x256x256) slower at equal load, so it wins where it halves the rounds
 // (128x128x128: 8.3 against 14.4 us) and not for a few per cent of balance.
-constexpr int F64_SMS = 152;
+constexpr int F64_SMS = 152;  // of the one GPU this code is for
 constexpr double COST_8 = 1.15;
 double busiest_sm(int64_t M, int64_t N, int64_t batch, int64_t t) {
   return (double)cdiv(cdiv(M, t) * cdiv(N, t) * batch, F64_SMS) * (double)(t * t);
@@ -171,6 +171,7 @@ osmps_status gemm_f64(const GemmF64& g, cudaStream_t stream) {
   if (g.K <= 0) {
     return set_error(OSMPS_ESHAPE, "gemm_f64: K=%lld", (long long)g.K);
   }
+  // (M: a row limit that callers have always met; the grid's own is the tiles')
   if (g.M > (int64_t)64 * 65535 || g.batch > 65535)
     return set_error(OSMPS_ESHAPE, "gemm_f64: M=%lld batch=%lld exceed the supported range",
                      (long long)g.M, (long long)g.batch);

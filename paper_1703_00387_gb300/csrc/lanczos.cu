@@ -273,18 +273,22 @@ __global__ void k_combine_scalar(const double* __restrict__ V, int64_t ld,
   }
 }
 
-// The lowest eigenpair of T_{j+1}, j = state ST_T; one block of four warps (one per SM sub-partition: the float64
-// pipe of a sub-partition is the limit for a single warp).
+// The lowest eigenpair of T_{j+1}, j = state ST_T; one block of four warps (one
+// per SM sub-partition: the float64 pipe of a sub-partition is the limit for a
+// single warp).
 //   * Eigenvalue: multisection, 128 points per round (one per thread),
 //     from the Gershgorin interval: first on float32 Sturm counts of T/||T||
 //     down to 1e-5 ||T|| (the float32 pipe is far wider), then the bracket
 //     is padded, checked with float64 counts at its ends (the full interval
 //     again if the check fails), and narrowed to 4e-16 relative width on
-//     division-free float64 counts (sturm.cuh).
-//   * Eigenvector: the twisted factorisation of T - e I (top-down and
-//     bottom-up pivot chains on two warps, twist index where |gamma| is
-//     least, the vector by two product chains from it), normalised in
-//     parallel.
+//     division-free float64 counts (sturm.cuh), the points of a round placed
+//     around the secant zero of the last minors.
+//   * Eigenvector: twisted, from the three-term recurrences of (T - e I) z = 0
+//     run down from the top and up from the bottom on two warps, with the
+//     off-diagonals' reciprocals formed beforehand; the twist index is where
+//     |gamma| is least. Only where T all but splits (an off-diagonal under
+//     1e-30 ||T||) the pivot chains of the twisted factorisation with their
+//     divisions. Normalised in parallel.
 // Then the stopping decision: a non-finite Ritz value or residual; converged
 // (residual estimate <= tol, beta = 0, or the Krylov space is the whole
 // space); the step cap. After a stop the kernel returns at once.

@@ -186,10 +186,11 @@ class BlockBudget:
 
 
 def coop_blocks(n, sms, solver=None):
-    """Blocks of the Householder panel's cooperative launch for an n x n
-    eigenproblem: min(SMs, 160, ceil(n / 8)) on the library's own route
+    """Blocks to reserve for the Householder panel's cooperative launches of an
+    n x n eigenproblem: min(SMs, 160, ceil(n / 8)) on the library's own route
     (from n = 64 under 'auto', from n = 2 under 'tridiag'), 0 where cuSOLVER
-    solves it (no cooperative launch)."""
+    solves it (no cooperative launch). An upper bound: panels of up to 256
+    trailing rows take at most 16 blocks and of up to 544 at most 32."""
     own_from = {None: 64, "auto": 64, "tridiag": 2}.get(solver)
     if own_from is None or n < own_from:
         return 0
@@ -249,7 +250,7 @@ class DeviceExecutor:
         """eig_top for every (G, n, nev) of jobs: the sectors of one split are
         independent, so up to eig_workers of them run at once, each on a
         worker thread with its own context and stream. The Householder panels
-        of this library's eigensolver are cooperative launches of
+        of this library's eigensolver are cooperative launches of at most
         min(SMs, n / 8) blocks from n = 64 on, which must all be resident: the
         solves running together are kept within one block per SM. Largest
         first, as the sectors' costs differ the most."""
