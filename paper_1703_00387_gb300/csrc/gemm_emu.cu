@@ -29,11 +29,12 @@
 // What bounds it: the MMAs, 64 clocks per 128 x 128 x 16. A group walks K once
 // and forms all its pairs from one copy of the slices in shared memory: 24
 // slice tiles per K block and output tile where a pass over K for each pair
-// took 72, which the 60 bytes per clock that an SM takes in from L2 allowed one
-// pair in 570 clocks; now 380, the rest being the single issuing warp and the
-// drains. 2048 x 2048 x 2048: kernel 764 -> 479 us (1290 TFLOP/s of bf16), 2560 x
-// 2048 x 512: 348 -> 208, 2048 x 512 x 2560 with K in shares: 475 -> 168, 381 x 1905
-// x 1000: 201 -> 68. (Shares are added as integers: rounded to float64 first they
+// took 72, 57 bytes per clock into an SM at one pair in 570 clocks; now 380 and a
+// tile's drains (ncu, 5120 x 4096 x 1024: 411 with them on the busiest SM, tensor
+// pipe 64% active, 25 bytes per clock), the rest being the single issuing warp.
+// 2048 x 2048 x 2048: kernel 764 -> 479 us (1290 TFLOP/s of bf16), 2560 x 2048 x
+// 512: 348 -> 208, 2048 x 512 x 2560 with K in shares: 475 -> 168, 381 x 1905 x
+// 1000: 201 -> 68. (Shares are added as integers: rounded to float64 first they
 // cost 177 and 75 us and seven more roundings, 1.3e-16 instead of 8e-17 against
 // 113-bit arithmetic at 128 x 128 x 2048.)
 // The kernel is persistent and warp-specialised: a TMA producer with a ring

@@ -21,11 +21,13 @@
 //   warps 2..17      : epilogue, TMEM partial sums -> float32 registers
 //                      (round-to-nearest adds) -> shared-memory staging ->
 //                      row-contiguous global stores (f32 or f64)
-// What bounds it: the tiles' way from L2 into the SM, about 60 bytes per clock
-// (a K block of 96 KB takes 1600 clocks, its 12 MMAs 1536). With the hi tiles
-// loaded again for the second and third product it was 144 KB: chi = 1024 XXZ
-// product in bf16x3 325 -> 291 us, AKLT 301 x 257 in tf32x3 275 -> 225, left
-// environment update at chi = 1024 264 -> 240.
+// What bounds it: a K block's 12 MMAs take 1536 clocks and its 96 KB of tiles
+// come in from L2 meanwhile; at chi = 1024 a block takes about 2000 with the
+// tensor pipe 67 to 71% active and 41 to 44 bytes per clock arriving (ncu, over a
+// launch on its busiest SM), and whole waves of tiles leave SMs idle. With the hi
+// tiles loaded again for the second and third product it was 144 KB and 52 bytes
+// per clock: chi = 1024 XXZ product in bf16x3 325 -> 291 us, AKLT 301 x 257 in
+// tf32x3 275 -> 225, left environment update at chi = 1024 264 -> 240.
 // Every mbarrier wait is bounded by %globaltimer (2 s); on expiry the kernel
 // records bit 0 in the context's error flag, drains its own copies (bounded),
 // frees TMEM and returns.

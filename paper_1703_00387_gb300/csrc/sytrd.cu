@@ -18,9 +18,11 @@
 //
 // A panel is one cooperative launch, its rows dealt to the blocks round robin;
 // each block keeps its rows of V and W in shared memory. What bounds a column
-// is not its float64 work (A22 v: 13 us at m = 2048, under 2 below m = 700) but
-// the way of its numbers between the blocks and the dependent float64 chains
-// around it, so the column is arranged for few exchanges off the critical
+// below m of about 1000 is not its float64 work (A22 v: under 2 us below m = 700,
+// 13 at 2048, where the float64 pipe issues for two thirds of the column, 16.7 us
+// at m = 1750 with the rows in L2 or in shared memory alike) but the way of its
+// numbers between the blocks and the dependent float64 chains around it, so the
+// column is arranged for few exchanges off the critical
 // path and none through a barrier:
 //   * v = e_(j+1) + inv u with u the column below j + 1 and inv known only
 //     after sigma = u^T u, a square root and two divisions (2000 clocks, formed
