@@ -156,8 +156,12 @@ struct alignas(sizeof(T) * V) Pack {
 // inputs are below 2^63 in float32 or 2^511 in float64 and the MPO entries
 // below 2^50, all that a W-step and the one fused behind it sum is finite (at
 // most 2^11 terms each) and zero entries can be left out. Else (one comparison
-// for all values of a block) they are summed like the others, because 0 x Inf =
-// NaN has to reach every output; finite sums have the same bits either way.
+// for all values that a thread loads) it marks the block's tables W_ALL before
+// the barrier that precedes the sums, and zero entries are summed like the
+// others, because 0 x Inf = NaN has to reach every output. Finite sums have the
+// same bits either way, so sums of earlier fibers may still be running. (A vote
+// at that barrier instead of the mark: left update at chi = 1024 239.7 us, with
+// the mark 238.2.)
 template <typename T, int V>
 __device__ __forceinline__ void note_top(int& top, const Pack<T, V>& x) {
 #pragma unroll
@@ -174,10 +178,10 @@ __device__ __forceinline__ bool wild_entry(double m) { return (__double2hiint(m)
 
 // Fill NT tables. Every thread of the block calls it (whole warps): a warp
 // per output, lanes over the inputs, the nonzero ones compacted by ballots.
-// Ends with a barrier, which also says whether any thread met wild values, in
-// its inputs (top) or in the tables.
+// Ends with a barrier. Threads that met wild values, in their inputs (top) or in
+// the tables, mark them.
 template <int NT, typename T>
-__device__ __forceinline__ bool gather_terms(int top, const double* const (&Mat)[NT], const int (&P)[NT],
+__device__ __forceinline__ void gather_terms(int top, const double* const (&Mat)[NT], const int (&P)[NT],
                                              const int (&Q)[NT], WTable<T>* const (&tab)[NT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   bool all = wild<T>(top);
@@ -206,7 +210,7 @@ __device__ __forceinline__ bool gather_terms(int top, const double* const (&Mat)
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < NT; ++k)
-    if (!tab[k]->dense)
+    if (tab[k]->ptr[Q[k]] <= WT_CAP && P[k] <= 32767)
       for (int o = warp; o < Q[k]; o += warps) {
         int n = tab[k]->ptr[o];
         for (int i0 = 0; i0 < P[k]; i0 += 32) {
@@ -217,7 +221,9 @@ __device__ __forceinline__ bool gather_terms(int top, const double* const (&Mat)
           n += __popc(nz);
         }
       }
-  return __syncthreads_or(all);
+  if (all)
+    for (int k = 0; k < NT; ++k) tab[k]->dense = W_ALL;
+  __syncthreads();
 }
 
 // Output o of a W-step: sum over its nonzero entries of v x_i, inputs in
@@ -365,14 +371,13 @@ __global__ void __launch_bounds__(32 * FIB_WARPS)
       if (staged) xs[i * 32] = x;
       note_top<T, V>(top, x);
     }
-    bool all = false;
-    if (first) all = gather_terms<1, T>(top, {Mat}, {P}, {Q}, {&tab});
-    else all = __syncthreads_or(wild<T>(top));
-    first = false;
-    if (all) {  // from here on
-      if (threadIdx.x == 0) tab.dense = W_ALL;
+    if (first) {
+      gather_terms<1, T>(top, {Mat}, {P}, {Q}, {&tab});
+    } else {
+      if (wild<T>(top)) tab.dense = W_ALL;  // from here on
       __syncthreads();
     }
+    first = false;
     for (int o = warp; o < Q; o += FIB_WARPS) {
       Pack<T, V> acc;
       if (staged) {
@@ -507,14 +512,13 @@ __global__ void __launch_bounds__(32 * FIB_WARPS, sizeof(T) == 8 && PACKED ? 5 :
       xs[k * 32] = x;
       note_top<T, V>(top, x);
     }
-    bool all = false;
-    if (first) all = gather_terms<2, T>(top, {Mat1, Mat2}, {P1, P2}, {Q1, Q2}, {&tab1, &tab2});
-    else all = __syncthreads_or(wild<T>(top));
-    first = false;
-    if (all) {  // from here on
-      if (threadIdx.x == 0) tab1.dense = tab2.dense = W_ALL;
+    if (first) {
+      gather_terms<2, T>(top, {Mat1, Mat2}, {P1, P2}, {Q1, Q2}, {&tab1, &tab2});
+    } else {
+      if (wild<T>(top)) tab1.dense = tab2.dense = W_ALL;  // from here on
       __syncthreads();
     }
+    first = false;
     for (int o = warp; o < Q1; o += FIB_WARPS)
 #pragma unroll
       for (int s2 = 0; s2 < D; ++s2) ms[(o * D + s2) * 32] = sum_terms<T, V>(tab1, o, xs + s2 * 32, D * 32);
